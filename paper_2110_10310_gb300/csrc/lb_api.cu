@@ -49,7 +49,7 @@ struct Region {
 struct Layout {
   Region prob, status, items, sysp, cu, cd, jf, ja, digits, D, Dinv, alpha, carriers, ctab, q0, tar, wgt, qT, ckpt, seg,
       gproj, gsum, sfac, pen, qb, jpen, mpart, pmap, Ginv, hgp, hgm, fgp, fgm, dfA, dfB, Dinvf, zsA, zsB, J, G, grad, gateV, emap, efull, zA, zB, lam, qf, partials, gslots, bar, hist, histf,
-      hkl;
+      hkl, ctabx, fxs, pmat, bst, bsc, jpart;
   size_t total = 0;
 };
 
@@ -118,6 +118,8 @@ struct lb_system {
   bool cluster = false;      // cluster-split sweeps (decided at bind)
   bool tapes_packed = false;  // the bound workspace holds the grid sweeps' tapes packed (k <= l)
   lbk::ClusterConfig cc{};
+  int fx_ws = 0;        // the workspace holds the fixed-point sweeps' tables (1), and the chunked sweep's (2)
+  bool fx_now = false;  // the call under way runs them
   // device binding
   char* ws = nullptr;
   size_t ws_bytes = 0;
@@ -142,7 +144,20 @@ struct lb_batch {
   int64_t n_grad = 0;
   int n_items = 0;
   int max_param_warps = 0;
+  int64_t max_steps = 0;
+  int max_cq = 0;
   lbk::ResidentConfig rc{};
+  // fixed-point sweeps: the items grouped by CTA shape, one launch per group,
+  // the groups after the first on streams of their own (fx_stream)
+  struct FxGroup {
+    int first, n;
+    lbk::FixedConfig fc;
+  };
+  std::vector<FxGroup> fx;
+  std::vector<cudaStream_t> fx_stream;
+  std::vector<cudaEvent_t> fx_event;
+  bool exec_fx[2] = {false, false};  // the captured graph runs them
+  WorkItem* d_items_fx = nullptr;
   char* ws = nullptr;
   size_t ws_bytes = 0;
   ProbDev* d_probs = nullptr;
@@ -239,6 +254,111 @@ int check_predictor(const lb_system* s) {
 // the recompute needs its own predictor history when it predicts
 bool recompute_predicts(const lb_system* s) { return effective_K(s) > 0 && effective_pred(s) > 0; }
 
+// the largest phase |h (E_k - E_l)| an element's free evolution turns by in
+// one step (H_sys, Sec. II)
+double largest_phase(const lb_system* s) {
+  double lo = 0.0, hi = 0.0;
+  for (int k = 0; k < s->N; ++k) {
+    int d[LB_MAXQ], rem = k;
+    for (int q = s->Q - 1; q >= 0; --q) {
+      d[q] = rem % s->levels[q];
+      rem /= s->levels[q];
+    }
+    double E = 0.0;
+    for (int q = 0; q < s->Q; ++q) {
+      E += s->det[q] * d[q] - 0.5 * s->kerr[q] * d[q] * (d[q] - 1.0);
+      for (int p = 0; p < q; ++p) E -= s->xkerr[p * s->Q + q] * d[p] * d[q];
+    }
+    lo = k ? std::min(lo, E) : E;
+    hi = k ? std::max(hi, E) : E;
+  }
+  return s->h * (hi - lo);
+}
+
+// an upper bound of an element's decay rate (1/ns) (collapse operators, Sec. II)
+double largest_decay(const lb_system* s) {
+  double g = 0.0;
+  for (int q = 0; q < s->Q; ++q) {
+    const double n = s->levels[q] - 1.0;
+    g += 0.5 * n * n * s->g2[q] + n * s->g1[q];
+  }
+  return g;
+}
+// no element's free evolution so fast that dt/2 D or (I - dt/2 D)^-1 - 1
+// leaves the coefficients' range of 1/2
+bool fixed_phase_ok(const lb_system* s) { return 0.5 * (largest_phase(s) + s->h * largest_decay(s)) < 0.5; }
+
+// rho_j of every step is at most this (k_stop_factors' bound with each
+// control amplitude at most the sum over its carriers of the largest
+// coefficient: the B-splines are a partition of unity); infinite for
+// controls that overflow it
+double rho_bound(const lb_system* s) {
+  double rho = 0.0;
+  size_t a = 0;
+  for (int q = 0; q < s->Q; ++q) {
+    double d = 0.0;
+    for (int f = 0; f < s->nf[q]; ++f) {
+      double m = 0.0;
+      for (int k = 0; k < s->Ns; ++k, a += 2) m = std::max(m, std::hypot(s->alpha[a], s->alpha[a + 1]));
+      d += m;
+    }
+    const double n = s->levels[q];
+    rho += 0.5 * s->h * kTwoPi * d * 2.0 * (std::sqrt(n - 1.0) + std::sqrt(n - 2.0)) + 0.5 * s->h * s->g1[q] * (n - 1.0);
+  }
+  for (size_t k = 0; k < s->jp.size(); ++k)
+    rho += 4.0 * 0.5 * s->h * std::fabs(s->jg[k]) *
+           std::sqrt((s->levels[s->jp[k]] - 1.0) * (s->levels[s->jq[k]] - 1.0));
+  return std::isfinite(rho) ? rho : INFINITY;
+}
+
+// Fixed-point sweep configuration for N^2 or (herm) N (N + 1) / 2 elements;
+// E == 0 when it cannot apply (a Jaynes-Cummings pair is a unit of the
+// register plan, so pairs need that plan)
+lbk::FixedConfig fixed_cfg(const lb_system* s, bool herm) {
+  if (use_grid(s) || s->V > lbk::kMaxResidentV) return lbk::FixedConfig{};
+  const int units = s->Q + (int)s->jp.size(), nel = herm ? s->N * (s->N + 1) / 2 : s->V;
+  const lbk::FixedConfig fc = lbk::fixed_config(nel, s->V, s->Q, units, n_coef(s), n_jcoef(s), s->N, units);
+  return !s->jp.empty() && fc.QT == 0 ? lbk::FixedConfig{} : fc;
+}
+
+// Their forward predictor: a system of the cluster sweep keeps that sweep's
+// rule, the full stage tape only, so that its results for K >= 1 do not
+// depend on the predictor's restart period.
+int fixed_forward_pred(const lb_system* s) { return !(s->cluster && effective_K(s) > 0); }
+
+// whether the workspace should hold the fixed-point sweeps' tables
+bool fixed_possible(const lb_system* s) {
+  if (s->method != LB_SOLVER_JACOBI || !fixed_phase_ok(s)) return false;
+  return fixed_cfg(s, true).E > 0;
+}
+
+// Chunked sweeps (lb_fixed_chunks.cu) of the small states the cluster sweep
+// took one cluster each: with the full stage tape, at least kChunkMinSteps
+// steps, and N^2 <= 144, where N (N + 1) / 2 columns per chunk cost less than the idle
+// SMs.  A chunk starts its predictor cold, so a step takes more iterations
+// there: max_iter must leave room for a cold start at rho = 1/4.
+constexpr int kChunkMaxV = 144, kChunkMinSteps = 64, kChunkMinIter = 64;
+bool chunks_possible(const lb_system* s) {
+  return !use_grid(s) && s->V <= kChunkMaxV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&
+         s->sweep != LB_SWEEP_RESIDENT && fixed_cfg(s, false).QT > 0;
+}
+// steps per chunk: the chunks of steps run at the same time, the C boundary
+// products one after another, so about the square root of the step count
+int chunk_steps(const lb_system* s) {
+  return std::max(8, (int)std::lround(0.8 * std::sqrt((double)s->NT)));
+}
+
+// Whether this call runs the fixed-point sweeps: the Jacobi iteration with
+// rho_j <= 1/4, where its sums stay inside 64 bits.
+bool use_fixed(const lb_system* s, bool herm) {
+  if (!s->fx_ws || s->method != LB_SOLVER_JACOBI) return false;
+  return fixed_cfg(s, herm).E > 0 && rho_bound(s) <= lbk::kFixedRho;
+}
+bool use_fixed(const lb_system* s) { return use_fixed(s, s->hp.herm != 0); }
+
+// ... and those in chunks: without the Hermitian element plan
+bool use_chunks(const lb_system* s) { return s->hp.chunkL > 0 && s->cluster && !s->hp.herm; }
+
 // Cluster sweep configuration of this system with 2 or 4 lanes per half
 // pair (cs = false / true; a subsystem's control terms, or a Jaynes-Cummings
 // pair, make one half pair); C == 0 when it cannot apply.
@@ -293,7 +413,9 @@ int gproj_used(const lb_system* s) {
 bool use_symmetry(const lb_system* s);
 bool packed_tapes(const lb_system* s);
 
-Layout make_layout(const lb_system* s) {
+// fixed: 0 without, 1 with the fixed-point sweeps' tables, 2 and those of the
+// chunked sweep where it can apply
+Layout make_layout(const lb_system* s, int fixed) {
   Layout L;
   size_t off = 0;
   auto take = [&](Region& r, size_t bytes) {
@@ -363,6 +485,14 @@ Layout make_layout(const lb_system* s) {
   take(L.zsB, grid && s->precision == LB_PREC_F32X2 ? sizeof(float4) * M * V : 0);
   take(L.hkl, sizeof(uint32_t) * (size_t)s->N * (s->N + 1) / 2);
   take(L.pmap, sizeof(int32_t) * (size_t)s->Mu);
+  take(L.ctabx, fixed ? sizeof(int4) * NT * (s->Q + s->jp.size() + 1) : 0);
+  take(L.fxs, fixed ? sizeof(int32_t) * 2 * M * NT : 0);
+  const bool chunks = fixed == 2 && chunks_possible(s);
+  const size_t C = chunks ? (NT + chunk_steps(s) - 1) / chunk_steps(s) : 0;
+  take(L.pmat, sizeof(int4) * C * ((size_t)s->N * (s->N + 1) / 2) * V);
+  take(L.bst, chunks ? sizeof(longlong2) * 3 * (C + 1) * M * V : 0);
+  take(L.bsc, chunks ? sizeof(int32_t) * 3 * (C + 1) * M : 0);
+  take(L.jpart, sizeof(double2) * C * M);
   L.total = off;
   return L;
 }
@@ -604,6 +734,10 @@ int upload_controls(lb_system* s, cudaStream_t st) {
   return LB_OK;
 }
 
+// Above this phase per step (rad) the fixed-point sweeps' predictor turns its
+// frame with the elements' free evolution.
+constexpr double kFramePhase = 0.1;
+
 void fill_prob(lb_system* s) {
   ProbDev& P = s->hp;
   std::memset(&P, 0, sizeof(P));
@@ -715,13 +849,31 @@ void fill_prob(lb_system* s) {
   // the paired-single apply covers the control and decay terms; with
   // Jaynes-Cummings pairs the iterations stay FP64
   P.ff = grid && s->precision == LB_PREC_F32X2 && s->jp.empty() ? 1 : 0;
+  for (int u = 0; u < P.cq; ++u) {
+    // 2^kc >= 4 times the unit's largest ladder factor
+    const double c = u < s->Q ? std::sqrt(s->levels[u] - 1.0)
+                              : std::sqrt((s->levels[s->jp[u - s->Q]] - 1.0) * (s->levels[s->jq[u - s->Q]] - 1.0));
+    P.kc[u] = (int)std::ceil(std::log2(4.0 * c) - 1e-9);
+  }
+  P.fxframe = largest_phase(s) > kFramePhase ? 1 : 0;
+  P.fxfwd = fixed_forward_pred(s);
+  P.ctabx = s->fx_ws ? at<int4>(s, s->L.ctabx) : nullptr;
+  P.fxs = s->fx_ws ? at<int32_t>(s, s->L.fxs) : nullptr;
+  if (s->fx_ws == 2 && chunks_possible(s)) {
+    P.chunkL = chunk_steps(s);
+    P.chunkC = (int32_t)((s->NT + P.chunkL - 1) / P.chunkL);
+    P.pmat = at<int4>(s, s->L.pmat);
+    P.bst = at<longlong2>(s, s->L.bst);
+    P.bsc = at<int32_t>(s, s->L.bsc);
+    P.jpart = at<double2>(s, s->L.jpart);
+  }
   P.zsA = P.ff ? at<float4>(s, s->L.zsA) : nullptr;
   P.zsB = P.ff ? at<float4>(s, s->L.zsB) : nullptr;
 }
 
 int ensure_ctab(lb_system* s, cudaStream_t st) {
   if (!s->ctab_dirty) return LB_OK;
-  LB_CUDA(lbk::launch_control_table(s->dp, s->hp, st), "control table kernels");
+  LB_CUDA(lbk::launch_control_table(s->dp, 1, s->NT, s->hp.cq, st), "control table kernels");
   s->launches += 2;  // control table, stopping factors
   s->ctab_dirty = false;
   return LB_OK;
@@ -740,9 +892,10 @@ int read_status(const DevStatus& d, lb_stats* st, int launches) {
     st->max_iterations = d.max_iter_seen;
     st->kernel_launches = launches;
   }
-  if (d.code == LB_ENOTCONV) {
+  if (d.code == LB_ENOTCONV || (d.code == 0 && d.late)) {
     char buf[160];
-    std::snprintf(buf, sizeof buf, "inner solve did not converge within max_iter at time step %d", d.step);
+    std::snprintf(buf, sizeof buf, "inner solve did not converge within max_iter at time step %d",
+                  d.code ? d.step : 0x7fffffff - d.late);
     return fail(LB_ENOTCONV, buf);
   }
   if (d.code == LB_ENAN) {
@@ -888,6 +1041,7 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
     s->cluster = c.sweep == LB_SWEEP_CLUSTER;
     if (s->cluster) s->cc = cluster_cfg(s, c.E != 0);
     s->hp.gM = gproj_used(s);
+    s->hp.fxfwd = fixed_forward_pred(s);
     s->hp.herm = use_symmetry(s) ? 1 : 0;
     if (c.sweep == LB_SWEEP_RESIDENT) {
       s->rc = lbk::resident_config(s->V, s->Q, n_coef(s), n_jcoef(s), s->N, s->jp.empty(), kry_elems(s));
@@ -928,6 +1082,7 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
     s->cc = cc0;
     s->method = s->hp.method = m0;
     s->hp.gM = gproj_used(s);
+    s->hp.fxfwd = fixed_forward_pred(s);
     s->hp.herm = use_symmetry(s) ? 1 : 0;
     LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
     return fail(LB_ENOTCONV, "no candidate's inner solve converged on the probe steps");
@@ -936,6 +1091,7 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
   s->cluster = win.sweep == LB_SWEEP_CLUSTER;
   s->cc = s->cluster ? cluster_cfg(s, win.E != 0) : cc0;
   s->hp.gM = gproj_used(s);
+  s->hp.fxfwd = fixed_forward_pred(s);
   s->hp.herm = use_symmetry(s) ? 1 : 0;
   if (win.sweep == LB_SWEEP_RESIDENT) {
     s->rc = lbk::resident_config(s->V, s->Q, n_coef(s), n_jcoef(s), s->N, s->jp.empty(), kry_elems(s));
@@ -1301,7 +1457,7 @@ int lb_workspace_bytes(const lb_system* s, size_t* bytes) {
   int rc = check_ready(s, false);
   if (rc) return rc;
   if (!bytes) return fail(LB_EINVAL, "null argument");
-  *bytes = make_layout(s).total;
+  *bytes = make_layout(s, fixed_possible(s) ? 2 : 0).total;
   return LB_OK;
 }
 
@@ -1317,7 +1473,10 @@ int lb_bind_workspace(lb_system* s, void* ws, size_t bytes, void* stream) {
   }
   rc = check_predictor(s);
   if (rc) return rc;
-  s->L = make_layout(s);
+  // a workspace sized without the fixed-point tables still binds (FP64 sweeps)
+  s->fx_ws = fixed_possible(s) ? 2 : 0;
+  while (s->fx_ws && bytes < make_layout(s, s->fx_ws).total) --s->fx_ws;
+  s->L = make_layout(s, s->fx_ws);
   if (bytes < s->L.total) return fail(LB_ENOMEM, "workspace smaller than lb_workspace_bytes");
   s->tapes_packed = packed_tapes(s);
   if (s->rho0.empty()) return fail(LB_EINVAL, "initial states are required before binding");
@@ -1408,6 +1567,7 @@ static int run_forward(lb_system* s, cudaStream_t st, int tape) {
   int rc = order_after_uploads(s, st);
   if (rc) return rc;
   s->launches = 0;
+  s->fx_now = false;
   rc = ensure_ctab(s, st);
   if (rc) return rc;
   LB_CUDA(cudaMemsetAsync(at<DevStatus>(s, s->L.status), 0, sizeof(DevStatus), st), "clear status");
@@ -1428,7 +1588,13 @@ static int run_forward(lb_system* s, cudaStream_t st, int tape) {
     return LB_OK;
   }
   if (s->timing) LB_CUDA(cudaEventRecord(s->ev[0], st), "cudaEventRecord");
-  if (s->cluster)
+  s->fx_now = use_fixed(s);
+  if (s->fx_now && use_chunks(s))
+    LB_CUDA(lbk::launch_forward_chunks(s->dp, s->hp, tape, fixed_cfg(s, false), st), "forward kernels");
+  else if (s->fx_now)
+    LB_CUDA(lbk::launch_forward_fixed(s->dp, s->d_items, s->M, tape, fixed_cfg(s, s->hp.herm != 0), st),
+            "forward kernel");
+  else if (s->cluster)
     LB_CUDA(lbk::launch_forward_cluster(s->dp, s->M, tape, s->cc, st), "forward cluster kernel");
   else
     LB_CUDA(lbk::launch_forward_resident(s->dp, s->d_items, s->M, tape, s->rc, st), "forward kernel");
@@ -1436,7 +1602,7 @@ static int run_forward(lb_system* s, cudaStream_t st, int tape) {
     LB_CUDA(cudaEventRecord(s->ev[1], st), "cudaEventRecord");
     s->timed_fwd = true;
   }
-  s->launches += 1;
+  s->launches += s->fx_now && use_chunks(s) ? 3 + (s->gamma1 != 0.0) : 1;
   return LB_OK;
 }
 
@@ -1474,7 +1640,7 @@ int lb_forward(lb_system* s, void* stream, double* G_out, void* rhoT_dev_out) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = run_forward(s, st, 0);
   if (rc) return rc;
-  LB_CUDA(lbk::launch_finalize(s->dp, 1, 0, 0, st), "objective kernel");
+  LB_CUDA(lbk::launch_finalize(s->dp, 1, 0, 0, 0, st), "objective kernel");
   s->launches += 1;
   if (rhoT_dev_out) {
     if (s->M == s->Mu) {
@@ -1509,6 +1675,10 @@ static int gradient_device(lb_system* s, cudaStream_t st) {
   if (s->timing) LB_CUDA(cudaEventRecord(s->ev[2], st), "cudaEventRecord");
   if (use_grid(s))
     LB_CUDA(lbk::launch_backward_grid(s->dp, s->gblocks_b, s->gsmem, s->hp.ff, st), "backward grid sweep");
+  else if (s->fx_now && use_chunks(s))
+    LB_CUDA(lbk::launch_backward_chunks(s->dp, s->hp, fixed_cfg(s, false), st), "backward kernels");
+  else if (s->fx_now)
+    LB_CUDA(lbk::launch_backward_fixed(s->dp, s->d_items, s->M, fixed_cfg(s, s->hp.herm != 0), st), "backward kernel");
   else if (s->cluster)
     LB_CUDA(lbk::launch_backward_cluster(s->dp, s->M, s->cc, st), "backward cluster kernel");
   else
@@ -1517,8 +1687,9 @@ static int gradient_device(lb_system* s, cudaStream_t st) {
     LB_CUDA(cudaEventRecord(s->ev[3], st), "cudaEventRecord");
     s->timed_bwd = true;
   }
-  LB_CUDA(lbk::launch_finalize(s->dp, 1, param_warps(s), 1, st), "finalize kernels");
-  s->launches += 4;  // backward sweep, objective, slot sum, projection
+  LB_CUDA(lbk::launch_finalize(s->dp, 1, param_warps(s), 1, s->fx_now && !use_grid(s) ? 1 : 0, st), "finalize kernels");
+  // backward sweep, objective, slot sum, projection
+  s->launches += 4 + (s->fx_now && use_chunks(s) ? 1 + (s->gamma1 != 0.0) : 0);
   return LB_OK;
 }
 
@@ -1681,6 +1852,9 @@ static int propagate_impl(lb_system* s, cudaStream_t st, int adjoint, int64_t j0
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
       LB_CUDA(lbk::launch_sweep_grid(s->dp, adjoint ? 2 : 1, 0, 0, j0, j1, x, n_vec, s->gblocks, s->gsmem, s->hp.ff, st),
               "propagate grid sweep");
+    } else if (use_fixed(s, false)) {
+      LB_CUDA(lbk::launch_propagate_fixed(s->dp, adjoint, j0, j1, x, n_vec, fixed_cfg(s, false), st),
+              "propagate kernel");
     } else if (s->cluster) {
       LB_CUDA(lbk::launch_propagate_cluster(s->dp, adjoint, j0, j1, x, n_vec, s->cc, st), "propagate cluster kernel");
     } else {
@@ -1754,6 +1928,8 @@ int lb_batch_create(lb_system* const* systems, int32_t n, lb_batch** out) {
     maxN = std::max(maxN, s->N);
     maxkry = std::max(maxkry, kry_elems(s));
     pairs = pairs || !s->jp.empty();
+    b->max_steps = std::max(b->max_steps, s->NT);
+    b->max_cq = std::max(b->max_cq, s->Q + (int)s->jp.size());
     b->max_param_warps = std::max(b->max_param_warps, param_warps(s));
   }
   b->rc = lbk::resident_config(maxV, maxQ, maxc, maxj, maxN, minQ == maxQ && !pairs, maxkry);
@@ -1777,6 +1953,8 @@ void lb_batch_destroy(lb_batch* b) {
     if (b->exec[m]) cudaGraphExecDestroy(b->exec[m]);
     if (b->graph[m]) cudaGraphDestroy(b->graph[m]);
   }
+  for (cudaEvent_t e : b->fx_event) cudaEventDestroy(e);
+  for (cudaStream_t t : b->fx_stream) cudaStreamDestroy(t);
   delete b;
 }
 
@@ -1787,7 +1965,7 @@ static size_t batch_layout(const lb_batch* b, size_t* o_probs, size_t* o_items, 
   *o_probs = off;
   off += align_up(sizeof(ProbDev) * n);
   *o_items = off;
-  off += align_up(sizeof(WorkItem) * b->n_items);
+  off += 2 * align_up(sizeof(WorkItem) * b->n_items);  // in the FP64 launch's order, then in the fixed-point groups'
   *o_goff = off;
   off += align_up(sizeof(int64_t) * n);
   *o_G = off;
@@ -1806,6 +1984,71 @@ int lb_batch_workspace_bytes(const lb_batch* b, size_t* bytes) {
   return LB_OK;
 }
 
+// The items (most expensive first) grouped for the fixed-point sweeps by CTA
+// shape -- elements per thread, and for E = 1 one warp, up to four, up to 16
+// -- largest groups' CTAs first; empty, with no groups, when some system's
+// workspace or solver rules them out.  Groups keep the many small states from
+// taking a CTA of the largest state's size each.
+static std::vector<WorkItem> fx_groups(lb_batch* b, const std::vector<WorkItem>& items) {
+  b->fx.clear();
+  std::vector<std::pair<int, WorkItem>> keyed;
+  for (const WorkItem& w : items) {
+    const lb_system* s = b->sys[w.prob];
+    const lbk::FixedConfig fc = fixed_cfg(s, s->hp.herm != 0);
+    if (!s->fx_ws || s->method != LB_SOLVER_JACOBI || fc.E <= 0) return {};
+    const int key = fc.QT == 0 ? 3 + fc.E : (fc.threads <= 32 ? 1 : (fc.threads <= 128 ? 2 : 3));
+    keyed.push_back({-key, w});
+  }
+  std::stable_sort(keyed.begin(), keyed.end(),
+                   [](const std::pair<int, WorkItem>& x, const std::pair<int, WorkItem>& y) { return x.first < y.first; });
+  std::vector<WorkItem> out;
+  for (size_t i = 0; i < keyed.size();) {
+    size_t e = i;
+    int nel = 0, V = 0, Q = 0, units = 0, nc = 0, nj = 0, N = 0;
+    for (; e < keyed.size() && keyed[e].first == keyed[i].first; ++e) {
+      const lb_system* s = b->sys[keyed[e].second.prob];
+      nel = std::max(nel, s->hp.herm ? s->N * (s->N + 1) / 2 : s->V);
+      V = std::max(V, s->V);
+      Q = std::max(Q, s->Q);
+      units = std::max(units, s->Q + (int)s->jp.size());
+      nc = std::max(nc, n_coef(s));
+      nj = std::max(nj, n_jcoef(s));
+      N = std::max(N, s->N);
+      out.push_back(keyed[e].second);
+    }
+    b->fx.push_back({(int)i, (int)(e - i), lbk::fixed_config(nel, V, Q, units, nc, nj, N, units)});
+    i = e;
+  }
+  return out;
+}
+
+// the fixed-point sweeps for this call: every system's controls in range
+static bool batch_fixed(const lb_batch* b) {
+  if (b->fx.empty()) return false;
+  for (const lb_system* s : b->sys)
+    if (!use_fixed(s)) return false;
+  return true;
+}
+
+// one launch per group, the groups after the first on their own streams
+// between two events of `st` (also under capture)
+static int batch_fixed_sweep(lb_batch* b, cudaStream_t st, bool backward, int tape) {
+  const size_t n = b->fx.size();
+  if (n > 1) LB_CUDA(cudaEventRecord(b->fx_event[0], st), "cudaEventRecord");
+  for (size_t g = 0; g < n; ++g) {
+    const lb_batch::FxGroup& G = b->fx[g];
+    cudaStream_t t = g ? b->fx_stream[g - 1] : st;
+    if (g) LB_CUDA(cudaStreamWaitEvent(t, b->fx_event[0], 0), "cudaStreamWaitEvent");
+    if (backward)
+      LB_CUDA(lbk::launch_backward_fixed(b->d_probs, b->d_items_fx + G.first, G.n, G.fc, t), "backward kernel");
+    else
+      LB_CUDA(lbk::launch_forward_fixed(b->d_probs, b->d_items_fx + G.first, G.n, tape, G.fc, t), "forward kernel");
+    if (g) LB_CUDA(cudaEventRecord(b->fx_event[g], t), "cudaEventRecord");
+  }
+  for (size_t g = 1; g < n; ++g) LB_CUDA(cudaStreamWaitEvent(st, b->fx_event[g], 0), "cudaStreamWaitEvent");
+  return LB_OK;
+}
+
 int lb_batch_bind_workspace(lb_batch* b, void* ws, size_t bytes, void* stream) {
   if (!b || !ws) return fail(LB_EINVAL, "null argument");
   if (reinterpret_cast<uintptr_t>(ws) % kAlign) return fail(LB_EINVAL, "workspace must be 256-byte aligned");
@@ -1818,6 +2061,7 @@ int lb_batch_bind_workspace(lb_batch* b, void* ws, size_t bytes, void* stream) {
   b->ws_bytes = bytes;
   b->d_probs = reinterpret_cast<ProbDev*>(base + o_probs);
   b->d_items = reinterpret_cast<WorkItem*>(base + o_items);
+  b->d_items_fx = reinterpret_cast<WorkItem*>(base + o_items + align_up(sizeof(WorkItem) * b->n_items));
   b->d_grad_off = reinterpret_cast<int64_t*>(base + o_goff);
   b->d_G = reinterpret_cast<double*>(base + o_G);
   b->d_grad = reinterpret_cast<double*>(base + o_grad);
@@ -1844,6 +2088,21 @@ int lb_batch_bind_workspace(lb_batch* b, void* ws, size_t bytes, void* stream) {
           "upload batch problems");
   LB_CUDA(cudaMemcpyAsync(b->d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, st),
           "upload batch items");
+  const std::vector<WorkItem> items_fx = fx_groups(b, items);
+  if (!items_fx.empty())
+    LB_CUDA(cudaMemcpyAsync(b->d_items_fx, items_fx.data(), sizeof(WorkItem) * items_fx.size(), cudaMemcpyHostToDevice,
+                            st),
+            "upload batch items");
+  while (b->fx_event.size() < b->fx.size()) {
+    cudaEvent_t e = nullptr;
+    LB_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "cudaEventCreate");
+    b->fx_event.push_back(e);
+  }
+  while (b->fx_stream.size() + 1 < b->fx.size()) {
+    cudaStream_t t = nullptr;
+    LB_CUDA(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking), "cudaStreamCreate");
+    b->fx_stream.push_back(t);
+  }
   LB_CUDA(cudaMemcpyAsync(b->d_grad_off, b->grad_off.data(), sizeof(int64_t) * b->grad_off.size(),
                           cudaMemcpyHostToDevice, st),
           "upload gradient offsets");
@@ -1852,38 +2111,53 @@ int lb_batch_bind_workspace(lb_batch* b, void* ws, size_t bytes, void* stream) {
 }
 
 // device work of one batch call (graph-capturable: no host synchronisation)
-static int batch_enqueue(lb_batch* b, cudaStream_t st, int with_grad) {
+static int batch_enqueue(lb_batch* b, cudaStream_t st, int with_grad, bool fixed) {
   NvtxRange nvtx(with_grad ? "lb batch gradient" : "lb batch forward");
-  for (lb_system* s : b->sys) {
-    LB_CUDA(lbk::launch_control_table(s->dp, s->hp, st), "control table kernel");
-    s->ctab_dirty = false;
-    LB_CUDA(cudaMemsetAsync(s->hp.status, 0, sizeof(DevStatus), st), "clear status");
+  const int n = (int)b->sys.size();
+  LB_CUDA(lbk::launch_control_table(b->d_probs, n, b->max_steps, b->max_cq, st), "control table kernel");
+  for (lb_system* s : b->sys) s->ctab_dirty = false;
+  LB_CUDA(lbk::launch_clear_status(b->d_probs, n, st), "clear status");
+  if (fixed) {
+    int rc = batch_fixed_sweep(b, st, false, with_grad);
+    if (rc == LB_OK && with_grad) rc = batch_fixed_sweep(b, st, true, 1);
+    if (rc) return rc;
+  } else {
+    LB_CUDA(lbk::launch_forward_resident(b->d_probs, b->d_items, b->n_items, with_grad, b->rc, st), "forward kernel");
+    if (with_grad)
+      LB_CUDA(lbk::launch_backward_resident(b->d_probs, b->d_items, b->n_items, b->rc, st), "backward kernel");
   }
-  LB_CUDA(lbk::launch_forward_resident(b->d_probs, b->d_items, b->n_items, with_grad, b->rc, st), "forward kernel");
-  if (with_grad)
-    LB_CUDA(lbk::launch_backward_resident(b->d_probs, b->d_items, b->n_items, b->rc, st), "backward kernel");
-  LB_CUDA(lbk::launch_finalize(b->d_probs, (int)b->sys.size(), b->max_param_warps, with_grad, st), "finalize kernels");
-  LB_CUDA(lbk::launch_gather(b->d_probs, (int)b->sys.size(), b->d_grad_off, b->d_G, with_grad ? b->d_grad : nullptr,
-                             b->d_st, st),
+  LB_CUDA(lbk::launch_finalize(b->d_probs, n, b->max_param_warps, with_grad, 1, st), "finalize kernels");
+  LB_CUDA(lbk::launch_gather(b->d_probs, n, b->d_grad_off, b->d_G, with_grad ? b->d_grad : nullptr, b->d_st, st),
           "gather kernel");
+  return LB_OK;
+}
+
+// `st` waits for the systems' uploads (one event per stream they were issued on)
+static int batch_order(lb_batch* b, cudaStream_t st) {
+  const lb_system* done = nullptr;
+  for (lb_system* s : b->sys) {
+    if (done && s->bind_stream == done->bind_stream) continue;
+    int rc = order_after_uploads(s, st);
+    if (rc) return rc;
+    done = s;
+  }
   return LB_OK;
 }
 
 static int batch_call(lb_batch* b, cudaStream_t st, int with_grad, double* G_out, double* grad_out) {
   if (!b->ws) return fail(LB_EINVAL, "no batch workspace bound");
   const int mode = with_grad ? 1 : 0;
-  for (lb_system* s : b->sys) {
-    int rc = order_after_uploads(s, st);
-    if (rc) return rc;
-  }
-  int launches = 0;
-  if (b->exec[mode]) {
+  const int order = batch_order(b, st);
+  if (order) return order;
+  const bool fixed = batch_fixed(b);
+  // control tables, status, objective, gather; with the gradient two sums more
+  const int launches = 5 + 2 * with_grad + (fixed ? (int)b->fx.size() : 1) * (1 + with_grad);
+  if (b->exec[mode] && (fixed || !b->exec_fx[mode])) {
     LB_CUDA(cudaGraphLaunch(b->exec[mode], st), "cudaGraphLaunch");
-    launches = 2 * (int)b->sys.size() + 3 + 3 * with_grad;
   } else {
-    int rc = batch_enqueue(b, st, with_grad);
+    // no graph, or one of the fixed-point sweeps for controls now out of their range
+    int rc = batch_enqueue(b, st, with_grad, fixed);
     if (rc) return rc;
-    launches = 2 * (int)b->sys.size() + 3 + 3 * with_grad;
   }
   const size_t n = b->sys.size();
   std::vector<DevStatus> stv(n);
@@ -1945,17 +2219,16 @@ int lb_batch_capture_graph(lb_batch* b, void* stream, int32_t mode) {
   if (!b->ws) return fail(LB_EINVAL, "no batch workspace bound");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (!st) return fail(LB_EINVAL, "graph capture needs a non-default stream");
-  for (lb_system* s : b->sys) {
-    int rc = order_after_uploads(s, st);
-    if (rc) return rc;
-  }
+  const int order = batch_order(b, st);
+  if (order) return order;
   LB_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
   if (b->exec[mode]) cudaGraphExecDestroy(b->exec[mode]);
   if (b->graph[mode]) cudaGraphDestroy(b->graph[mode]);
   b->exec[mode] = nullptr;
   b->graph[mode] = nullptr;
   LB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
-  int rc = batch_enqueue(b, st, mode);
+  const bool fixed = batch_fixed(b);
+  int rc = batch_enqueue(b, st, mode, fixed);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(st, &g);
   if (rc) {
@@ -1964,6 +2237,7 @@ int lb_batch_capture_graph(lb_batch* b, void* stream, int32_t mode) {
   }
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
   b->graph[mode] = g;
+  b->exec_fx[mode] = fixed;
   LB_CUDA(cudaGraphInstantiate(&b->exec[mode], g, 0), "cudaGraphInstantiate");
   return LB_OK;
 }
@@ -2023,7 +2297,8 @@ int static_bind(lb_system* s, void* ws, cudaStream_t st) {
   int rc0 = decide_krylov(s);
   if (rc0) return rc0;
   s->cluster = false;  // this entry point always runs one CTA per state
-  s->L = make_layout(s);
+  s->fx_ws = fixed_possible(s) && make_layout(s, 1).total <= (size_t)LB_STATIC_SCRATCH_BYTES ? 1 : 0;
+  s->L = make_layout(s, s->fx_ws);
   s->tapes_packed = packed_tapes(s);
   s->ws = static_cast<char*>(ws);
   s->ws_bytes = LB_STATIC_SCRATCH_BYTES;
@@ -2101,7 +2376,7 @@ extern "C" int lb_gradient_static(lb_system* s, void* stream, double* G_out, dou
   if (rc) return rc;
   if (s->target_mode == 0) return fail(LB_EINVAL, "no objective (lb_objective_set or lb_objective_set_gate)");
   if (s->rho0.empty()) return fail(LB_EINVAL, "no initial states");
-  const size_t need = make_layout(s).total;
+  const size_t need = make_layout(s, 0).total;
   if (need > (size_t)LB_STATIC_SCRATCH_BYTES) {
     char buf[200];
     std::snprintf(buf, sizeof buf, "problem needs %zu bytes of device scratch; the static scratch holds %zu",

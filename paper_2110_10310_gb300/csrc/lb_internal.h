@@ -16,7 +16,7 @@ struct DevStatus {
   int32_t code;                 // 0 or LB_ENOTCONV / LB_ENAN (first error wins)
   int32_t step;                 // time step of the first error
   int32_t max_iter_seen;        // largest iteration count of one step
-  int32_t pad;
+  int32_t late;                 // chunked sweeps: INT32_MAX - the earliest step that did not converge, 0 if none
   unsigned long long iters[3];  // iterations per phase: forward, recompute, adjoint
   unsigned long long steps[3];  // state-steps per phase
   unsigned long long diters[3]; // of iters: difference iterations in single precision (grid sweeps)
@@ -118,6 +118,18 @@ struct ProbDev {
   float2* Dinvf;             // [V] grid sweeps: (I - dt/2 D)^-1 in single precision
   int32_t ff;                // grid sweeps: FP64 iterations apply O in single-precision pairs (lb_set_precision)
   int32_t pad2;
+  // fixed-point sweeps (lb_fixed.cu; null without their workspace)
+  int32_t kc[LB_MAXQ + LB_MAXQ * (LB_MAXQ - 1) / 2];  // 2^kc >= 4 times the largest ladder factor, per subsystem, then pair
+  int32_t fxframe;           // their predictor turns its frame (the phases per step are not small)
+  int32_t fxfwd;             // ... and is used in the forward solves (like the cluster sweep's: not with checkpoints)
+  // chunks of steps advanced at the same time (lb_fixed_chunks.cu; chunkL == 0: not used)
+  int32_t chunkL, chunkC;    // steps per chunk, chunks
+  int4* pmat;                // [C][N(N+1)/2][V] split entries of the chunks' propagators, one column per k <= l
+  longlong2* bst;            // [3][C + 1][M][V] states, adjoint states and penalty responses at the chunk boundaries
+  int32_t* bsc;              // [3][C + 1][M] their scales
+  double2* jpart;            // [M][C] the running penalty's sums per chunk
+  int4* ctabx;               // [NT][cq + 1] the rows of ctab split for them, last the stopping factor and range flag
+  int32_t* fxs;              // [M][2 NT] scales of the stage vectors and the checkpoints
   float4* zsA;               // [M*V] the iterates zA / zB split into single-precision pairs (x_hi, x_lo, y_hi, y_lo)
   float4* zsB;
 };
@@ -154,13 +166,18 @@ int gmres_krylov_dim(int V, int ncoef, int njcoef, int N, size_t smem_limit);
 cudaError_t launch_tables(ProbDev* d_prob, const ProbDev& h_prob, cudaStream_t s);
 cudaError_t launch_gate_targets(const ProbDev& h_prob, const double2* Vg, const int32_t* emap, const int32_t* efull,
                                 int32_t Ne, cudaStream_t s);
-cudaError_t launch_control_table(const ProbDev* d_prob, const ProbDev& h_prob, cudaStream_t s);
+// control factors and stopping factors of n_probs systems of the device array
+// d_probs (at most max_steps steps, max_cq table entries per step)
+cudaError_t launch_control_table(const ProbDev* d_probs, int n_probs, int64_t max_steps, int max_cq, cudaStream_t s);
+cudaError_t launch_clear_status(const ProbDev* d_probs, int n_probs, cudaStream_t s);
 cudaError_t launch_forward_resident(const ProbDev* d_probs, const WorkItem* d_items, int n_items, int tape,
                                     const ResidentConfig& rc, cudaStream_t s);
 cudaError_t launch_backward_resident(const ProbDev* d_probs, const WorkItem* d_items, int n_items,
                                      const ResidentConfig& rc, cudaStream_t s);
 // objective (and gradient projection) for n_probs systems of the device array d_probs
-cudaError_t launch_finalize(const ProbDev* d_probs, int n_probs, int max_param_warps, int with_grad, cudaStream_t s);
+// (one_slot: every state's gradient pieces are in its own slot, gM = M)
+cudaError_t launch_finalize(const ProbDev* d_probs, int n_probs, int max_param_warps, int with_grad, int one_slot,
+                            cudaStream_t s);
 // copy G, gradients and status words of n_probs systems into contiguous arrays
 cudaError_t launch_gather(const ProbDev* d_probs, int n_probs, const int64_t* grad_off, double* G_all,
                           double* grad_all, DevStatus* st_all, cudaStream_t s);
@@ -168,6 +185,34 @@ cudaError_t launch_apply(const ProbDev* d_prob, const ProbDev& h_prob, int adjoi
                          double2* y, int n_vec, cudaStream_t s);
 cudaError_t launch_propagate_resident(const ProbDev* d_prob, int adjoint, int64_t j0, int64_t j1, double2* x,
                                       int n_vec, const ResidentConfig& rc, cudaStream_t s);
+
+// one-CTA-per-state sweeps in fixed point (lb_fixed.cu)
+constexpr double kFixedRho = 0.25;  // largest iteration-matrix bound rho_j they take
+struct FixedConfig {
+  int threads, E, QT;  // CTA size, elements per thread (0: not applicable), units of the register plan (E = 1)
+  size_t smem;
+};
+// nel: elements a CTA computes; units: subsystems plus Jaynes-Cummings pairs
+// (maxima over the launch's problems)
+FixedConfig fixed_config(int nel, int V, int Q, int units, int ncoef, int njcoef, int N, int cq);
+cudaError_t launch_forward_fixed(const ProbDev* d_probs, const WorkItem* d_items, int n_items, int tape,
+                                 const FixedConfig& fc, cudaStream_t s);
+cudaError_t launch_backward_fixed(const ProbDev* d_probs, const WorkItem* d_items, int n_items, const FixedConfig& fc,
+                                  cudaStream_t s);
+cudaError_t launch_propagate_fixed(const ProbDev* d_prob, int adjoint, int64_t j0, int64_t j1, double2* x, int n_vec,
+                                   const FixedConfig& fc, cudaStream_t s);
+
+// the forward (backward) sweep of a system whose steps are advanced in chunks
+cudaError_t launch_forward_chunks(const ProbDev* d_prob, const ProbDev& h_prob, int tape, const FixedConfig& fc,
+                                  cudaStream_t s);
+cudaError_t launch_backward_chunks(const ProbDev* d_prob, const ProbDev& h_prob, const FixedConfig& fc,
+                                   cudaStream_t s);
+// chunked = 1: one CTA per (state, chunk) of the first problem; mode: 0 the
+// sweep, 1 the penalty's response alone (backward)
+cudaError_t launch_forward_fixed_chunked(const ProbDev* d_prob, int n_ctas, int tape, const FixedConfig& fc,
+                                         cudaStream_t s);
+cudaError_t launch_backward_fixed_chunked(const ProbDev* d_prob, int n_ctas, int mode, const FixedConfig& fc,
+                                          cudaStream_t s);
 
 // grid-wide cooperative sweeps for states too large for one CTA
 constexpr int kGridThreads = 256;

@@ -3,6 +3,7 @@
 // and gradient projection, the batch gather, and the Lindblad apply.
 
 #include "lb_device.cuh"
+#include "lb_fixed.cuh"
 
 namespace lbk {
 
@@ -112,9 +113,19 @@ __global__ void k_gate_targets(ProbDev P, const double2* __restrict__ Vg, const 
   P.tar[tid] = acc;
 }
 
+// one factor (dt/2) d = a + i b of the control table, and for the fixed-point
+// sweeps its split form scaled by the unit's 2^kc
+__device__ __forceinline__ void put_factor(const ProbDev& P, int j, int u, double2 c) {
+  P.ctab[(size_t)j * P.cq + u] = c;
+  if (!P.ctabx) return;
+  const Fx a = fx_coef(__double2ll_rn(scalbn(c.x, 62 + P.kc[u])));
+  const Fx b = fx_coef(__double2ll_rn(scalbn(c.y, 62 + P.kc[u])));
+  P.ctabx[(size_t)j * (P.cq + 1) + u] = make_int4(a.h, a.l, b.h, b.l);
+}
+
 // (dt/2) d_q(t_j + dt/2) for every step j and subsystem q (eq. rotctrl)
-__global__ void k_control_table(const ProbDev* __restrict__ pp) {
-  const ProbDev& P = *pp;
+__global__ void k_control_table(const ProbDev* __restrict__ probs) {
+  const ProbDev& P = probs[blockIdx.y];
   const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (tid >= (size_t)P.NT * P.cq) return;
   const int j = (int)(tid / P.cq), q = (int)(tid % P.cq);
@@ -125,7 +136,7 @@ __global__ void k_control_table(const ProbDev* __restrict__ pp) {
     double sn, cs;
     sincos(P.je[k] * t, &sn, &cs);
     const double gg = 0.5 * P.h * P.jg[k];
-    P.ctab[tid] = make_double2(gg * cs, gg * sn);
+    put_factor(P, j, q, make_double2(gg * cs, gg * sn));
     return;
   }
   const double dtau = P.Tc / (P.Ns - 2);
@@ -146,31 +157,37 @@ __global__ void k_control_table(const ProbDev* __restrict__ pp) {
     di += wr * sn + wi * cs;
   }
   const double sc = 0.5 * P.h * kTwoPi;
-  P.ctab[tid] = make_double2(sc * dr, sc * di);
+  put_factor(P, j, q, make_double2(sc * dr, sc * di));
 }
 
 // rho_j >= ||(I - dt/2 D)^-1 dt/2 O_j||_inf and the same for the adjoint:
 // |(I - dt/2 D)^-1| <= 1 (Re D <= 0); per subsystem the control couplings of
 // one row (or column) sum to at most |dt/2 d_q| 2 (sqrt(n-1) + sqrt(n-2)), and
 // the decay sandwich to at most (dt/2)/T1 (n - 1).  One thread per step.
-__global__ void k_stop_factors(const ProbDev* __restrict__ pp) {
-  const ProbDev& P = *pp;
+__global__ void k_stop_factors(const ProbDev* __restrict__ probs) {
+  const ProbDev& P = probs[blockIdx.y];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= P.NT) return;
   double rho = 0.0;
+  bool range = true;  // every factor within the fixed-point sweeps' 1/2
   for (int q = 0; q < P.Q; ++q) {
     const double n = P.levels[q];
     const double2 c = P.ctab[(size_t)j * P.cq + q];
+    if (P.ctabx) range = range && scalbn(fmax(fabs(c.x), fabs(c.y)), P.kc[q]) <= 0.5;
     rho += hypot(c.x, c.y) * 2.0 * (sqrt(n - 1.0) + sqrt(n - 2.0)) + P.jump[q] * (n - 1.0);
   }
   // each of the four terms of a Jaynes-Cummings pair couples with at most
   // |dt/2 g| sqrt((n_p - 1)(n_q - 1))
   for (int k = 0; k < P.npair; ++k) {
     const double2 c = P.ctab[(size_t)j * P.cq + P.Q + k];
+    if (P.ctabx) range = range && scalbn(fmax(fabs(c.x), fabs(c.y)), P.kc[P.Q + k]) <= 0.5;
     rho += 4.0 * hypot(c.x, c.y) * sqrt((P.levels[P.jp[k]] - 1.0) * (P.levels[P.jq[k]] - 1.0));
   }
   // (1 - rho)/rho, capped so that rtol ||q|| times it stays finite
   P.sfac[j] = rho < 0.5 ? fmin((1.0 - rho) / fmax(rho, 1e-200), 1e200) : 1.0;
+  if (P.ctabx)
+    P.ctabx[(size_t)j * (P.cq + 1) + P.cq] =
+        make_int4(__float_as_int((float)(P.rtol * P.sfac[j])), range && rho <= kFixedRho ? 0 : 1, 0, 0);
   // running penalty weight dt beta(t_j), beta(t) = exp(-((t - T)/a)^2)/a, left rectangle rule
   if (P.gamma1 != 0.0) {
     const double x = (j * P.h - P.T) / P.pen_a;
@@ -192,12 +209,13 @@ __global__ void k_objective(const ProbDev* __restrict__ probs) {
 
 // Sum of the gradient pieces over their gM state slots (states, CTAs, warps),
 // in slot order, for every (step, subsystem, piece): gsum[NT][Q][2].
-__global__ void k_gproj_reduce(const ProbDev* __restrict__ probs) {
+__global__ void k_gproj_reduce(const ProbDev* __restrict__ probs, int one_slot) {
   const ProbDev& P = probs[blockIdx.y];
+  const int slots = one_slot ? P.M : P.gM;
   const size_t n = (size_t)P.NT * P.Q * 2, stride = (size_t)gridDim.x * blockDim.x;
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
     double2 t = make_double2(0.0, 0.0);
-    for (int i = 0; i < P.gM; ++i) {
+    for (int i = 0; i < slots; ++i) {
       const double2 g = P.gproj[(size_t)i * n + k];
       t.x += g.x;
       t.y += g.y;
@@ -246,6 +264,12 @@ __global__ void k_gradient_project(const ProbDev* __restrict__ probs) {
     P.grad[k] = sc * gr + P.gamma2 * P.alpha[k];
     P.grad[k + 1] = sc * gi + P.gamma2 * P.alpha[k + 1];
   }
+}
+
+// zero the status block of every system of a batch
+__global__ void k_clear_status(const ProbDev* __restrict__ probs) {
+  static_assert(sizeof(DevStatus) % 4 == 0 && sizeof(DevStatus) / 4 <= 32, "one warp clears a status block");
+  if (threadIdx.x < sizeof(DevStatus) / 4) reinterpret_cast<int*>(probs[blockIdx.x].status)[threadIdx.x] = 0;
 }
 
 // G, gradient and status of every system of a batch into contiguous arrays
@@ -324,20 +348,27 @@ cudaError_t launch_gate_targets(const ProbDev& h, const double2* Vg, const int32
   return cudaGetLastError();
 }
 
-cudaError_t launch_control_table(const ProbDev* d_prob, const ProbDev& h, cudaStream_t s) {
-  const size_t n = (size_t)h.NT * h.cq;
-  k_control_table<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d_prob);
+cudaError_t launch_control_table(const ProbDev* d_probs, int n_probs, int64_t max_steps, int max_cq,
+                                 cudaStream_t s) {
+  const size_t n = (size_t)max_steps * max_cq;
+  k_control_table<<<dim3((unsigned)((n + 255) / 256), n_probs), 256, 0, s>>>(d_probs);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_stop_factors<<<(unsigned)((h.NT + 255) / 256), 256, 0, s>>>(d_prob);
+  k_stop_factors<<<dim3((unsigned)((max_steps + 255) / 256), n_probs), 256, 0, s>>>(d_probs);
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const ProbDev* d_probs, int n_probs, int max_param_warps, int with_grad, cudaStream_t s) {
+cudaError_t launch_clear_status(const ProbDev* d_probs, int n_probs, cudaStream_t s) {
+  k_clear_status<<<n_probs, 32, 0, s>>>(d_probs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finalize(const ProbDev* d_probs, int n_probs, int max_param_warps, int with_grad, int one_slot,
+                            cudaStream_t s) {
   k_objective<<<n_probs, 32, 0, s>>>(d_probs);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !with_grad) return e;
-  k_gproj_reduce<<<dim3(304, n_probs), 256, 0, s>>>(d_probs);
+  k_gproj_reduce<<<dim3(304, n_probs), 256, 0, s>>>(d_probs, one_slot);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int threads = 128;
