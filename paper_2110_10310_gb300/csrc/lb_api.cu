@@ -49,7 +49,7 @@ struct Region {
 struct Layout {
   Region prob, status, items, sysp, cu, cd, jf, ja, digits, D, Dinv, alpha, carriers, ctab, q0, tar, wgt, qT, ckpt, seg,
       gproj, gsum, sfac, pen, qb, jpen, mpart, pmap, Ginv, hgp, hgm, fgp, fgm, dfA, dfB, Dinvf, zsA, zsB, J, G, grad, gateV, emap, efull, zA, zB, lam, qf, partials, gslots, bar, hist, histf,
-      hkl, ctabx, fxs, pmat, bst, bsc, jpart;
+      hkl, ctabx, fxs, pmat, bst, bsc, jpart, fxd, fxh, fxu, gsc;
   size_t total = 0;
 };
 
@@ -321,6 +321,13 @@ lbk::FixedConfig fixed_cfg(const lb_system* s, bool herm) {
   return !s->jp.empty() && fc.QT == 0 ? lbk::FixedConfig{} : fc;
 }
 
+// The grid-wide sweeps in fixed point (lb_gridx.cu): no Jaynes-Cummings pairs
+// or running penalty, a forward predictor (cold solves take many iterations,
+// where the FP64 sweeps' single-precision difference iterations win).
+bool gridx_possible(const lb_system* s) {
+  return s->jp.empty() && s->gamma1 == 0.0 && effective_pred(s) != LB_PRED_NONE && s->Mu <= lbk::kGridFixedStates;
+}
+
 // Their forward predictor: a system of the cluster sweep keeps that sweep's
 // rule, the full stage tape only, so that its results for K >= 1 do not
 // depend on the predictor's restart period.
@@ -329,6 +336,7 @@ int fixed_forward_pred(const lb_system* s) { return !(s->cluster && effective_K(
 // whether the workspace should hold the fixed-point sweeps' tables
 bool fixed_possible(const lb_system* s) {
   if (s->method != LB_SOLVER_JACOBI || !fixed_phase_ok(s)) return false;
+  if (use_grid(s)) return gridx_possible(s);
   return fixed_cfg(s, true).E > 0;
 }
 
@@ -352,6 +360,7 @@ int chunk_steps(const lb_system* s) {
 // rho_j <= 1/4, where its sums stay inside 64 bits.
 bool use_fixed(const lb_system* s, bool herm) {
   if (!s->fx_ws || s->method != LB_SOLVER_JACOBI) return false;
+  if (use_grid(s)) return rho_bound(s) <= lbk::kGridFixedRho;
   return fixed_cfg(s, herm).E > 0 && rho_bound(s) <= lbk::kFixedRho;
 }
 bool use_fixed(const lb_system* s) { return use_fixed(s, s->hp.herm != 0); }
@@ -468,7 +477,7 @@ Layout make_layout(const lb_system* s, int fixed) {
   take(L.lam, grid ? c2 * M * V : 0);
   take(L.qf, grid ? c2 * M * V : 0);
   take(L.partials, grid ? sizeof(double) * lbk::kMaxGridBlocks * LB_MAXQ * 4 : 0);
-  take(L.gslots, grid ? sizeof(unsigned long long) * 5 * M : 0);
+  take(L.gslots, grid ? sizeof(unsigned long long) * 5 * M : 0);  // or 6 M words of 32 bits (fixed point)
   take(L.bar, grid ? sizeof(GridBar) : 0);
   take(L.hist, c2 * lbk::kRingOrder * M * V);
   take(L.histf, recompute_predicts(s) ? c2 * lbk::kRingOrder * M * V : 0);
@@ -487,6 +496,10 @@ Layout make_layout(const lb_system* s, int fixed) {
   take(L.pmap, sizeof(int32_t) * (size_t)s->Mu);
   take(L.ctabx, fixed ? sizeof(int4) * NT * (s->Q + s->jp.size() + 1) : 0);
   take(L.fxs, fixed ? sizeof(int32_t) * 2 * M * NT : 0);
+  take(L.fxd, fixed && grid ? sizeof(int4) * V : 0);
+  take(L.fxh, fixed && grid ? sizeof(int4) * V : 0);
+  take(L.fxu, fixed && grid ? sizeof(longlong2) * V : 0);
+  take(L.gsc, fixed && grid ? sizeof(int32_t) * M : 0);
   const bool chunks = fixed == 2 && chunks_possible(s);
   const size_t C = chunks ? (NT + chunk_steps(s) - 1) / chunk_steps(s) : 0;
   take(L.pmat, sizeof(int4) * C * ((size_t)s->N * (s->N + 1) / 2) * V);
@@ -859,6 +872,12 @@ void fill_prob(lb_system* s) {
   P.fxfwd = fixed_forward_pred(s);
   P.ctabx = s->fx_ws ? at<int4>(s, s->L.ctabx) : nullptr;
   P.fxs = s->fx_ws ? at<int32_t>(s, s->L.fxs) : nullptr;
+  if (grid && s->fx_ws) {
+    P.fxd = at<int4>(s, s->L.fxd);
+    P.fxh = at<int4>(s, s->L.fxh);
+    P.fxu = at<longlong2>(s, s->L.fxu);
+    P.gsc = at<int32_t>(s, s->L.gsc);
+  }
   if (s->fx_ws == 2 && chunks_possible(s)) {
     P.chunkL = chunk_steps(s);
     P.chunkC = (int32_t)((s->NT + P.chunkL - 1) / P.chunkL);
@@ -1119,8 +1138,11 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.gslots), 0, s->L.gslots.bytes, st), "clear grid slots");
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
       LB_CUDA(cudaEventRecord(a, st), "cudaEventRecord");
-      LB_CUDA(lbk::launch_sweep_grid(s->dp, 0, 1, 0, 0, pst, nullptr, s->M, s->gblocks, s->gsmem, s->hp.ff, st),
-              "forward grid sweep");
+      if (use_fixed(s))
+        LB_CUDA(lbk::launch_sweep_gx(s->dp, s->hp, 0, 0, 0, pst, nullptr, s->M, st), "forward grid sweep");
+      else
+        LB_CUDA(lbk::launch_sweep_grid(s->dp, 0, 1, 0, 0, pst, nullptr, s->M, s->gblocks, s->gsmem, s->hp.ff, st),
+                "forward grid sweep");
       LB_CUDA(cudaEventRecord(b, st), "cudaEventRecord");
       DevStatus d{};
       LB_CUDA(cudaMemcpyAsync(&d, at<DevStatus>(s, s->L.status), sizeof(DevStatus), cudaMemcpyDeviceToHost, st),
@@ -1577,8 +1599,12 @@ static int run_forward(lb_system* s, cudaStream_t st, int tape) {
     LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
     if (s->gamma1 != 0.0) LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.jpen), 0, s->L.jpen.bytes, st), "clear penalty");
     if (s->timing) LB_CUDA(cudaEventRecord(s->ev[0], st), "cudaEventRecord");
-    LB_CUDA(lbk::launch_sweep_grid(s->dp, 0, 1, tape, 0, s->NT, nullptr, s->M, s->gblocks, s->gsmem, s->hp.ff, st),
-            "forward grid sweep");
+    s->fx_now = use_fixed(s);
+    if (s->fx_now)
+      LB_CUDA(lbk::launch_sweep_gx(s->dp, s->hp, 0, tape, 0, s->NT, nullptr, s->M, st), "forward grid sweep");
+    else
+      LB_CUDA(lbk::launch_sweep_grid(s->dp, 0, 1, tape, 0, s->NT, nullptr, s->M, s->gblocks, s->gsmem, s->hp.ff, st),
+              "forward grid sweep");
     if (s->timing) {
       LB_CUDA(cudaEventRecord(s->ev[1], st), "cudaEventRecord");
       s->timed_fwd = true;
@@ -1673,7 +1699,9 @@ static int gradient_device(lb_system* s, cudaStream_t st) {
     LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
   }
   if (s->timing) LB_CUDA(cudaEventRecord(s->ev[2], st), "cudaEventRecord");
-  if (use_grid(s))
+  if (use_grid(s) && s->fx_now)
+    LB_CUDA(lbk::launch_backward_gx(s->dp, s->hp, st), "backward grid sweep");
+  else if (use_grid(s))
     LB_CUDA(lbk::launch_backward_grid(s->dp, s->gblocks_b, s->gsmem, s->hp.ff, st), "backward grid sweep");
   else if (s->fx_now && use_chunks(s))
     LB_CUDA(lbk::launch_backward_chunks(s->dp, s->hp, fixed_cfg(s, false), st), "backward kernels");
@@ -1850,8 +1878,12 @@ static int propagate_impl(lb_system* s, cudaStream_t st, int adjoint, int64_t j0
       if (n_vec > s->M) return fail(LB_EINVAL, "grid sweeps propagate at most M vectors at a time");
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.gslots), 0, s->L.gslots.bytes, st), "clear grid slots");
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
-      LB_CUDA(lbk::launch_sweep_grid(s->dp, adjoint ? 2 : 1, 0, 0, j0, j1, x, n_vec, s->gblocks, s->gsmem, s->hp.ff, st),
-              "propagate grid sweep");
+      if (use_fixed(s, false))
+        LB_CUDA(lbk::launch_sweep_gx(s->dp, s->hp, adjoint ? 2 : 1, 0, j0, j1, x, n_vec, st), "propagate grid sweep");
+      else
+        LB_CUDA(lbk::launch_sweep_grid(s->dp, adjoint ? 2 : 1, 0, 0, j0, j1, x, n_vec, s->gblocks, s->gsmem, s->hp.ff,
+                                       st),
+                "propagate grid sweep");
     } else if (use_fixed(s, false)) {
       LB_CUDA(lbk::launch_propagate_fixed(s->dp, adjoint, j0, j1, x, n_vec, fixed_cfg(s, false), st),
               "propagate kernel");

@@ -141,6 +141,12 @@ __device__ __forceinline__ Cx fx_frame(double2 D, double hh) {
   return u;
 }
 
+// dt/2 D, 62 fraction bits (magnitude below 1/2 where it is used)
+__device__ __forceinline__ int4 fx_halfd(double2 D, double hh) {
+  const Fx x = fx_coef(__double2ll_rn(scalbn(hh * D.x, 62))), y = fx_coef(__double2ll_rn(scalbn(hh * D.y, 62)));
+  return make_int4(x.h, x.l, y.h, y.l);
+}
+
 // headroom of a state's scale: the largest entry is set to [2^59, 2^60) at the
 // start and the scale moved by 2 when it has left [2^58.5, 2^60)
 constexpr int kFxTop = 59;

@@ -128,6 +128,10 @@ struct ProbDev {
   longlong2* bst;            // [3][C + 1][M][V] states, adjoint states and penalty responses at the chunk boundaries
   int32_t* bsc;              // [3][C + 1][M] their scales
   double2* jpart;            // [M][C] the running penalty's sums per chunk
+  int4* fxd;                 // [V] grid sweeps: (I - dt/2 D)^-1 - 1, split
+  int4* fxh;                 // [V] dt/2 D, split
+  longlong2* fxu;            // [V] the frame's factor per step, half of the unit-modulus part of g
+  int32_t* gsc;              // [M] the adjoint states' scales during a recompute
   int4* ctabx;               // [NT][cq + 1] the rows of ctab split for them, last the stopping factor and range flag
   int32_t* fxs;              // [M][2 NT] scales of the stage vectors and the checkpoints
   float4* zsA;               // [M*V] the iterates zA / zB split into single-precision pairs (x_hi, x_lo, y_hi, y_lo)
@@ -227,6 +231,12 @@ size_t grid_smem_bytes(int ncoef, int njcoef);
 cudaError_t launch_sweep_grid(const ProbDev* d_prob, int mode, int init_from_q0, int tape, int64_t j0, int64_t j1,
                               double2* x, int nstates, int nblocks, size_t smem, int ff, cudaStream_t s);
 cudaError_t launch_backward_grid(const ProbDev* d_prob, int nblocks, size_t smem, int ff, cudaStream_t s);
+// the same sweeps in fixed point (lb_gridx.cu)
+constexpr double kGridFixedRho = 0.0625;  // largest iteration-matrix bound they take
+constexpr int kGridFixedStates = 4096;    // most states (their scales are in shared memory)
+cudaError_t launch_sweep_gx(const ProbDev* d_prob, const ProbDev& h_prob, int mode, int tape, int64_t j0, int64_t j1,
+                            double2* x, int nstates, cudaStream_t s);
+cudaError_t launch_backward_gx(const ProbDev* d_prob, const ProbDev& h_prob, cudaStream_t s);
 
 // cluster-split sweeps for small states: one cluster of C CTAs per state,
 // 2Q lanes per element, or 4Q with the component split (Q <= 4,

@@ -78,6 +78,12 @@ __global__ void k_tables(ProbDev* __restrict__ pp) {
     const double den = ar * ar + ai * ai;
     P.Dinv[tid] = make_double2(ar / den, -ai / den);
     if (P.Dinvf) P.Dinvf[tid] = make_float2((float)(ar / den), (float)(-ai / den));
+    if (P.fxd) {
+      P.fxd[tid] = fx_dinv1(D, hh);
+      P.fxh[tid] = fx_halfd(D, hh);
+      const Cx u = fx_frame(D, hh);
+      P.fxu[tid] = make_longlong2(u.x, u.y);
+    }
     if (P.Ginv) {
       // 1/g = (1 - dt/2 D)/(1 + dt/2 D), g the element's free step factor
       const double br = 1.0 + hh * D.x, bi = hh * D.y;

@@ -208,3 +208,28 @@ def test_batch_in_and_out_of_the_fixed_point_range(L):
     ss[1].set_alpha(ps[1].controls.alpha)
     G3, g3 = b.gradient(stream=st)
     assert np.array_equal(G3, G0) and np.array_equal(g3, g0)
+
+
+# the grid sweep in fixed point: elements packed or not, several states per
+# block and one state over many, checkpoints, subsystem counts with an unrolled
+# loop (3, 4) and without
+@gpu
+@pytest.mark.parametrize("levels,n_states,herm,K,objective", [
+    ((3, 3), 3, True, 0, "frob"), ((2, 3), 9, False, 5, "trace"), ((3, 2, 4), 2, True, 7, "frob"),
+    ((2, 2, 2, 2), 5, False, 0, "frob"), ((2, 3, 2, 2), 2, True, 4, "trace"), ((5,), 40, True, 0, "frob")])
+def test_grid_sweep_matches_the_oracle(L, levels, n_states, herm, K, objective):
+    p = _problem(levels, 23, herm, K, n_states=n_states, objective=objective)
+    s, G, g = _against_oracle(p, sweep=L.LB_SWEEP_GRID)
+    st = s.stats()
+    assert st["sweep"] == "grid" and st["phase_diff_iterations"] == [0, 0, 0]
+    r = _sys(p, sweep=L.LB_SWEEP_RESIDENT)
+    Gr, gr = r.gradient()
+    assert abs(G - Gr) <= 1e-12 * abs(Gr) and _rel(g, gr) < 1e-11
+    # steps on given vectors, both directions, against the one-CTA sweep
+    rng = np.random.default_rng(4)
+    N = int(np.prod(levels))
+    x = torch.from_numpy(rng.standard_normal((2, N, N)) + 1j * rng.standard_normal((2, N, N))).cuda()
+    for adj in (False, True):
+        a = s.propagate(x, 3, 17, adjoint=adj).cpu().numpy()
+        b = r.propagate(x, 3, 17, adjoint=adj).cpu().numpy()
+        assert _rel(a, b) < 1e-13
