@@ -285,8 +285,8 @@ double largest_decay(const lb_system* s) {
   return g;
 }
 // no element's free evolution so fast that dt/2 D or (I - dt/2 D)^-1 - 1
-// leaves the coefficients' range of 1/2
-bool fixed_phase_ok(const lb_system* s) { return 0.5 * (largest_phase(s) + s->h * largest_decay(s)) < 0.5; }
+// leaves the coefficients' range (0.48)
+bool fixed_phase_ok(const lb_system* s) { return 0.5 * (largest_phase(s) + s->h * largest_decay(s)) < 0.45; }
 
 // rho_j of every step is at most this (k_stop_factors' bound with each
 // control amplitude at most the sum over its carriers of the largest
@@ -342,12 +342,12 @@ bool fixed_possible(const lb_system* s) {
 
 // Chunked sweeps (lb_fixed_chunks.cu) of the small states the cluster sweep
 // took one cluster each: with the full stage tape, at least kChunkMinSteps
-// steps, and N^2 <= 144, where N (N + 1) / 2 columns per chunk cost less than the idle
+// steps, and N^2 <= 128, where N (N + 1) / 2 columns per chunk cost less than the idle
 // SMs.  A chunk starts its predictor cold, so a step takes more iterations
 // there: max_iter must leave room for a cold start at rho = 1/4.
-constexpr int kChunkMaxV = 144, kChunkMinSteps = 64, kChunkMinIter = 64;
+constexpr int kChunkMinSteps = 64, kChunkMinIter = 64;
 bool chunks_possible(const lb_system* s) {
-  return !use_grid(s) && s->V <= kChunkMaxV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&
+  return !use_grid(s) && s->V <= lbk::kFxChunkV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&
          s->sweep != LB_SWEEP_RESIDENT && fixed_cfg(s, false).QT > 0;
 }
 // steps per chunk: the chunks of steps run at the same time, the C boundary
@@ -357,7 +357,7 @@ int chunk_steps(const lb_system* s) {
 }
 
 // Whether this call runs the fixed-point sweeps: the Jacobi iteration with
-// rho_j <= 1/4, where its sums stay inside 64 bits.
+// rho_j <= 0.24, where its sums stay inside 64 bits.
 bool use_fixed(const lb_system* s, bool herm) {
   if (!s->fx_ws || s->method != LB_SOLVER_JACOBI) return false;
   if (use_grid(s)) return rho_bound(s) <= lbk::kGridFixedRho;
@@ -1916,6 +1916,15 @@ int lb_apply(lb_system* s, void* stream, int32_t adjoint, int64_t step, const vo
   if (rc) return rc;
   rc = ensure_ctab(s, st);
   if (rc) return rc;
+  // many elements: the off-diagonal part in fixed point, split into the sweeps'
+  // iterate buffer of M states (every control factor within its range)
+  if (use_grid(s) && s->fx_ws && n_vec <= s->M && (long long)n_vec * s->V >= lbk::kApplyFixedElements &&
+      rho_bound(s) <= lbk::kFixedRho) {
+    LB_CUDA(lbk::launch_apply_gx(s->dp, s->hp, adjoint, step, static_cast<const double2*>(x_dev),
+                                 static_cast<double2*>(y_dev), n_vec, st),
+            "apply kernels");
+    return LB_OK;
+  }
   LB_CUDA(lbk::launch_apply(s->dp, s->hp, adjoint, step, static_cast<const double2*>(x_dev), static_cast<double2*>(y_dev),
                             n_vec, st),
           "apply kernel");

@@ -26,8 +26,7 @@ struct FxG {
   long long ar, ai, br, bi;
 };
 __device__ __forceinline__ long long fx_prod(long long a, long long b) {
-  // 2^30 for rounding and 2^29 for the mean of the left-out low product
-  FxAcc s{0, (1LL << 30) + (1LL << 29)};
+  FxAcc s = fx_acc();
   fx_mac(s, fx_split(a), fx_split(b));
   return fx_val(s);
 }
@@ -90,14 +89,14 @@ __device__ __forceinline__ void fx_grad(const FxState<E, QT>& st, const FxSmem& 
     for (int q = 0; q < Q; ++q) {
       FxG g{0, 0, 0, 0};
       const FxSub b = S.sub[q];
-      const int n = b.n_sh & 0xff, sh = (b.n_sh >> 8) & 0xff, s = b.s, sN = s * H.N, dm = H.dm;
-      const Fx *cu = S.cu + b.co, *cd = S.cd + b.co, *z = zh + im;
+      const int sh = (b.n_sh >> 8) & 0xff, s = b.s, sN = s * H.N, dm = H.dm;
+      const int4 *ck = S.ck + b.co, *cl = S.cl + b.co;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int v = fx_v(st, S, H, e);
         if (v < V) {
           const Cx Z = Zt[v];
-          const FxPR p = fx_pr_tab(z, cu, cd, n, s, sN, v, (st.kd[e] >> sh) & dm, (st.ld[e] >> sh) & dm);
+          const FxPR p = fx_pr_tab(zh + 2 * v + im, ck[(st.kd[e] >> sh) & dm], cl[(st.ld[e] >> sh) & dm], s, sN);
           fx_grad_acc(g, p, im ? Z.y : Z.x, im ? Z.x : Z.y, im, H.herm ? (fx_m(st, S, H, e) >= 0 ? 1 : 2) : 0);
         }
       }
@@ -337,7 +336,7 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_backward_fx(const Prob
       if (QT == 0 || mode == 0) {
         fx_grad(st, S, zh, Zt, Z, gstep);
         jprev = j;
-        sprev = sz + st.sc - 62;
+        sprev = sz + st.sc - 64;
         ++gstep;
       }
       // qhat^j = 2 zhat - qhat^{j+1}, plus the penalty's source

@@ -17,7 +17,7 @@
 //   5. every (chunk, state) pair runs its adjoint steps and gradient pieces.
 // The results are those of the sequential sweep up to rounding.  The work
 // grows by N (N + 1) / 2 columns against the M states of the problem, which
-// the idle SMs and the overlap of many CTAs per SM pay for while N^2 <= 144.
+// the idle SMs and the overlap of many CTAs per SM pay for while N^2 <= 128.
 
 #include "lb_fixed_sweep.cuh"
 
@@ -25,11 +25,11 @@ namespace lbk {
 
 namespace {
 
-constexpr int kPShift = 61;  // fraction bits of the propagators' entries (at most 1 in magnitude, up to the step error)
+constexpr int kPShift = 62;  // the propagators' entries (at most 1 in magnitude, up to the step error) as coefficients: a quarter
 
 // columns of the chunks' propagators: CTA (chunk, column)
 template <int QT>
-__global__ void __launch_bounds__(fx_max_threads<QT>()) k_columns_fx(const ProbDev* __restrict__ pp) {
+__global__ void __launch_bounds__(2 * kFxChunkV, 3) k_columns_fx(const ProbDev* __restrict__ pp) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
   const int Vc = P.N * (P.N + 1) / 2, ch = blockIdx.x / Vc, col = blockIdx.x % Vc;
@@ -65,19 +65,23 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_columns_fx(const ProbD
   }
 }
 
-// shared memory of the boundary products
+// Boundary products.  One CTA per state multiplies it by the chunks' propagators
+// one after another; a chunk's matrix is fetched into shared memory while the
+// one before is used (two buffers; read from global memory when they do not fit),
+// and every thread sums a share of a column (forward) or row (adjoint) group.
 struct FxCombine {
-  longlong2* part;  // [G][V] partial sums (forward), [V] new values (adjoint)
+  longlong2* part;  // [G][V] partial sums
   int4* x;          // [V] the state, split
   int* vkl;         // [Vc] vec index of column e's |k><l|
   int* vlk;         // [Vc] ... of |l><k| (-1 on the diagonal)
   unsigned long long* mx;  // [32]
+  int4* mat;        // [2][Vc * V], or null
 };
-__host__ __device__ inline size_t fx_combine_bytes(int V, int Vc, int G) {
+__host__ __device__ inline size_t fx_combine_bytes(int V, int Vc, int G, bool stage) {
   return align16(sizeof(longlong2) * (size_t)G * V) + sizeof(int4) * V + align16(sizeof(int) * Vc) * 2 +
-         sizeof(unsigned long long) * 32;
+         sizeof(unsigned long long) * 32 + (stage ? sizeof(int4) * 2 * (size_t)Vc * V : 0);
 }
-__device__ FxCombine fx_combine_carve(unsigned char* base, const ProbDev& P, int G) {
+__device__ FxCombine fx_combine_carve(unsigned char* base, const ProbDev& P, int G, bool stage) {
   FxCombine S;
   const int V = P.V, Vc = P.N * (P.N + 1) / 2;
   size_t o = 0;
@@ -90,6 +94,8 @@ __device__ FxCombine fx_combine_carve(unsigned char* base, const ProbDev& P, int
   S.vlk = reinterpret_cast<int*>(base + o);
   o += align16(sizeof(int) * Vc);
   S.mx = reinterpret_cast<unsigned long long*>(base + o);
+  o += sizeof(unsigned long long) * 32;
+  S.mat = stage ? reinterpret_cast<int4*>(base + o) : nullptr;
   for (int e = threadIdx.x; e < Vc; e += blockDim.x) {
     const uint32_t t = P.hkl[e];
     const int k = (int)(t & 0xffffu), l = (int)(t >> 16);
@@ -98,6 +104,28 @@ __device__ FxCombine fx_combine_carve(unsigned char* base, const ProbDev& P, int
   }
   __syncthreads();
   return S;
+}
+// chunk c's matrix on its way to buffer c & 1 (c < 0 or >= C: nothing)
+__device__ __forceinline__ void fx_fetch(const FxCombine& S, const ProbDev& P, int c) {
+  if (!S.mat) return;
+  if (c >= 0 && c < P.chunkC) {
+    const int n = P.N * (P.N + 1) / 2 * P.V;
+    const int4* src = P.pmat + (size_t)c * n;
+    int4* dst = S.mat + (size_t)(c & 1) * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(dst + i));
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src + i) : "memory");
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// wait for every matrix but the newest fetched; the matrix of chunk c
+__device__ __forceinline__ const int4* fx_fetched(const FxCombine& S, const ProbDev& P, int c) {
+  const size_t n = (size_t)(P.N * (P.N + 1) / 2) * P.V;
+  if (!S.mat) return P.pmat + c * n;
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+  __syncthreads();
+  return S.mat + (c & 1) * n;
 }
 __device__ unsigned long long fx_block_max(unsigned long long* w, unsigned long long m) {
   m = warp_max_u64(m);
@@ -108,12 +136,12 @@ __device__ unsigned long long fx_block_max(unsigned long long* w, unsigned long 
   __syncthreads();
   return m;
 }
-// a += A x (conj: A^* x) for split A and x (half of it: the entries have 61
-// fraction bits), folded into 64-bit sums that may wrap before the last
+// a += A x / 4 (conj: A^* x / 4) for split A and x, folded into 64-bit sums
+// that may wrap before the last
 template <bool CONJ>
 __device__ __forceinline__ void fx_cmac(long long& re, long long& im, int4 A, int4 x) {
   const Fx ax{A.x, A.y}, ay{A.z, A.w}, xr{x.x, x.y}, xi{x.z, x.w};
-  FxAcc r = fx_acc(CONJ ? ax.l + ay.l : ax.l - ay.l), i = fx_acc(CONJ ? ax.l - ay.l : ax.l + ay.l);
+  FxAcc r = fx_acc(), i = fx_acc();
   fx_mac(r, ax, xr);
   fx_mac(r, CONJ ? ay : fx_neg(ay), xi);
   fx_mac(i, ax, xi);
@@ -127,41 +155,73 @@ __device__ __forceinline__ int4 fx_split2(Cx q) {
 }
 
 // Take the value of entry threadIdx.x (< V, else ignored) of the next boundary
-// state: set its scale by its largest entry, keep it split in S.x and store it.
+// state, plus `add` (ADD): set its scale by its largest entry, keep it split in
+// S.x and store it.
+template <bool ADD>
 __device__ void fx_boundary(const FxCombine& S, const ProbDev& P, Cx q, double2 add, int& sc, int V, size_t b) {
   const int t = threadIdx.x;
-  double2 d = make_double2(0.0, 0.0);
-  if (t < V) d = make_double2(fx_to(q.x, sc) + add.x, fx_to(q.y, sc) + add.y);
-  const unsigned long long mx = fx_block_max(S.mx, t < V ? umax64(abs_bits(d.x), abs_bits(d.y)) : 0ull);
-  const int ns = mx && mx < kInfBits ? fx_scale(mx) : sc;
-  const int s = sc - ns;
-  sc = ns;
+  int s = 0;
+  if (ADD) {
+    double2 d = make_double2(0.0, 0.0);
+    if (t < V) d = make_double2(fx_to(q.x, sc) + add.x, fx_to(q.y, sc) + add.y);
+    const unsigned long long mx = fx_block_max(S.mx, t < V ? umax64(abs_bits(d.x), abs_bits(d.y)) : 0ull);
+    if (mx && mx < kInfBits) s = sc - fx_scale(mx);
+  } else {
+    unsigned* w = reinterpret_cast<unsigned*>(S.mx);
+    const unsigned m = __reduce_max_sync(kFull, t < V ? max(fx_hi_abs(q.x), fx_hi_abs(q.y)) : 0u);
+    if ((t & 31) == 0) w[t >> 5] = m;
+    __syncthreads();
+    const unsigned top = __reduce_max_sync(kFull, (t & 31) < (int)(blockDim.x >> 5) ? w[t & 31] : 0u);
+    // the top bit of the largest high word to bit 27: the largest entry in [2^59, 2^60)
+    if (top && (top >= kFxHigh || top < kFxLow)) s = 4 - __clz(top);
+  }
+  sc -= s;
   if (t < V) {
-    q.x = fx_shift(q.x, s) + fx_from(add.x, sc);
-    q.y = fx_shift(q.y, s) + fx_from(add.y, sc);
+    q.x = fx_shift(q.x, s);
+    q.y = fx_shift(q.y, s);
+    if (ADD) {
+      q.x += fx_from(add.x, sc);
+      q.y += fx_from(add.y, sc);
+    }
     S.x[t] = fx_split2(q);
     P.bst[b * V + t] = make_longlong2(q.x, q.y);
   }
   if (t == 0) P.bsc[b] = sc;
   __syncthreads();
 }
+// entry threadIdx.x of the product from the G partial sums (a quarter each)
+__device__ __forceinline__ Cx fx_take(const FxCombine& S, int G, int V) {
+  Cx q{0, 0};
+  if ((int)threadIdx.x < V) {
+    for (int k = 0; k < G; ++k) {
+      const longlong2 p = S.part[k * V + threadIdx.x];
+      q.x += p.x;
+      q.y += p.y;
+    }
+    q.x <<= 2;
+    q.y <<= 2;
+  }
+  return q;
+}
 
-// boundary states: CTA per state, thread (g, v) the columns e = g, g + G, ...
-__global__ void __launch_bounds__(1024) k_boundary_fx(const ProbDev* __restrict__ pp, int G) {
+// boundary states: thread (g, v) sums entry v over the columns e = g, g + G, ...
+__global__ void __launch_bounds__(1024) k_boundary_fx(const ProbDev* __restrict__ pp, int G, int stage) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
   const int V = P.V, N = P.N, Vc = N * (N + 1) / 2, M = P.M, i = blockIdx.x, t = threadIdx.x;
-  const FxCombine S = fx_combine_carve(smem, P, G);
+  const FxCombine S = fx_combine_carve(smem, P, G, stage);
+  fx_fetch(S, P, 0);
   const double2 q0 = t < V ? P.q0[(size_t)i * V + t] : make_double2(0.0, 0.0);
   const unsigned long long mx = fx_block_max(S.mx, umax64(abs_bits(q0.x), abs_bits(q0.y)));
   const bool bad = mx >= kInfBits;
   if (bad && t == 0) record_error(P.status, LB_ENAN, 0);
   int sc = kFxTop;
-  fx_boundary(S, P, Cx{0, 0}, bad ? make_double2(0.0, 0.0) : q0, sc, V, i);
+  fx_boundary<true>(S, P, Cx{0, 0}, bad ? make_double2(0.0, 0.0) : q0, sc, V, i);
   const int g = t / V, v = t - g * V, vt = v / N + N * (v % N);
   for (int c = 0; c < P.chunkC; ++c) {
+    fx_fetch(S, P, c + 1);
+    const int4* A = fx_fetched(S, P, c);
     if (g < G) {
-      const int4* A = P.pmat + (size_t)c * Vc * V;
       long long re = 0, im = 0;
 #pragma unroll 4
       for (int e = g; e < Vc; e += G) {
@@ -173,27 +233,19 @@ __global__ void __launch_bounds__(1024) k_boundary_fx(const ProbDev* __restrict_
       S.part[g * V + v] = make_longlong2(re, im);
     }
     __syncthreads();
-    Cx q{0, 0};
-    if (t < V) {
-      for (int k = 0; k < G; ++k) {
-        q.x += S.part[k * V + t].x;
-        q.y += S.part[k * V + t].y;
-      }
-      q.x <<= 1;
-      q.y <<= 1;
-    }
-    fx_boundary(S, P, q, make_double2(0.0, 0.0), sc, V, (size_t)(c + 1) * M + i);
+    fx_boundary<false>(S, P, fx_take(S, G, V), make_double2(0.0, 0.0), sc, V, (size_t)(c + 1) * M + i);
   }
 }
 
-// adjoint states at the boundaries: CTA per state, warp per column
-__global__ void __launch_bounds__(1024) k_boundary_adj_fx(const ProbDev* __restrict__ pp) {
+// adjoint states at the boundaries: thread (e, g) sums the products with
+// columns |k><l| and |l><k| of pair e over the entries v = g, g + G, ...
+__global__ void __launch_bounds__(1024) k_boundary_adj_fx(const ProbDev* __restrict__ pp, int G, int stage) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
   const int V = P.V, N = P.N, Vc = N * (N + 1) / 2, M = P.M, i = blockIdx.x, t = threadIdx.x;
-  const int lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5;
-  const FxCombine S = fx_combine_carve(smem, P, 1);
+  const FxCombine S = fx_combine_carve(smem, P, G, stage);
   const size_t base = (size_t)i * V, C1 = P.chunkC + 1;
+  fx_fetch(S, P, P.chunkC - 1);
   // terminal condition qhat^{N_T} = beta_i/M g_i (Appendix B)
   double2 lam = make_double2(0.0, 0.0);
   if (t < V) {
@@ -211,43 +263,37 @@ __global__ void __launch_bounds__(1024) k_boundary_adj_fx(const ProbDev* __restr
   const bool bad = mx >= kInfBits;
   if (bad && t == 0) record_error(P.status, LB_ENAN, P.NT - 1);
   int sc = kFxTop;
-  fx_boundary(S, P, Cx{0, 0}, bad ? make_double2(0.0, 0.0) : lam, sc, V, (C1 + P.chunkC) * M + i);
+  fx_boundary<true>(S, P, Cx{0, 0}, bad ? make_double2(0.0, 0.0) : lam, sc, V, (C1 + P.chunkC) * M + i);
+  const int e = t / G, g = t - e * G;
   for (int c = P.chunkC - 1; c >= 0; --c) {
-    const int4* A = P.pmat + (size_t)c * Vc * V;
-    for (int e = warp; e < Vc; e += nwarps) {
+    fx_fetch(S, P, c - 1);
+    const int4* A = fx_fetched(S, P, c);
+    if (e < Vc) {
       // <P(|k><l|), lam> and <P(|l><k|), lam>
       long long ar = 0, ai = 0, br = 0, bi = 0;
 #pragma unroll 3
-      for (int v = lane; v < V; v += 32) {
+      for (int v = g; v < V; v += G) {
         const int4 a = A[(size_t)e * V + v];
         fx_cmac<true>(ar, ai, a, S.x[v]);
         fx_cmac<false>(br, bi, a, S.x[v / N + N * (v % N)]);
       }
-#pragma unroll
-      for (int o = 16; o; o >>= 1) {
-        ar += __shfl_xor_sync(kFull, ar, o);
-        ai += __shfl_xor_sync(kFull, ai, o);
-        br += __shfl_xor_sync(kFull, br, o);
-        bi += __shfl_xor_sync(kFull, bi, o);
-      }
-      if (lane == 0) {
-        S.part[S.vkl[e]] = make_longlong2(ar << 1, ai << 1);
-        if (S.vlk[e] >= 0) S.part[S.vlk[e]] = make_longlong2(br << 1, bi << 1);
-      }
+      S.part[g * V + S.vkl[e]] = make_longlong2(ar, ai);
+      if (S.vlk[e] >= 0) S.part[g * V + S.vlk[e]] = make_longlong2(br, bi);
     }
     __syncthreads();
-    Cx q{0, 0};
-    double2 add = make_double2(0.0, 0.0);
-    if (t < V) {
-      q = Cx{S.part[t].x, S.part[t].y};
-      if (P.gamma1 != 0.0) {
-        // the chunk's response to its own penalty sources
+    const Cx q = fx_take(S, G, V);
+    if (P.gamma1 != 0.0) {
+      // the chunk's response to its own penalty sources
+      double2 add = make_double2(0.0, 0.0);
+      if (t < V) {
         const size_t b = (2 * C1 + c) * M + i;
         const longlong2 r = P.bst[b * V + t];
         add = make_double2(fx_to(r.x, P.bsc[b]), fx_to(r.y, P.bsc[b]));
       }
+      fx_boundary<true>(S, P, q, add, sc, V, (C1 + c) * M + i);
+    } else {
+      fx_boundary<false>(S, P, q, make_double2(0.0, 0.0), sc, V, (C1 + c) * M + i);
     }
-    fx_boundary(S, P, q, add, sc, V, (C1 + c) * M + i);
   }
 }
 
@@ -273,11 +319,27 @@ cudaError_t run_columns(const ProbDev* p, int n, const FixedConfig& fc, cudaStre
   return cudaGetLastError();
 }
 
-// threads of a boundary product: every entry of the state, times G column groups
+// thread groups of a boundary product: 1024 threads over the V entries
+// (forward), or up to 16 per pair of columns (adjoint)
 int boundary_groups(int V, int Vc) {
-  int g = 1024 / V;
-  if (g < 1) g = 1;
-  return g < Vc ? g : Vc;
+  const int g = 1024 / V;
+  return g < 1 ? 1 : (g < Vc ? g : Vc);
+}
+int boundary_groups_adj(int V, int Vc) {
+  int g = 1024 / Vc;
+  if (g > 16) g = 16;
+  return g < V ? g : V;
+}
+// whether two matrices fit shared memory with G groups' sums, and the bytes
+template <class K>
+cudaError_t boundary_shape(K kern, int V, int Vc, int G, int* stage, size_t* smem) {
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  *stage = fx_combine_bytes(V, Vc, G, true) <= (size_t)optin;
+  *smem = fx_combine_bytes(V, Vc, G, *stage);
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
 }
 
 }  // namespace
@@ -294,7 +356,11 @@ cudaError_t launch_forward_chunks(const ProbDev* d_prob, const ProbDev& h, int t
   }
   if (e != cudaSuccess) return e;
   const int G = boundary_groups(h.V, Vc);
-  k_boundary_fx<<<h.M, (G * h.V + 31) / 32 * 32, fx_combine_bytes(h.V, Vc, G), s>>>(d_prob, G);
+  int stage = 0;
+  size_t smem = 0;
+  e = boundary_shape(k_boundary_fx, h.V, Vc, G, &stage, &smem);
+  if (e != cudaSuccess) return e;
+  k_boundary_fx<<<h.M, (G * h.V + 31) / 32 * 32, smem, s>>>(d_prob, G, stage);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = launch_forward_fixed_chunked(d_prob, h.M * h.chunkC, tape, fc, s);
@@ -308,8 +374,12 @@ cudaError_t launch_backward_chunks(const ProbDev* d_prob, const ProbDev& h, cons
   if (h.gamma1 != 0.0) e = launch_backward_fixed_chunked(d_prob, h.M * h.chunkC, 1, fc, s);
   if (e != cudaSuccess) return e;
   const int Vc = h.N * (h.N + 1) / 2;
-  const int threads = h.V <= 32 ? 256 : 1024;
-  k_boundary_adj_fx<<<h.M, threads, fx_combine_bytes(h.V, Vc, 1), s>>>(d_prob);
+  const int G = boundary_groups_adj(h.V, Vc);
+  int stage = 0;
+  size_t smem = 0;
+  e = boundary_shape(k_boundary_adj_fx, h.V, Vc, G, &stage, &smem);
+  if (e != cudaSuccess) return e;
+  k_boundary_adj_fx<<<h.M, (G * Vc + 31) / 32 * 32, smem, s>>>(d_prob, G, stage);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_backward_fixed_chunked(d_prob, h.M * h.chunkC, 0, fc, s);

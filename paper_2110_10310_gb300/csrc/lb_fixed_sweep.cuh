@@ -69,8 +69,8 @@ struct FxSub {
 struct FxSmem {
   Hdr* hdr;
   FxSub* sub;       // [Q]
-  Fx* cu;           // [ncoef] sqrt(n+1) 2^-kc of the subsystem (0 at the top level)
-  Fx* cd;           // [ncoef] sqrt(n) 2^-kc
+  int4* ck;         // [ncoef] (cu, cd): sqrt(n+1) 2^-kc of the subsystem (0 at the top level), sqrt(n) 2^-kc
+  int4* cl;         // [ncoef] (-cd, -cu)
   Fx* jf;           // [njcoef] decay factors
   Fx* ja;
   uint32_t* dig;    // [N]
@@ -87,15 +87,18 @@ struct FxSmem {
 
 __host__ __device__ inline size_t fx_smem_bytes(int ncoef, int njcoef, int N, int V, int Q, int cq, int nel, int QT) {
   size_t b = align16(sizeof(Hdr)) + sizeof(FxSub) * LB_MAXQ;
-  b += 2 * align16(sizeof(Fx) * ncoef) + 2 * align16(sizeof(Fx) * njcoef);
+  b += 2 * sizeof(int4) * ncoef + 2 * align16(sizeof(Fx) * njcoef);
   b += align16(sizeof(uint32_t) * N);
   b += 2 * align16(sizeof(uint16_t) * (size_t)N * (N + 1) / 2);
   b += sizeof(unsigned) * 128;
   b += sizeof(int4) * 2 * (cq + 1);
   b += align16(sizeof(int) * 2 * 4 * Q * kFxWarps * 3);
   b += sizeof(unsigned long long) * kFxWarps;
-  if (QT == 0) b += sizeof(int4) * (size_t)nel;
+  // the table path reads up to V/2 + N/2 entries before and after a buffer
+  const size_t pad = sizeof(Fx) * (size_t)(V + N);
+  if (QT == 0 && b < pad) b = align16(pad);
   b += sizeof(Fx) * 4 * (size_t)V;
+  if (QT == 0) b += sizeof(int4) * (size_t)nel > pad ? sizeof(int4) * (size_t)nel : pad;
   return b;
 }
 
@@ -109,8 +112,8 @@ __device__ FxSmem fx_carve(unsigned char* base, const ProbDev& P, int nel, int Q
   };
   S.hdr = reinterpret_cast<Hdr*>(take(sizeof(Hdr)));
   S.sub = reinterpret_cast<FxSub*>(take(sizeof(FxSub) * LB_MAXQ));
-  S.cu = reinterpret_cast<Fx*>(take(sizeof(Fx) * P.ncoef));
-  S.cd = reinterpret_cast<Fx*>(take(sizeof(Fx) * P.ncoef));
+  S.ck = reinterpret_cast<int4*>(take(sizeof(int4) * P.ncoef));
+  S.cl = reinterpret_cast<int4*>(take(sizeof(int4) * P.ncoef));
   S.jf = reinterpret_cast<Fx*>(take(sizeof(Fx) * P.njcoef));
   S.ja = reinterpret_cast<Fx*>(take(sizeof(Fx) * P.njcoef));
   S.dig = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * P.N));
@@ -120,15 +123,16 @@ __device__ FxSmem fx_carve(unsigned char* base, const ProbDev& P, int nel, int Q
   S.ctl = reinterpret_cast<int4*>(take(sizeof(int4) * 2 * (P.cq + 1)));
   S.gred = reinterpret_cast<int*>(take(sizeof(int) * 2 * 4 * P.Q * kFxWarps * 3));
   S.mx = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * kFxWarps));
-  S.dsm = reinterpret_cast<int4*>(QT == 0 ? take(sizeof(int4) * (size_t)nel) : nullptr);
+  const size_t pad = sizeof(Fx) * (size_t)(P.V + P.N);
+  if (QT == 0 && o < pad) o = align16(pad);
   S.zb0 = reinterpret_cast<Fx*>(take(sizeof(Fx) * 2 * (size_t)P.V));
   S.zb1 = reinterpret_cast<Fx*>(take(sizeof(Fx) * 2 * (size_t)P.V));
+  S.dsm = reinterpret_cast<int4*>(QT == 0 ? take(sizeof(int4) * (size_t)nel) : nullptr);
   return S;
 }
 
 __device__ __forceinline__ long long fx_from(double x, int sc) { return __double2ll_rn(scalbn(x, sc)); }
 __device__ __forceinline__ double fx_to(long long X, int sc) { return scalbn((double)X, -sc); }
-__device__ __forceinline__ long long fx_join(Fx a) { return ((long long)a.h << 31) + a.l; }
 __device__ __forceinline__ long long fx_other(long long x) { return __shfl_xor_sync(kFull, x, 1); }
 __device__ void fx_setup(const FxSmem& S, const ProbDev& P, int herm) {
   if (threadIdx.x == 0) {
@@ -154,12 +158,14 @@ __device__ void fx_setup(const FxSmem& S, const ProbDev& P, int herm) {
   for (int i = threadIdx.x; i < P.ncoef; i += blockDim.x) {
     int q = 0;
     while (q + 1 < P.Q && P.coff[q + 1] <= i) ++q;
-    S.cu[i] = fx_coef(__double2ll_rn(scalbn(P.cu[i], 62 - P.kc[q])));
-    S.cd[i] = fx_coef(__double2ll_rn(scalbn(P.cd[i], 62 - P.kc[q])));
+    const Fx u = fx_coef(__double2ll_rn(scalbn(P.cu[i], 64 - P.kc[q])));
+    const Fx d = fx_coef(__double2ll_rn(scalbn(P.cd[i], 64 - P.kc[q])));
+    S.ck[i] = make_int4(u.h, u.l, d.h, d.l);
+    S.cl[i] = make_int4(-d.h, -d.l, -u.h, -u.l);
   }
   for (int i = threadIdx.x; i < P.njcoef; i += blockDim.x) {
-    S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 62)));
-    S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 62)));
+    S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 64)));
+    S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 64)));
   }
   for (int i = threadIdx.x; i < P.N; i += blockDim.x) S.dig[i] = P.digits[i];
   for (int i = threadIdx.x; i < 128; i += blockDim.x) S.slots[i] = 0u;
@@ -245,10 +251,11 @@ __device__ void fx_plan(FxPlan<QT>& pl, const FxSmem& S, const ProbDev& P, int v
       pl.o[u][1] = at(v - (nl > 0 ? sN : 0));
       pl.o[u][2] = at(v - (nk > 0 ? s : 0));
       pl.o[u][3] = at(v + (nl + 1 < n ? sN : 0));
-      pl.c[u][0] = S.cu[co + nk];
-      pl.c[u][1] = fx_neg(S.cd[co + nl]);
-      pl.c[u][2] = S.cd[co + nk];
-      pl.c[u][3] = fx_neg(S.cu[co + nl]);
+      const int4 ck = S.ck[co + nk], cl = S.cl[co + nl];
+      pl.c[u][0] = Fx{ck.x, ck.y};
+      pl.c[u][1] = Fx{cl.x, cl.y};
+      pl.c[u][2] = Fx{ck.z, ck.w};
+      pl.c[u][3] = Fx{cl.z, cl.w};
       pl.oj[u][0] = at(v + ((nk + 1 < n && nl + 1 < n) ? s + sN : 0));
       pl.oj[u][1] = at(v - ((nk > 0 && nl > 0) ? s + sN : 0));
       pl.cj[u][0] = S.jf[jo];
@@ -259,7 +266,7 @@ __device__ void fx_plan(FxPlan<QT>& pl, const FxSmem& S, const ProbDev& P, int v
       const int np = H.lev[p], nq = H.lev[q], d = H.stride[q] - H.stride[p], cp = H.coff[p], cq = H.coff[q];
       const int pk = (kd >> (H.db * p)) & H.dm, qk = (kd >> (H.db * q)) & H.dm;
       const int pL = (ld >> (H.db * p)) & H.dm, qL = (ld >> (H.db * q)) & H.dm;
-      auto cf = [&](double a, double b) { return fx_coef(__double2ll_rn(scalbn(a * b, 62 - P.kc[u]))); };
+      auto cf = [&](double a, double b) { return fx_coef(__double2ll_rn(scalbn(a * b, 64 - P.kc[u]))); };
       pl.o[u][0] = at(v + ((pk > 0 && qk + 1 < nq) ? d : 0));
       pl.o[u][1] = at(v - ((qL > 0 && pL + 1 < np) ? d * H.N : 0));
       pl.o[u][2] = at(v - ((qk > 0 && pk + 1 < np) ? d : 0));
@@ -291,13 +298,10 @@ __device__ __forceinline__ void fx_unit(long long& own, long long& cross, const 
                                         Fx x5) {
   const Fx a{t.x, t.y}, b{t.z, t.w};
   const Fx u = fx_split(p.p + p.r), w = fx_split(p.p - p.r);
-  FxAcc o = fx_acc(b.l), x = fx_acc(a.l);
+  FxAcc o = fx_acc(), x = fx_acc();
   fx_mac(o, b, w);
   fx_mac(x, a, u);
-  if (decay) {
-    o.mid += (long long)(cj.l >> 1);
-    fx_mac(o, cj, x5);
-  }
+  if (decay) fx_mac(o, cj, x5);
   own += fx_val(o);
   cross += fx_val(x);
 }
@@ -306,13 +310,10 @@ __device__ __forceinline__ void fx_unit_adj(long long& own, long long& cross, co
                                             Fx x5) {
   const Fx a{t.x, t.y}, b{t.z, t.w};
   const Fx u = fx_split(p.p + p.r), w = fx_split(p.r - p.p);
-  FxAcc o = fx_acc(b.l), x = fx_acc(a.l);
+  FxAcc o = fx_acc(), x = fx_acc();
   fx_mac(o, b, w);
   fx_mac(x, a, u);
-  if (decay) {
-    o.mid += (long long)(cj.l >> 1);
-    fx_mac(o, cj, x5);
-  }
+  if (decay) fx_mac(o, cj, x5);
   own += fx_val(o);
   cross -= fx_val(x);
 }
@@ -340,33 +341,35 @@ __device__ __forceinline__ void fx_apply_plan(long long& own, long long& cross, 
     }
 }
 
-// neighbour combinations of a subsystem for an element of the table path (z
-// at the lane's component); cu, cd: the subsystem's ladder factors
-__device__ __forceinline__ FxPR fx_pr_tab(const Fx* __restrict__ z, const Fx* __restrict__ cu,
-                                          const Fx* __restrict__ cd, int n, int s, int sN, int v, int nk, int nl) {
-  return fx_pr(z[2 * (v + (nk + 1 < n ? s : 0))], z[2 * (v - (nl > 0 ? sN : 0))], z[2 * (v - (nk > 0 ? s : 0))],
-               z[2 * (v + (nl + 1 < n ? sN : 0))], cu[nk], fx_neg(cd[nl]), cd[nk], fx_neg(cu[nl]));
+// Neighbour combinations of a subsystem for an element of the table path, z at
+// the element and the lane's component, s and sN the strides in entries.  A
+// neighbour outside the range has the factor 0 and is read wherever it lies:
+// fx_carve leaves room for it on both sides of the iterate buffers.
+__device__ __forceinline__ FxPR fx_pr_tab(const Fx* __restrict__ z, int4 ck, int4 cl, int s, int sN) {
+  return fx_pr(z[2 * s], z[-2 * sN], z[-2 * s], z[2 * sN], Fx{ck.x, ck.y}, Fx{cl.x, cl.y}, Fx{ck.z, ck.w},
+               Fx{cl.z, cl.w});
 }
 // (not inlined: the element loops call it once per element; everything it
 // needs comes in registers)
 template <bool ADJ>
 __device__ __noinline__ Cx fx_apply_tab(const Fx* __restrict__ z, const FxSub* __restrict__ sub,
-                                        const Fx* __restrict__ cu, const Fx* __restrict__ cd,
-                                        const Fx* __restrict__ cj, const int4* __restrict__ ctl, int QN, int v,
-                                        uint32_t kd, uint32_t ld) {
+                                        const int4* __restrict__ ck, const int4* __restrict__ cl,
+                                        const Fx* __restrict__ cj, const int4* __restrict__ ctl, int QN, uint32_t kd,
+                                        uint32_t ld) {
   // QN: Q | N << 8 | bits of a digit << 24
   const int Q = QN & 0xff, N = (QN >> 8) & 0xffff, dm = (1 << (QN >> 24)) - 1;
   Cx r{0, 0};
+#pragma unroll 1
   for (int q = 0; q < Q; ++q) {
     const FxSub b = sub[q];
-    const int n = b.n_sh & 0xff, sh = (b.n_sh >> 8) & 0xff, s = b.s, sN = s * N;
+    const int sh = (b.n_sh >> 8) & 0xff, s = b.s, sN = s * N;
     const int nk = (kd >> sh) & dm, nl = (ld >> sh) & dm;
-    const FxPR p = fx_pr_tab(z, cu + b.co, cd + b.co, n, s, sN, v, nk, nl);
+    const FxPR p = fx_pr_tab(z, ck[b.co + nk], cl[b.co + nl], s, sN);
     const bool dec = b.n_sh >> 16;
     Fx c5{0, 0}, x5{0, 0};
     if (dec) {
-      c5 = cj[b.jo + nk * n + nl];
-      x5 = z[2 * (ADJ ? v - ((nk > 0 && nl > 0) ? s + sN : 0) : v + ((nk + 1 < n && nl + 1 < n) ? s + sN : 0))];
+      c5 = cj[b.jo + nk * (b.n_sh & 0xff) + nl];
+      x5 = z[ADJ ? -2 * (s + sN) : 2 * (s + sN)];
     }
     if (ADJ)
       fx_unit_adj(r.x, r.y, p, ctl[q], dec, c5, x5);
@@ -376,15 +379,18 @@ __device__ __noinline__ Cx fx_apply_tab(const Fx* __restrict__ z, const FxSub* _
   return r;
 }
 
+// ax own + s oth
+__device__ __forceinline__ long long fx_cmuls(Fx ax, Fx s, long long own, long long oth) {
+  FxAcc a = fx_acc();
+  fx_mac(a, ax, fx_split(own));
+  fx_mac(a, s, fx_split(oth));
+  return fx_val(a);
+}
 // component c of (ax + i ay) t for t_c = own, t_{1-c} = oth; ADJ: the conjugate factor
 template <bool ADJ>
 __device__ __forceinline__ long long fx_cmulc(Fx ax, Fx ay, long long own, long long oth, bool im) {
   // real: ax x - ay y, imaginary: ax y + ay x
-  const Fx s = im != ADJ ? ay : fx_neg(ay);
-  FxAcc a = fx_acc(ax.l + s.l);
-  fx_mac(a, ax, fx_split(own));
-  fx_mac(a, s, fx_split(oth));
-  return fx_val(a);
+  return fx_cmuls(ax, im != ADJ ? ay : fx_neg(ay), own, oth);
 }
 
 // ---------------------------------------------------------------------------
@@ -415,7 +421,7 @@ struct FxState {
   int v[1], m[1];          // QT > 0: vec index (V: none) and mirror (-1: none)
   uint32_t kd[E], ld[E];   // QT == 0: packed digits
   FxPlan<QT> pl;
-  Fx dx, dy;               // QT > 0: (I - dt/2 D)^-1 - 1
+  Fx dx, dy;               // QT > 0: (I - dt/2 D)^-1 - 1, its imaginary part negated in the real lane
   bool im;                 // the lane's component
   long long q[E];          // right-hand side of the step (q^j, or the adjoint's qhat^{j+1}), its component
   int sc;                  // its scale: X = x 2^sc
@@ -481,9 +487,9 @@ __device__ void fx_init(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P) {
     fx_plan<QT>(st.pl, S, P, st.v[0]);
     const int4 d = v < H.V ? fx_dinv1(P.D[v], hh) : make_int4(0, 0, 0, 0);
     st.dx = Fx{d.x, d.y};
-    st.dy = Fx{d.z, d.w};
-    st.pr.u = v < H.V ? fx_frame(P.D[v], hh) : Cx{1LL << 61, 0};
-    st.pr.p = Cx{1LL << 61, 0};
+    st.dy = st.im ? Fx{d.z, d.w} : fx_neg(Fx{d.z, d.w});
+    st.pr.u = v < H.V ? fx_frame(P.D[v], hh) : Cx{kFxPhase1, 0};
+    st.pr.p = Cx{kFxPhase1, 0};
     st.pr.s = 0;
 #pragma unroll
     for (int k = 0; k < kFxOrder; ++k) st.pr.d[k] = 0;
@@ -596,7 +602,7 @@ __device__ __noinline__ long long fx_ring_sum(const long long* __restrict__ ring
   } else {
     for (int i = 0; i < n; ++i) term(i);
   }
-  return (hi << 31) + lo;
+  return (long long)((unsigned long long)hi << 32) + lo;
 }
 
 // One implicit-midpoint solve (I - dt/2 M) z = q (ADJ: M^+) of the CTA's
@@ -627,15 +633,15 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
     long long t = q;
     if (pred) {
       if (st.n == 0) {
-        st.pr.p = Cx{1LL << 61, 0};
+        st.pr.p = Cx{kFxPhase1, 0};
         st.pr.s = 0;
       } else if (st.frame) {
-        t += fx_cmulc<ADJ>(fx_coef(st.pr.p.x), fx_coef(st.pr.p.y), st.pr.s, fx_other(st.pr.s), im) << 1;
+        t += fx_cmulc<ADJ>(fx_coef(st.pr.p.x), fx_coef(st.pr.p.y), st.pr.s, fx_other(st.pr.s), im) << 2;
       } else {
         t += st.pr.s;
       }
     }
-    zr = t + fx_cmulc<ADJ>(st.dx, st.dy, t, fx_other(t), im);
+    zr = t + fx_cmuls(st.dx, ADJ ? fx_neg(st.dy) : st.dy, t, fx_other(t));
     if (st.v[0] < V) fx_put(cur ? S.zb0 : S.zb1, st.v[0], st.m[0], im, zr);
   } else {
 #pragma unroll
@@ -652,7 +658,7 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
         d = S.dsm[fx_u<E, QT>(e)];
         if (pred) {
           if (st.n == 0) {
-            if (!im) st.pr.ph[v] = Cx{1LL << 61, 0};
+            if (!im) st.pr.ph[v] = Cx{kFxPhase1, 0};
           } else {
             s = fx_ring_sum(st.pr.ring + 2 * v + im, st.pr.stride, st.slot, st.n);
             if (st.frame) p = st.pr.ph[v];
@@ -660,7 +666,7 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
         }
       }
       if (pred && st.frame && st.n > 0)
-        s = fx_cmulc<ADJ>(fx_coef(p.x), fx_coef(p.y), s, fx_other(s), im) << 1;
+        s = fx_cmulc<ADJ>(fx_coef(p.x), fx_coef(p.y), s, fx_other(s), im) << 2;
       t += s;
       t += fx_cmulc<ADJ>(Fx{d.x, d.y}, Fx{d.z, d.w}, t, fx_other(t), im);
       if (ok) fx_put(cur ? S.zb0 : S.zb1, v, fx_m(st, S, H, e), im, t);
@@ -688,7 +694,7 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
       const long long t0 = st.q[0] + own, to = fx_other(t0), xo = fx_other(cross);
       const long long t = im ? t0 - xo : t0 + xo, o = im ? to + cross : to - cross;
       cr = t - st.q[0];
-      const long long z = t + fx_cmulc<ADJ>(st.dx, st.dy, t, o, im);
+      const long long z = t + fx_cmuls(st.dx, ADJ ? fx_neg(st.dy) : st.dy, t, o);
       if (st.v[0] < V) {
         fx_put(zn, st.v[0], st.m[0], im, z);
         dm = fx_abs_sat(z - zr);
@@ -703,7 +709,7 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
         int4 d = make_int4(0, 0, 0, 0);
         Cx p{0, 0};
         if (ok) {
-          r = fx_apply_tab<ADJ>(zc + im, S.sub, S.cu, S.cd, ADJ ? S.ja : S.jf, ctl, qn, v, st.kd[e], st.ld[e]);
+          r = fx_apply_tab<ADJ>(zc + 2 * v + im, S.sub, S.ck, S.cl, ADJ ? S.ja : S.jf, ctl, qn, st.kd[e], st.ld[e]);
           d = S.dsm[fx_u<E, QT>(e)];
           if (pred && st.frame) p = st.pr.ph[v];
         }
@@ -713,7 +719,7 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
         if (pred) {
           // the correction in the frame, to the ring slot of this step
           long long c = t - st.q[e];
-          if (st.frame) c = fx_cmulc<!ADJ>(fx_coef(p.x), fx_coef(p.y), c << 1, fx_other(c) << 1, im);
+          if (st.frame) c = fx_cmulc<!ADJ>(fx_coef(p.x), fx_coef(p.y), c << 2, fx_other(c) << 2, im);
           if (ok) st.pr.ring[(size_t)st.slot * st.pr.stride + 2 * v + im] = c;
         }
         if (ok) {
@@ -740,10 +746,10 @@ __device__ __forceinline__ void fx_commit(FxState<E, QT>& st, const FxSmem& S, l
   if constexpr (QT > 0) {
     long long c = cr;
     if (st.frame) {
-      c = fx_cmulc<!ADJ>(fx_coef(st.pr.p.x), fx_coef(st.pr.p.y), cr << 1, fx_other(cr) << 1, st.im);
-      // p <- p u (both halved: the product is a quarter)
+      c = fx_cmulc<!ADJ>(fx_coef(st.pr.p.x), fx_coef(st.pr.p.y), cr << 2, fx_other(cr) << 2, st.im);
+      // p <- p u (both quarters: the product is a sixteenth)
       const Cx w = fx_cmul(fx_coef(st.pr.u.x), fx_coef(st.pr.u.y), st.pr.p);
-      st.pr.p = Cx{w.x << 1, w.y << 1};
+      st.pr.p = Cx{w.x << 2, w.y << 2};
     }
     // the newest difference of order n is the prediction's error; the lower
     // ones follow by adding it up
@@ -778,7 +784,7 @@ __device__ __forceinline__ void fx_commit(FxState<E, QT>& st, const FxSmem& S, l
       if (v < H.V && !st.im) {
         const Cx u = st.pr.fu[v];
         const Cx w = fx_cmul(fx_coef(u.x), fx_coef(u.y), st.pr.ph[v]);
-        st.pr.ph[v] = Cx{w.x << 1, w.y << 1};
+        st.pr.ph[v] = Cx{w.x << 2, w.y << 2};
       }
     }
     __syncwarp();

@@ -24,6 +24,7 @@ namespace lbk {
 namespace {
 
 constexpr int kGxWarps = kGridThreads / 32;
+constexpr int kGxBlocks = 2;  // blocks per SM
 
 // kernel parameter: what the element loops need of the system, in the
 // constant bank (the subsystem loop is unrolled for QN > 0)
@@ -43,7 +44,7 @@ struct GxSmem {
   Fx* ja;
   int4* ctl;      // [LB_MAXQ] this solve's control factors (a, b), negated for the adjoint
   unsigned* red;  // [kLocal][kGxWarps]
-  double* dred;   // [4][kGxWarps]
+  longlong2* gs;  // [kGxQP][4][kGxWarps] the warps' gradient sums
   int* flag;      // [0] decision, [1] stopping factor (float bits)
   int* sc;        // [M] scale of each state
   int* sh;        // [M] the commit's change of it
@@ -51,7 +52,7 @@ struct GxSmem {
 
 __host__ __device__ inline size_t gx_smem_bytes(int ncoef, int njcoef, int M) {
   return align16(sizeof(GridHdr)) + sizeof(int4) * ncoef + 2 * align16(sizeof(Fx) * njcoef) + sizeof(int4) * LB_MAXQ +
-         align16(sizeof(unsigned) * 4 * kGxWarps) + sizeof(double) * 4 * kGxWarps + 16 + 2 * align16(sizeof(int) * M);
+         align16(sizeof(unsigned) * 4 * kGxWarps) + sizeof(longlong2) * 12 * kGxWarps + 16 + 2 * align16(sizeof(int) * M);
 }
 
 __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, int herm) {
@@ -68,7 +69,7 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
   S.ja = reinterpret_cast<Fx*>(take(sizeof(Fx) * P.njcoef));
   S.ctl = reinterpret_cast<int4*>(take(sizeof(int4) * LB_MAXQ));
   S.red = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * 4 * kGxWarps));
-  S.dred = reinterpret_cast<double*>(take(sizeof(double) * 4 * kGxWarps));
+  S.gs = reinterpret_cast<longlong2*>(take(sizeof(longlong2) * 12 * kGxWarps));
   S.flag = reinterpret_cast<int*>(take(16));
   S.sc = reinterpret_cast<int*>(take(sizeof(int) * P.M));
   S.sh = reinterpret_cast<int*>(take(sizeof(int) * P.M));
@@ -84,13 +85,13 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
   for (int i = threadIdx.x; i < P.ncoef; i += blockDim.x) {
     int q = 0;
     while (q + 1 < P.Q && P.coff[q + 1] <= i) ++q;
-    const Fx u = fx_coef(__double2ll_rn(scalbn(P.cu[i], 62 - P.kc[q])));
-    const Fx d = fx_coef(__double2ll_rn(scalbn(P.cd[i], 62 - P.kc[q])));
+    const Fx u = fx_coef(__double2ll_rn(scalbn(P.cu[i], 64 - P.kc[q])));
+    const Fx d = fx_coef(__double2ll_rn(scalbn(P.cd[i], 64 - P.kc[q])));
     S.cc[i] = make_int4(u.h, u.l, d.h, d.l);
   }
   for (int i = threadIdx.x; i < P.njcoef; i += blockDim.x) {
-    S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 62)));
-    S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 62)));
+    S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 64)));
+    S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 64)));
   }
   for (int i = threadIdx.x; i < P.M; i += blockDim.x) S.sc[i] = S.sh[i] = 0;
   __syncthreads();
@@ -102,7 +103,7 @@ __device__ __forceinline__ int4 gx_pack(Cx z) {
   return make_int4(a.h, a.l, b.h, b.l);
 }
 __device__ __forceinline__ Cx gx_join(int4 p) {
-  return Cx{((long long)p.x << 31) + p.y, ((long long)p.z << 31) + p.w};
+  return Cx{fx_join(Fx{p.x, p.y}), fx_join(Fx{p.z, p.w})};
 }
 __device__ __forceinline__ Cx gx_ld(const double2* p) {
   const longlong2 a = *reinterpret_cast<const longlong2*>(p);
@@ -248,14 +249,12 @@ __device__ __forceinline__ Cx gx_apply(const int4* __restrict__ z, const GxParam
       }
       x5 = z[o];
     }
-    FxAcc cr = fx_acc(bb.l + a.l), ci = fx_acc(bb.l - a.l);
+    FxAcc cr = fx_acc(), ci = fx_acc();
     fx_mac(cr, bb, wx);
     fx_mac(cr, a, uy);
     fx_mac(ci, bb, wy);
     fx_mac(ci, fx_neg(a), ux);
     if (b.decay) {
-      cr.mid += (long long)(cj.l >> 1);
-      ci.mid += (long long)(cj.l >> 1);
       fx_mac(cr, cj, gx_re(x5));
       fx_mac(ci, cj, gx_im(x5));
     }
@@ -323,8 +322,8 @@ __device__ __forceinline__ void gx_first(const ProbDev& P, const GEl& g, size_t 
   if (pred) {
     if (frame) {
       s = fx_cmul(fx_coef(p.x), fx_coef(ADJ ? -p.y : p.y), s);
-      s.x <<= 1;
-      s.y <<= 1;
+      s.x <<= 2;
+      s.y <<= 2;
     }
     t.x += s.x;
     t.y += s.y;
@@ -376,7 +375,7 @@ __device__ __forceinline__ Cx gx_ring_sum(const int4* __restrict__ ring, size_t 
       term(kGxW[n][i], ring[(size_t)sl * stride]);
     }
   }
-  return Cx{(xh << 31) + xl, (yh << 31) + yl};
+  return Cx{(long long)((unsigned long long)xh << 32) + xl, (long long)((unsigned long long)yh << 32) + yl};
 }
 
 // Commit of a converged step at one element: q <- 2 z - q and, with the
@@ -396,11 +395,11 @@ __device__ __forceinline__ Cx gx_commit(const ProbDev& P, const GEl& g, size_t o
   Cx c{z.x - w.x - q.x, z.y - w.y - q.y};
   if (frame) {
     p = gx_ld(h.ph + o);
-    if (h.n == 0) p = Cx{1LL << 61, 0};  // a fresh frame
-    c = fx_cmul(fx_coef(p.x), fx_coef(ADJ ? p.y : -p.y), Cx{c.x << 1, c.y << 1});
+    if (h.n == 0) p = Cx{kFxPhase1, 0};  // a fresh frame
+    c = fx_cmul(fx_coef(p.x), fx_coef(ADJ ? p.y : -p.y), Cx{c.x << 2, c.y << 2});
     const longlong2 u = __ldg(P.fxu + g.v);
     const Cx pn = fx_cmul(fx_coef(u.x), fx_coef(u.y), p);
-    p = Cx{pn.x << 1, pn.y << 1};
+    p = Cx{pn.x << 2, pn.y << 2};
     gx_st(h.ph + o, p);
   }
   if (sh) {
@@ -589,7 +588,7 @@ __device__ void gx_first_pass(const ProbDev& P, const GxSmem& S, const double2* 
 // mode 0: forward sweep of the system's states (checkpoints or stage tape if
 // tape); mode 1 (ADJ: 2): steps j0..j1-1 in place on the vectors x
 template <bool ADJ, int QN>
-__global__ void __launch_bounds__(kGridThreads, 2)
+__global__ void __launch_bounds__(kGridThreads, kGxBlocks)
     k_sweep_gx(const ProbDev* __restrict__ pp, const __grid_constant__ GxParams gp, int mode, int tape, int j0, int j1,
                double2* __restrict__ x, int nstates) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -690,39 +689,46 @@ __global__ void __launch_bounds__(kGridThreads, 2)
   }
 }
 
-// Gradient pieces of one step over a block's chunk (eq. reducedgradient), QP
-// subsystems from q0 per pass: per subsystem A = sum Z conj(R), B = sum Z
-// conj(P) of zhat, to P.partials.  Integer sums per thread and state: each
-// product's 62-bit value is added in two halves, so that any number of
-// elements fits; a state's sums become FP64 when the thread leaves it.
+// Gradient pieces of one step over a block's chunk (eq. reducedgradient),
+// kGxQP subsystems from q0 per pass: per subsystem A = sum Z conj(R), B = sum
+// Z conj(P) of zhat, scaled by 2^-kc and both states' scales.  Everything is
+// summed in integers -- each product's value in two halves, so that any number
+// of elements fits, every state's sums brought to the smallest scale eref -- and
+// added over the blocks by 64-bit integer atomics: exact, whatever their order.
+// (Summed in FP64 and over the blocks by block 0, these sums took 55 us of
+// an adjoint step of three states of vec 65536, the elements' products 12.)
 constexpr int kGxQP = 3;
+__device__ __forceinline__ void gx_addsum(long long& hi, long long& lo, long long h, long long l, int s) {
+  if (s) {
+    // (h 2^32 + l) >> s, rounded
+    const __int128 v = (((__int128)h << 32) + l + (((__int128)1 << s) >> 1)) >> s;
+    h = (long long)(v >> 32);
+    l = (long long)((unsigned long long)v & 0xffffffffull);
+  }
+  hi += h;
+  lo += l;
+}
 template <bool PK>
 __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, const GxSmem& S, long long e0,
                                         long long e1, const int4* __restrict__ zh, const double2* __restrict__ tape,
-                                        size_t tslabs, int trow, const int* __restrict__ zsc, int q0) {
+                                        size_t tslabs, int trow, const int* __restrict__ zsc, int eref, int q0,
+                                        unsigned long long* acc) {
   const GridHdr& G = *S.g;
   const int N = G.h.N;
   constexpr int NS = PK ? 2 : 4;  // sums per subsystem
-  long long hi[kGxQP][NS], lo[kGxQP][NS];
-  double tot[kGxQP][4];
+  long long hi[kGxQP][NS], lo[kGxQP][NS], th[kGxQP][NS], tl[kGxQP][NS];
 #pragma unroll
-  for (int u = 0; u < kGxQP; ++u) {
+  for (int u = 0; u < kGxQP; ++u)
 #pragma unroll
-    for (int c = 0; c < NS; ++c) hi[u][c] = lo[u][c] = 0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) tot[u][c] = 0.0;
-  }
+    for (int c = 0; c < NS; ++c) hi[u][c] = lo[u][c] = th[u][c] = tl[u][c] = 0;
   auto leave = [&](int b) {
-    // value = (hi 2^31 + lo) 2^62 / (2^scales 2^-kc)
-    const int e = 62 - zsc[(size_t)b * 2 * G.h.NT] - S.sc[b];
+    const int s = min(zsc[(size_t)b * 2 * G.h.NT] + S.sc[b] - eref, 100);
 #pragma unroll
     for (int u = 0; u < kGxQP; ++u)
-      if (q0 + u < gp.Q) {
 #pragma unroll
-        for (int c = 0; c < NS; ++c) {
-          tot[u][c] += scalbn(fma((double)hi[u][c], 2147483648.0, (double)lo[u][c]), e + P.kc[q0 + u]);
-          hi[u][c] = lo[u][c] = 0;
-        }
+      for (int c = 0; c < NS; ++c) {
+        gx_addsum(th[u][c], tl[u][c], hi[u][c], lo[u][c], s);
+        hi[u][c] = lo[u][c] = 0;
       }
   };
   int bcur = -1;
@@ -736,9 +742,8 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
     const uint32_t kd = __ldg(P.digits + g.k), ld = __ldg(P.digits + g.l);
     const Cx Z = gx_ld(tape + ((size_t)g.b * tslabs + trow) * G.Vh + g.i);
     const Fx zx = fx_split(Z.x), zy = fx_split(Z.y), nzx = fx_split(-Z.x);
-    // 2^30 for rounding and 2^29 for the mean of each left-out low product
     auto add = [&](long long& h, long long& l, Fx a, long long x, Fx b, long long y) {
-      FxAcc s{0, 1LL << 31};
+      FxAcc s = fx_acc();
       fx_mac(s, a, fx_split(x));
       fx_mac(s, b, fx_split(y));
       const Fx v = fx_split(fx_val(s));
@@ -766,24 +771,39 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
   }
   if (bcur >= 0) leave(bcur);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __syncthreads();  // the sums of the pass before are taken
 #pragma unroll
   for (int u = 0; u < kGxQP; ++u)
-    if (q0 + u < gp.Q) {
-      if (PK) {
-        // the g_ad sum is minus the conjugate of the g_a sum
-        tot[u][2] = -tot[u][0];
-        tot[u][3] = tot[u][1];
+#pragma unroll
+    for (int c = 0; c < NS; ++c) {
+      // in limbs of 24, 24 and the rest of the bits: exact in 32-bit warp sums
+      const long long h = th[u][c] + (tl[u][c] >> 32);
+      const unsigned l = (unsigned)tl[u][c];
+      const int r0 = __reduce_add_sync(kFull, (int)(l & 0xffffffu));
+      const int r1 = __reduce_add_sync(kFull, (int)((l >> 24) | (((unsigned)h & 0xffffu) << 8)));
+      const int r2 = __reduce_add_sync(kFull, (int)(h >> 16));
+      if (lane == 0) {
+        // value = sum r0 + r1 2^24 + r2 2^48
+        S.gs[(u * 4 + c) * kGxWarps + warp] = make_longlong2((long long)r0 + ((long long)r1 << 24), r2);
       }
-      const double r = warp_sum4(tot[u][0], tot[u][1], tot[u][2], tot[u][3], lane);
-      if ((lane & 7) == 0) S.dred[(lane >> 3) * kGxWarps + warp] = r;
-      __syncthreads();
-      if (threadIdx.x < 4) {
-        double t = 0.0;
-        for (int w = 0; w < kGxWarps; ++w) t += S.dred[threadIdx.x * kGxWarps + w];
-        P.partials[((size_t)blockIdx.x * LB_MAXQ + q0 + u) * 4 + threadIdx.x] = t;
-      }
-      __syncthreads();
     }
+  __syncthreads();
+  if (threadIdx.x < kGxQP * 4) {
+    const int u = threadIdx.x >> 2, c = threadIdx.x & 3;
+    if (c < NS && q0 + u < gp.Q) {
+      long long a = 0, b = 0;
+      for (int w = 0; w < kGxWarps; ++w) {
+        const longlong2 v = S.gs[(u * 4 + c) * kGxWarps + w];
+        a += v.x;
+        b += v.y;
+      }
+      // 48 bits in the low part: the blocks' low parts add up without overflow
+      b += a >> 48;
+      a &= (1LL << 48) - 1;
+      atomicAdd(acc + ((q0 + u) * 4 + c) * 2, (unsigned long long)a);
+      atomicAdd(acc + ((q0 + u) * 4 + c) * 2 + 1, (unsigned long long)b);
+    }
+  }
 }
 
 // Backward sweep over all states: recompute each checkpoint segment, then the
@@ -792,7 +812,7 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
 // reads zhat's neighbours in the buffer the solve left it in, which the first
 // pass may write: a barrier separates the two.
 template <int QN>
-__global__ void __launch_bounds__(kGridThreads, 2)
+__global__ void __launch_bounds__(kGridThreads, kGxBlocks)
     k_backward_gx(const ProbDev* __restrict__ pp, const __grid_constant__ GxParams gp) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
@@ -802,6 +822,9 @@ __global__ void __launch_bounds__(kGridThreads, 2)
   const int V = H.V;
   const long long e0 = (long long)blockIdx.x * G.chunk, e1 = min(G.total, e0 + G.chunk);
   const long long limit = P.spin_limit > 0 ? P.spin_limit : kSpinLimit;
+  if (blockIdx.x == 0)
+    for (int t = threadIdx.x; t < 3 * LB_MAXQ * 8; t += blockDim.x)
+      reinterpret_cast<unsigned long long*>(P.partials)[t] = 0ull;
   // terminal condition qhat^{N_T} = beta_i/M g_i (Appendix B)
   const int ld = gx_load(P, S, P.lam, [&](const GEl& g) {
     const size_t o = (size_t)g.b * V + g.v;
@@ -837,6 +860,11 @@ __global__ void __launch_bounds__(kGridThreads, 2)
   fhist.cap = P.pred_order;
   const size_t stride = (size_t)G.M * G.Vh;
   int* const asc = S.sc;
+  // the pieces' sums of a step, [3][LB_MAXQ][4][2] by step: added to by every
+  // block, read and cleared by block 0 after the step's barrier
+  unsigned long long* const gacc = reinterpret_cast<unsigned long long*>(P.partials);
+  constexpr int kAcc = LB_MAXQ * 8;
+  unsigned gstep = 0;
   for (int sg = nseg - 1; sg >= 0 && !failed; --sg) {
     const int j0 = H.K > 0 ? sg * H.K : 0, j1 = H.K > 0 ? min(H.NT, j0 + H.K) : H.NT;
     if (H.K > 0) {
@@ -912,17 +940,28 @@ __global__ void __launch_bounds__(kGridThreads, 2)
       it_adj += (unsigned long long)it * G.M;
       st_adj += G.M;
       maxit = max(maxit, it);
-      // S.sc already holds the next step's scales: the pieces use this step's
+      // S.sc already holds the next step's scales: the pieces use this step's;
+      // eref: the smallest sum of both scales
       __syncthreads();
-      for (int b = threadIdx.x; b < G.M; b += blockDim.x) S.sc[b] += S.sh[b];
+      if (threadIdx.x < 32) {
+        int m = INT32_MAX;
+        for (int b = threadIdx.x; b < G.M; b += 32) {
+          S.sc[b] += S.sh[b];
+          m = min(m, fxs[(size_t)b * 2 * H.NT + j] + S.sc[b]);
+        }
+        m = __reduce_min_sync(kFull, m);
+        if (threadIdx.x == 0) S.flag[3] = m;
+      }
       __syncthreads();
+      const int eref = S.flag[3];
+      unsigned long long* const acc = gacc + (gstep % 3) * kAcc;
       const double2* tp = H.K > 0 ? P.seg : P.ckpt;
       const size_t slabs = H.K > 0 ? H.K : H.NT;
       for (int q0 = 0; q0 < H.Q; q0 += kGxQP) {
         if (G.herm)
-          gx_grad<true>(P, gp, S, e0, e1, zh, tp, slabs, j - j0, fxs + j, q0);
+          gx_grad<true>(P, gp, S, e0, e1, zh, tp, slabs, j - j0, fxs + j, eref, q0, acc);
         else
-          gx_grad<false>(P, gp, S, e0, e1, zh, tp, slabs, j - j0, fxs + j, q0);
+          gx_grad<false>(P, gp, S, e0, e1, zh, tp, slabs, j - j0, fxs + j, eref, q0, acc);
       }
       __syncthreads();
       for (int b = threadIdx.x; b < G.M; b += blockDim.x) S.sc[b] -= S.sh[b];
@@ -932,16 +971,27 @@ __global__ void __launch_bounds__(kGridThreads, 2)
         failed = true;
         break;
       }
-      // block 0: fixed-order sum over blocks; multiply by -i: g = (S.im, -S.re)
+      // block 0: the step's sums, multiplied by -i: g = (S.im, -S.re)
+      ++gstep;
       if (blockIdx.x == 0 && threadIdx.x < 4 * H.Q) {
-        const int q = threadIdx.x >> 2, c = threadIdx.x & 3;
-        double t = 0.0;
-        for (int bb = 0; bb < (int)gridDim.x; ++bb) t += __ldcg(P.partials + ((size_t)bb * LB_MAXQ + q) * 4 + c);
+        const int q = threadIdx.x >> 2;
+        int c = threadIdx.x & 3;
+        // Hermitian Z and zhat: the g_ad sum is minus the conjugate of the g_a sum
+        const bool flip = G.herm && c == 2;
+        if (G.herm) c &= 1;
+        long long lo = (long long)__ldcg(acc + (q * 4 + c) * 2), hi = (long long)__ldcg(acc + (q * 4 + c) * 2 + 1);
+        hi += lo >> 48;
+        lo &= (1LL << 48) - 1;
+        double t = scalbn(fma((double)hi, 281474976710656.0, (double)lo), 64 - eref + P.kc[q]);
+        if (flip) t = -t;
         double* gg = reinterpret_cast<double*>(P.gproj + ((size_t)j * H.Q + q) * 2);
-        if (c == 0) gg[1] = -t;
-        if (c == 1) gg[0] = t;
-        if (c == 2) gg[3] = -t;
-        if (c == 3) gg[2] = t;
+        const int d = threadIdx.x & 3;
+        if (d == 0) gg[1] = -t;
+        if (d == 1) gg[0] = t;
+        if (d == 2) gg[3] = -t;
+        if (d == 3) gg[2] = t;
+        __syncwarp(__activemask());
+        if (!G.herm || d < 2) acc[(q * 4 + c) * 2] = acc[(q * 4 + c) * 2 + 1] = 0ull;
       }
       const bool next = j > j0;
       GxHist hn = ahist;
@@ -969,6 +1019,98 @@ __global__ void __launch_bounds__(kGridThreads, 2)
     atomicAdd(&P.status->iters[2], it_adj);
     atomicAdd(&P.status->steps[2], st_adj);
     atomicMax(&P.status->max_iter_seen, maxit);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// y = M x on many elements (lb_apply): the off-diagonal part on the integer pipe.
+// The vectors are split once (k_apply_split, scaled by each one's largest entry)
+// into the sweeps' iterate buffer; the control factors are scaled up by a
+// common 2^ka so that the small sums keep 2^-60 of the largest entry times
+// 2^-ka.  The diagonal and the result are FP64.
+
+// high words of the largest magnitudes of n_vec vectors (slots cleared before)
+__global__ void k_apply_max(const double2* __restrict__ x, int V, unsigned* __restrict__ slots) {
+  const double2* xv = x + (size_t)blockIdx.y * V;
+  unsigned m = 0;
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
+    const double2 a = xv[v];
+    const unsigned long long b = umax64(abs_bits(a.x), abs_bits(a.y));
+    m = max(m, b ? max((unsigned)(b >> 32), 1u) : 0u);
+  }
+  m = __reduce_max_sync(kFull, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(slots + blockIdx.y, m);
+}
+// scale with the largest entry in [2^59, 2^60) from its magnitude's high word
+__device__ __forceinline__ int gx_scale_of(unsigned h) {
+  const int e = (int)(h >> 20);
+  return h ? kFxTop - (e ? e - 1023 : -1022) : kFxTop;
+}
+__global__ void k_apply_split(const double2* __restrict__ x, int V, const unsigned* __restrict__ slots,
+                              int4* __restrict__ z) {
+  const unsigned h = slots[blockIdx.y];
+  if (h >= 0x7ff00000u) return;  // NaN or Inf: k_apply_gx computes this vector in FP64
+  const int sc = gx_scale_of(h);
+  const size_t base = (size_t)blockIdx.y * V;
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
+    const double2 a = x[base + v];
+    z[base + v] = gx_pack(Cx{fx_from_bits(a.x, sc), fx_from_bits(a.y, sc)});
+  }
+}
+template <bool ADJ, int QN>
+__global__ void __launch_bounds__(kGridThreads, 3)
+    k_apply_gx(const ProbDev* __restrict__ pp, const __grid_constant__ GxParams gp, int step,
+               const double2* __restrict__ x, const int4* __restrict__ z, const unsigned* __restrict__ slots,
+               double2* __restrict__ y, int n_vec) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_ka;
+  const ProbDev& P = *pp;
+  const GxSmem S = gx_setup(smem, P, n_vec, 0);
+  const Hdr& H = S.g->h;
+  const int V = H.V, N = H.N;
+  const double2* ct = P.ctab + (size_t)step * H.cq;
+  if (threadIdx.x == 0) {
+    // the largest power of two that keeps every factor below 0.45 (decay: below 2^-ka there)
+    double m = 0.0;
+    for (int q = 0; q < gp.Q; ++q) m = fmax(m, scalbn(fmax(fabs(ct[q].x), fabs(ct[q].y)), P.kc[q]));
+    for (int i = 0; i < P.njcoef; ++i) m = fmax(m, fmax(P.jf[i], P.ja[i]));
+    s_ka = m > 0.0 ? min(20, ilogb(0.45 / m)) : 20;
+  }
+  __syncthreads();
+  const int ka = s_ka;
+  if ((int)threadIdx.x < gp.Q) {
+    const int q = threadIdx.x;
+    const double sg = ADJ ? -1.0 : 1.0;
+    const Fx a = fx_coef(__double2ll_rn(scalbn(sg * ct[q].x, 64 + P.kc[q] + ka)));
+    const Fx b = fx_coef(__double2ll_rn(scalbn(sg * ct[q].y, 64 + P.kc[q] + ka)));
+    S.ctl[q] = make_int4(a.h, a.l, b.h, b.l);
+  }
+  for (int i = threadIdx.x; i < P.njcoef; i += blockDim.x) {
+    S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 64 + ka)));
+    S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 64 + ka)));
+  }
+  __syncthreads();
+  const double inv = 2.0 / H.h;
+  const long long n = (long long)n_vec * V, nt = (long long)gridDim.x * blockDim.x;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += nt) {
+    const int b = (int)(e / V), v = (int)(e - (long long)b * V), k = v % N, l = v / N;
+    const uint32_t kd = __ldg(P.digits + k), ld = __ldg(P.digits + l);
+    const unsigned h = __ldg(slots + b);
+    double cr = 0.0, ci = 0.0;
+    if (h < 0x7ff00000u) {
+      const Cx c = gx_apply<ADJ, false, QN>(z + (size_t)b * V, gp, S, v, k, l, N, kd, ld);
+      const double f = scalbn(inv, -gx_scale_of(h) - ka);
+      cr = f * (double)c.x;
+      ci = f * (double)c.y;
+    } else {
+      const Tabs T{P.cu, P.cd, P.jf, P.ja};
+      offdiag_acc<ADJ>(cr, ci, x + (size_t)b * V, v, kd, ld, H, T, ct);
+      cr *= inv;
+      ci *= inv;
+    }
+    const double2 D = __ldg(P.D + v), xx = x[e];
+    const double di = ADJ ? -D.y : D.y;
+    y[e] = make_double2(fma(D.x, xx.x, -di * xx.y) + cr, fma(D.x, xx.y, di * xx.x) + ci);
   }
 }
 
@@ -1026,7 +1168,39 @@ cudaError_t gx_launch(const void* k, long long elements, size_t smem, void** arg
   return cudaLaunchCooperativeKernel(k, dim3((unsigned)n), dim3(kGridThreads), args, smem, s);
 }
 
+template <bool ADJ>
+void run_apply(int Q, unsigned blocks, size_t smem, cudaStream_t s, const ProbDev* p, const GxParams& gp, int step,
+               const double2* x, const int4* z, const unsigned* slots, double2* y, int n_vec) {
+  switch (Q) {
+    case 4: k_apply_gx<ADJ, 4><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec); break;
+    case 6: k_apply_gx<ADJ, 6><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec); break;
+    default: k_apply_gx<ADJ, 0><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec); break;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h, int adjoint, int64_t step, const double2* x,
+                            double2* y, int n_vec, cudaStream_t s) {
+  const GxParams gp = gx_params(h);
+  unsigned* slots = reinterpret_cast<unsigned*>(h.gslots);
+  int4* z = reinterpret_cast<int4*>(h.zA);
+  cudaError_t e = cudaMemsetAsync(slots, 0, sizeof(unsigned) * n_vec, s);
+  if (e != cudaSuccess) return e;
+  const unsigned bx = (unsigned)((h.V + 8 * 256 - 1) / (8 * 256));
+  k_apply_max<<<dim3(bx, n_vec), 256, 0, s>>>(x, h.V, slots);
+  k_apply_split<<<dim3(bx, n_vec), 256, 0, s>>>(x, h.V, slots, z);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const long long nb = ((long long)n_vec * h.V + kGridThreads - 1) / kGridThreads;
+  const unsigned blocks = (unsigned)(nb < 152 * 12 ? nb : 152 * 12);  // the tables are set up once per block
+  const size_t smem = gx_smem_bytes(h.ncoef, h.njcoef, h.M);
+  if (adjoint)
+    run_apply<true>(h.Q, blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
+  else
+    run_apply<false>(h.Q, blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_sweep_gx(const ProbDev* d_prob, const ProbDev& h, int mode, int tape, int64_t j0, int64_t j1,
                             double2* x, int nstates, cudaStream_t s) {

@@ -130,7 +130,7 @@ struct ProbDev {
   double2* jpart;            // [M][C] the running penalty's sums per chunk
   int4* fxd;                 // [V] grid sweeps: (I - dt/2 D)^-1 - 1, split
   int4* fxh;                 // [V] dt/2 D, split
-  longlong2* fxu;            // [V] the frame's factor per step, half of the unit-modulus part of g
+  longlong2* fxu;            // [V] the frame's factor per step, a quarter of the unit-modulus part of g
   int32_t* gsc;              // [M] the adjoint states' scales during a recompute
   int4* ctabx;               // [NT][cq + 1] the rows of ctab split for them, last the stopping factor and range flag
   int32_t* fxs;              // [M][2 NT] scales of the stage vectors and the checkpoints
@@ -191,7 +191,8 @@ cudaError_t launch_propagate_resident(const ProbDev* d_prob, int adjoint, int64_
                                       int n_vec, const ResidentConfig& rc, cudaStream_t s);
 
 // one-CTA-per-state sweeps in fixed point (lb_fixed.cu)
-constexpr double kFixedRho = 0.25;  // largest iteration-matrix bound rho_j they take
+constexpr int kFxChunkV = 128;      // largest N^2 of the chunked sweep
+constexpr double kFixedRho = 0.24;  // largest iteration-matrix bound rho_j they take
 struct FixedConfig {
   int threads, E, QT;  // CTA size, elements per thread (0: not applicable), units of the register plan (E = 1)
   size_t smem;
@@ -237,6 +238,10 @@ constexpr int kGridFixedStates = 4096;    // most states (their scales are in sh
 cudaError_t launch_sweep_gx(const ProbDev* d_prob, const ProbDev& h_prob, int mode, int tape, int64_t j0, int64_t j1,
                             double2* x, int nstates, cudaStream_t s);
 cudaError_t launch_backward_gx(const ProbDev* d_prob, const ProbDev& h_prob, cudaStream_t s);
+// y = M x with the off-diagonal part in fixed point (n_vec <= M)
+constexpr long long kApplyFixedElements = 1 << 17;  // fewest elements of a call that take it
+cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h_prob, int adjoint, int64_t step, const double2* x,
+                            double2* y, int n_vec, cudaStream_t s);
 
 // cluster-split sweeps for small states: one cluster of C CTAs per state,
 // 2Q lanes per element, or 4Q with the component split (Q <= 4,

@@ -124,8 +124,8 @@ __global__ void k_gate_targets(ProbDev P, const double2* __restrict__ Vg, const 
 __device__ __forceinline__ void put_factor(const ProbDev& P, int j, int u, double2 c) {
   P.ctab[(size_t)j * P.cq + u] = c;
   if (!P.ctabx) return;
-  const Fx a = fx_coef(__double2ll_rn(scalbn(c.x, 62 + P.kc[u])));
-  const Fx b = fx_coef(__double2ll_rn(scalbn(c.y, 62 + P.kc[u])));
+  const Fx a = fx_coef(__double2ll_rn(scalbn(c.x, 64 + P.kc[u])));
+  const Fx b = fx_coef(__double2ll_rn(scalbn(c.y, 64 + P.kc[u])));
   P.ctabx[(size_t)j * (P.cq + 1) + u] = make_int4(a.h, a.l, b.h, b.l);
 }
 
@@ -175,18 +175,18 @@ __global__ void k_stop_factors(const ProbDev* __restrict__ probs) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= P.NT) return;
   double rho = 0.0;
-  bool range = true;  // every factor within the fixed-point sweeps' 1/2
+  bool range = true;  // every factor within the fixed-point sweeps' range
   for (int q = 0; q < P.Q; ++q) {
     const double n = P.levels[q];
     const double2 c = P.ctab[(size_t)j * P.cq + q];
-    if (P.ctabx) range = range && scalbn(fmax(fabs(c.x), fabs(c.y)), P.kc[q]) <= 0.5;
+    if (P.ctabx) range = range && scalbn(fmax(fabs(c.x), fabs(c.y)), P.kc[q]) < 0.49;
     rho += hypot(c.x, c.y) * 2.0 * (sqrt(n - 1.0) + sqrt(n - 2.0)) + P.jump[q] * (n - 1.0);
   }
   // each of the four terms of a Jaynes-Cummings pair couples with at most
   // |dt/2 g| sqrt((n_p - 1)(n_q - 1))
   for (int k = 0; k < P.npair; ++k) {
     const double2 c = P.ctab[(size_t)j * P.cq + P.Q + k];
-    if (P.ctabx) range = range && scalbn(fmax(fabs(c.x), fabs(c.y)), P.kc[P.Q + k]) <= 0.5;
+    if (P.ctabx) range = range && scalbn(fmax(fabs(c.x), fabs(c.y)), P.kc[P.Q + k]) < 0.49;
     rho += 4.0 * hypot(c.x, c.y) * sqrt((P.levels[P.jp[k]] - 1.0) * (P.levels[P.jq[k]] - 1.0));
   }
   // (1 - rho)/rho, capped so that rtol ||q|| times it stays finite
@@ -230,14 +230,15 @@ __global__ void k_gproj_reduce(const ProbDev* __restrict__ probs, int one_slot) 
   }
 }
 
-// dG/dalpha (eq. reducedgradient): one warp per (q, f, s); the sum over the
+// dG/dalpha (eq. reducedgradient): one block per (q, f, s); the sum over the
 // spline's support in time is in a fixed order (the states were summed by
-// k_gproj_reduce).
-__global__ void k_gradient_project(const ProbDev* __restrict__ probs) {
+// k_gproj_reduce).  A thread's steps are a chain of FP64 with a sine and a
+// cosine each: with one warp per spline 10000 steps took 133 us.
+constexpr int kProjThreads = 256;
+__global__ void __launch_bounds__(kProjThreads) k_gradient_project(const ProbDev* __restrict__ probs) {
   const ProbDev& P = probs[blockIdx.y];
-  const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int q = 0, rem = gw;
+  __shared__ double red[2][kProjThreads / 32];
+  int q = 0, rem = blockIdx.x;
   while (q < P.Q && rem >= P.nf[q] * P.Ns) {
     rem -= P.nf[q] * P.Ns;
     ++q;
@@ -250,7 +251,7 @@ __global__ void k_gradient_project(const ProbDev* __restrict__ probs) {
   const int jlo = max(0, (int)floor((s - 2) * dtau / P.h - 1.0));
   const int jhi = min(P.NT - 1, (int)ceil((s + 1) * dtau / P.h));
   double gr = 0.0, gi = 0.0;
-  for (int j = jlo + lane; j <= jhi; j += 32) {
+  for (int j = jlo + (int)threadIdx.x; j <= jhi; j += kProjThreads) {
     const double t = (j + 0.5) * P.h;
     const double S = bspline2(t / dtau - (s - 0.5));
     if (S == 0.0) continue;
@@ -262,9 +263,15 @@ __global__ void k_gradient_project(const ProbDev* __restrict__ probs) {
     gr += S * (cs * ga_r - sn * ga_i + cs * gd_r + sn * gd_i);
     gi += S * (-(cs * ga_i + sn * ga_r) + cs * gd_i - sn * gd_r);
   }
-  gr = warp_sum(gr);
-  gi = warp_sum(gi);
-  if (lane == 0) {
+  const double r = warp_sum2(gr, gi, threadIdx.x & 31);
+  if ((threadIdx.x & 15) == 0) red[(threadIdx.x >> 4) & 1][threadIdx.x >> 5] = r;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    gr = gi = 0.0;
+    for (int w = 0; w < kProjThreads / 32; ++w) {
+      gr += red[0][w];
+      gi += red[1][w];
+    }
     const int k = P.aoff[q] + 2 * (f * P.Ns + s);
     const double sc = P.h * kTwoPi;
     P.grad[k] = sc * gr + P.gamma2 * P.alpha[k];
@@ -377,9 +384,7 @@ cudaError_t launch_finalize(const ProbDev* d_probs, int n_probs, int max_param_w
   k_gproj_reduce<<<dim3(304, n_probs), 256, 0, s>>>(d_probs, one_slot);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int threads = 128;
-  dim3 grid((max_param_warps * 32 + threads - 1) / threads, n_probs);
-  k_gradient_project<<<grid, threads, 0, s>>>(d_probs);
+  k_gradient_project<<<dim3(max_param_warps, n_probs), kProjThreads, 0, s>>>(d_probs);
   return cudaGetLastError();
 }
 

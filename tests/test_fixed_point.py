@@ -50,20 +50,23 @@ def test_products_are_exact_to_two_units(tmp_path):
     r = subprocess.run([nvcc, "-std=c++17", "-O2", "-I", B.CSRC, "-o", exe, str(src)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     rng = random.Random(5)
-    one, top = 1 << 62, 1 << 60
-    cases = [(-one, 0, top, -top), (-one, one // 2, top, top), (0, -one // 2, -top, 1), (1, -1, -1, 0), (0, 0, 0, 0)]
+    one, top = 1 << 64, 1 << 61
+    big = int(0.47 * one)
+    cases = [(-big, 0, top, -top), (big, 0, top, top), (0, -big, -top, 1), (0, big, top, -top), (1, -1, -1, 0),
+             (0, 0, 0, 0), (int(0.33 * one), -int(0.33 * one), top, -top)]
     for _ in range(2000):
+        a = [rng.randrange(-big, big) * 0.7 for _ in range(2)]
         k = rng.randrange(0, 62)
-        cases.append((-rng.randrange(0, one >> k or 1), rng.randrange(-(one // 2) >> k, (one // 2 >> k) + 1),
-                      rng.randrange(-top, top) >> rng.randrange(0, 40), rng.randrange(-top, top)))
+        cases.append((int(a[0]) >> k, int(a[1]) >> k, rng.randrange(-top, top) >> rng.randrange(0, 40),
+                      rng.randrange(-top, top)))
     inp = "\n".join(" ".join(str(v) for v in c) for c in cases)
     out = subprocess.run([exe], input=inp, capture_output=True, text=True, timeout=60).stdout.split("\n")
     low = 0.0
     for (ax, ay, x, y), line in zip(cases, out):
         ah, al, sh, sl, rx, ry, hx, ya, d2, u2 = (int(v) for v in line.split())
-        assert ah * 2**31 + al == ax and -2**30 <= al < 2**30
-        assert sh * 2**31 + sl == x and 0 <= sl < 2**31
-        ex, ey = ax * x - ay * y, ax * y + ay * x  # times 2^62
+        assert ah * 2**32 + al == ax and sh * 2**32 + sl == x
+        assert -2**31 <= min(al, sl) and max(al, sl) < 2**31
+        ex, ey = ax * x - ay * y, ax * y + ay * x  # times 2^64
         assert abs(rx * one - ex) <= 2 * one and abs(ry * one - ey) <= 2 * one
         low += (rx * one - ex) / one
         assert hx == ((abs(x) if x >= 0 else -x - 1) >> 32) and ya == min(abs(y), 2**32 - 1)
