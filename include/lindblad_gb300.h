@@ -123,8 +123,11 @@ typedef struct lb_system_desc {
 } lb_system_desc;
 
 /* Solver statistics of the last lb_forward / lb_gradient / lb_propagate.
- * Phases: 0 = forward sweep, 1 = recompute of checkpoint segments, 2 = adjoint
- * steps (which also evaluate the gradient pieces of eq. reducedgradient). */
+ * Phases: 0 = forward sweep, 1 = stage vectors of the checkpoint segments, 2 =
+ * adjoint steps (which also evaluate the gradient pieces of eq. reducedgradient).
+ * Phase 1 covers every step once.  The FP64 sweeps recompute all of them; the
+ * fixed-point sweeps keep the last segment's from the forward sweep and
+ * count them with the iterations they took there. */
 typedef struct lb_stats {
   int64_t state_steps;      /* state-steps integrated, all phases */
   int64_t inner_iterations; /* fixed-point iterations summed over those state-steps */

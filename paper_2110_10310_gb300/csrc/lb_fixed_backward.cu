@@ -227,8 +227,9 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_backward_fx(const Prob
   unsigned gstep = 0;
   for (int sg = nseg - 1; sg >= 0; --sg) {
     const int j0 = K > 0 ? sg * K : ja, j1 = K > 0 ? min(NT, j0 + K) : jb;
-    if (K > 0) {
-      // recompute the stage vectors of this segment from its checkpoint
+    if (K > 0 && sg < nseg - 1) {
+      // recompute the stage vectors of this segment from its checkpoint (the
+      // last segment's are still there from the forward sweep)
       __syncthreads();
       if (jprev >= 0) fx_grad_store(S, P, P.gproj + (((size_t)i * NT + jprev) * Q) * 2, sprev, gstep - 1);
       jprev = -1;

@@ -35,12 +35,18 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_forward_fx(const ProbD
   const int R = P.pred_restart;
   const bool pred = R >= 0 && P.fxfwd, penal = H.gamma1 != 0.0;
   int* const scz = P.fxs + (size_t)i * 2 * NT;  // scale of each step's stage vector, then of each checkpoint
+  // Stage vectors kept: all of them, or with checkpoints those of the last
+  // segment, which the backward sweep starts with: it recomputes the others only.
+  // phase 1's counters take the kept steps with the iterations they took here.
+  const int jkeep = !tape ? NT : K > 0 ? (NT - 1) / K * K : 0;
   const double* const tar = reinterpret_cast<const double*>(P.tar + base) + st.im;
   double jpen = 0.0, psum = 0.0;
   FxCount cnt;
   int cur = 0;
+  unsigned itkeep = 0;  // iterations before step jkeep
   fx_ctl(S, P, H.cq, ja, 0);
   for (int j = ja; j < jb; ++j) {
+    if (j == jkeep) itkeep = (unsigned)stats.iters[0];
     if (penal) {
       const double pj = P.pen[j];
       psum += pj;
@@ -71,7 +77,10 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_forward_fx(const ProbD
     }
     stats.add(0, it);
     if (pred) fx_commit<E, QT, false>(st, S, c);
-    long long* tp = (tape && K == 0) ? reinterpret_cast<long long*>(P.ckpt + ((size_t)i * NT + j) * V) : nullptr;
+    long long* tp = nullptr;
+    if (j >= jkeep)
+      tp = reinterpret_cast<long long*>(K > 0 ? P.seg + ((size_t)i * K + (j - jkeep)) * V
+                                              : P.ckpt + ((size_t)i * NT + j) * V);
     if (tp && threadIdx.x == 0) scz[j] = st.sc;
     fx_update(st, S, cur ? S.zb1 : S.zb0, z, tp);
     fx_rescale(st, S, qtop, pred);
@@ -83,6 +92,10 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_forward_fx(const ProbD
   if (jb < NT) {
     stats.flush(P.status);
     return;
+  }
+  if (K > 0 && tape) {
+    stats.iters[1] = (unsigned)stats.iters[0] - itkeep;
+    stats.steps[1] = NT - jkeep;
   }
   // final state and merit functional (Sec. III)
   double acc = 0.0;

@@ -236,3 +236,22 @@ def test_grid_sweep_matches_the_oracle(L, levels, n_states, herm, K, objective):
         a = s.propagate(x, 3, 17, adjoint=adj).cpu().numpy()
         b = r.propagate(x, 3, 17, adjoint=adj).cpu().numpy()
         assert _rel(a, b) < 1e-13
+
+
+# The last checkpoint segment's stage vectors come from the forward sweep: the
+# gradient is bitwise the full tape's with the same predictor restarts, whether
+# the last segment is the only one, full, or a single step.
+@gpu
+@pytest.mark.parametrize("levels,sweep", [((2, 2), "resident"), ((3, 2, 3), "resident"), ((7, 4), "resident"),
+                                          ((3, 3), "grid")])
+@pytest.mark.parametrize("K", [1, 8, 11, 23, 24, 60])
+def test_last_segment_kept_by_the_forward_sweep(L, levels, sweep, K):
+    p = _problem(levels, 24, True, 0, n_states=2)
+    sw = {"resident": L.LB_SWEEP_RESIDENT, "grid": L.LB_SWEEP_GRID}[sweep]
+    G0, g0 = _sys(p, ckpt_every=0, predictor=K, sweep=sw).gradient()
+    s = _sys(p, ckpt_every=K, sweep=sw)
+    for _ in range(2):
+        G, g = s.gradient()
+        assert G == G0 and np.array_equal(g, g0)
+        st = s.stats()
+        assert st["phase_steps"][1] == st["phase_steps"][0] and st["phase_iterations"][1] == st["phase_iterations"][0]
