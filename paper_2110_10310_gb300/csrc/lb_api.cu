@@ -344,7 +344,7 @@ bool fixed_possible(const lb_system* s) {
 // took one cluster each: with the full stage tape, at least kChunkMinSteps
 // steps, and N^2 <= 128, where N (N + 1) / 2 columns per chunk cost less than the idle
 // SMs.  A chunk starts its predictor cold, so a step takes more iterations
-// there: max_iter must leave room for a cold start at rho = 1/4.
+// there: max_iter must leave room for a cold start at rho = 0.24.
 constexpr int kChunkMinSteps = 64, kChunkMinIter = 64;
 bool chunks_possible(const lb_system* s) {
   return !use_grid(s) && s->V <= lbk::kFxChunkV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&

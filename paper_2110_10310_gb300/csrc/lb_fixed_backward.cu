@@ -138,7 +138,7 @@ __device__ __forceinline__ void fx_grad_store(const FxSmem& S, const ProbDev& P,
 // table and the frame, in the slots of the ring this predictor does not use.
 // They would otherwise stay in registers through the recompute's loop.
 template <int E, int QT, bool PUT>
-__device__ void fx_aside(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, size_t base) {
+__device__ __forceinline__ void fx_aside(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, size_t base) {
   const Hdr& H = *S.hdr;
   const size_t stride = 2 * (size_t)P.M * P.V;
   auto mv = [&](long long& x, long long* p) {
@@ -161,9 +161,9 @@ __device__ void fx_aside(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, 
   }
 }
 
-template <int E, int QT>
-__global__ void __launch_bounds__(fx_max_threads<QT>()) k_backward_fx(const ProbDev* __restrict__ probs,
-                                                                      const WorkItem* __restrict__ items, int mode) {
+template <int E, int QT, int T>
+__global__ void __launch_bounds__(T)
+    k_backward_fx(const ProbDev* __restrict__ probs, const WorkItem* __restrict__ items, int mode) {
   extern __shared__ __align__(16) unsigned char smem[];
   // items == null: one CTA per (chunk, state) of the first problem (full
   // stage tape); mode 1: no gradient, only the chunk's adjoint state that its
@@ -365,11 +365,11 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_backward_fx(const Prob
 
 }  // namespace
 
-template <int E, int QT>
+template <int E, int QT, int T = fx_max_threads<QT>()>
 static cudaError_t run(const FixedConfig& fc, int n, cudaStream_t s, const ProbDev* p, const WorkItem* it, int mode = 0) {
-  cudaError_t e = cudaFuncSetAttribute(k_backward_fx<E, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fc.smem);
+  cudaError_t e = cudaFuncSetAttribute(k_backward_fx<E, QT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fc.smem);
   if (e != cudaSuccess) return e;
-  k_backward_fx<E, QT><<<n, fc.threads, fc.smem, s>>>(p, it, mode);
+  k_backward_fx<E, QT, T><<<n, fc.threads, fc.smem, s>>>(p, it, mode);
   return cudaGetLastError();
 }
 
@@ -392,7 +392,9 @@ cudaError_t launch_backward_fixed(const ProbDev* d_probs, const WorkItem* d_item
     default: break;
   }
   switch (fc.E) {
-    case 1: return run<1, 0>(fc, n_items, s, d_probs, d_items);
+    case 1:
+      return fc.threads <= kFxTabFew ? run<1, 0, kFxTabFew>(fc, n_items, s, d_probs, d_items)
+                                     : run<1, 0>(fc, n_items, s, d_probs, d_items);
     case 2: return run<2, 0>(fc, n_items, s, d_probs, d_items);
     case 3: return run<3, 0>(fc, n_items, s, d_probs, d_items);
     case 5: return run<5, 0>(fc, n_items, s, d_probs, d_items);

@@ -6,9 +6,9 @@ namespace lbk {
 
 namespace {
 
-template <int E, int QT>
-__global__ void __launch_bounds__(fx_max_threads<QT>()) k_forward_fx(const ProbDev* __restrict__ probs,
-                                                                     const WorkItem* __restrict__ items, int tape) {
+template <int E, int QT, int T>
+__global__ void __launch_bounds__(T)
+    k_forward_fx(const ProbDev* __restrict__ probs, const WorkItem* __restrict__ items, int tape) {
   extern __shared__ __align__(16) unsigned char smem[];
   // items == null: one CTA per (chunk, state) of the first problem
   const bool chunked = QT > 0 && items == nullptr;
@@ -120,11 +120,11 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_forward_fx(const ProbD
 
 }  // namespace
 
-template <int E, int QT>
+template <int E, int QT, int T = fx_max_threads<QT>()>
 static cudaError_t run(const FixedConfig& fc, int n, cudaStream_t s, const ProbDev* p, const WorkItem* it, int tape) {
-  cudaError_t e = cudaFuncSetAttribute(k_forward_fx<E, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fc.smem);
+  cudaError_t e = cudaFuncSetAttribute(k_forward_fx<E, QT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fc.smem);
   if (e != cudaSuccess) return e;
-  k_forward_fx<E, QT><<<n, fc.threads, fc.smem, s>>>(p, it, tape);
+  k_forward_fx<E, QT, T><<<n, fc.threads, fc.smem, s>>>(p, it, tape);
   return cudaGetLastError();
 }
 
@@ -169,7 +169,9 @@ cudaError_t launch_forward_fixed(const ProbDev* d_probs, const WorkItem* d_items
     default: break;
   }
   switch (fc.E) {
-    case 1: return run<1, 0>(fc, n_items, s, d_probs, d_items, tape);
+    case 1:
+      return fc.threads <= kFxTabFew ? run<1, 0, kFxTabFew>(fc, n_items, s, d_probs, d_items, tape)
+                                     : run<1, 0>(fc, n_items, s, d_probs, d_items, tape);
     case 2: return run<2, 0>(fc, n_items, s, d_probs, d_items, tape);
     case 3: return run<3, 0>(fc, n_items, s, d_probs, d_items, tape);
     case 5: return run<5, 0>(fc, n_items, s, d_probs, d_items, tape);

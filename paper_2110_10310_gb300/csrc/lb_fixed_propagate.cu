@@ -6,9 +6,9 @@ namespace lbk {
 
 namespace {
 
-template <int E, int QT, bool ADJ>
-__global__ void __launch_bounds__(fx_max_threads<QT>()) k_propagate_fx(const ProbDev* __restrict__ pp, int j0, int j1,
-                                                                       double2* __restrict__ x) {
+template <int E, int QT, int T, bool ADJ>
+__global__ void __launch_bounds__(T)
+    k_propagate_fx(const ProbDev* __restrict__ pp, int j0, int j1, double2* __restrict__ x) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
   const FxSmem S = fx_carve(smem, P, E * (blockDim.x / 2), QT);
@@ -56,10 +56,10 @@ __global__ void __launch_bounds__(fx_max_threads<QT>()) k_propagate_fx(const Pro
 
 }  // namespace
 
-template <int E, int QT>
+template <int E, int QT, int T = fx_max_threads<QT>()>
 static cudaError_t run(const FixedConfig& fc, int n, cudaStream_t s, const ProbDev* p, int adj, int j0, int j1,
                        double2* x) {
-  auto k = adj ? k_propagate_fx<E, QT, true> : k_propagate_fx<E, QT, false>;
+  auto k = adj ? k_propagate_fx<E, QT, T, true> : k_propagate_fx<E, QT, T, false>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fc.smem);
   if (e != cudaSuccess) return e;
   k<<<n, fc.threads, fc.smem, s>>>(p, j0, j1, x);
@@ -76,7 +76,9 @@ cudaError_t launch_propagate_fixed(const ProbDev* d_prob, int adjoint, int64_t j
     default: break;
   }
   switch (fc.E) {
-    case 1: return run<1, 0>(fc, n_vec, s, d_prob, adjoint, a, b, x);
+    case 1:
+      return fc.threads <= kFxTabFew ? run<1, 0, kFxTabFew>(fc, n_vec, s, d_prob, adjoint, a, b, x)
+                                     : run<1, 0>(fc, n_vec, s, d_prob, adjoint, a, b, x);
     case 2: return run<2, 0>(fc, n_vec, s, d_prob, adjoint, a, b, x);
     case 3: return run<3, 0>(fc, n_vec, s, d_prob, adjoint, a, b, x);
     case 5: return run<5, 0>(fc, n_vec, s, d_prob, adjoint, a, b, x);

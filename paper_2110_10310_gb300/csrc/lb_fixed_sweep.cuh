@@ -4,7 +4,7 @@
 // their forward, backward and propagation kernels share.
 //
 // The Jacobi sweeps of small and medium states (N^2 <= 4096) with every step's
-// iteration matrix bounded by 1/4 (lb_api.cu decides; larger controls, the
+// iteration matrix bounded by kFixedRho (lb_api.cu decides; larger controls, the
 // Neumann iteration and GMRES keep the FP64 sweeps).  One CTA owns a state,
 // its iterate in shared memory as split 64-bit integers, and runs the whole
 // time loop; a step whose predicted first iterate is within the tolerance
@@ -38,6 +38,11 @@ namespace {
 
 constexpr int kFxPlanThreads = 512;  // largest CTA of the register plan (128 registers per thread)
 constexpr int kFxTabThreads = 1024;  // ... of the table path (64 registers)
+// ... of its smaller CTAs with one element per lane pair: 80 registers and next
+// to no spills (300 elements, 9 states: forward 4.33 us per step against 4.70
+// in 64 registers).  More elements in one pair instead of more threads
+// is slower (406 elements, 28 states: 11.8 us with two in 416 threads, 8.3 in 832).
+constexpr int kFxTabFew = 768;
 constexpr int kFxWarps = 32;
 constexpr int kFxOrder = 8;          // highest extrapolation order of the register difference table
 template <int QT>
@@ -83,6 +88,10 @@ struct FxSmem {
   int4* dsm;        // [nel] (I - dt/2 D)^-1 - 1 (QT == 0)
   Fx* zb0;          // [V][2] iterate, split, component by component
   Fx* zb1;
+  unsigned char* base;
+  __device__ __forceinline__ int off(const void* p) const {
+    return (int)(reinterpret_cast<const unsigned char*>(p) - base);
+  }
 };
 
 __host__ __device__ inline size_t fx_smem_bytes(int ncoef, int njcoef, int N, int V, int Q, int cq, int nel, int QT) {
@@ -102,8 +111,9 @@ __host__ __device__ inline size_t fx_smem_bytes(int ncoef, int njcoef, int N, in
   return b;
 }
 
-__device__ FxSmem fx_carve(unsigned char* base, const ProbDev& P, int nel, int QT) {
+__device__ __forceinline__ FxSmem fx_carve(unsigned char* base, const ProbDev& P, int nel, int QT) {
   FxSmem S;
+  S.base = base;
   size_t o = 0;
   auto take = [&](size_t bytes) {
     unsigned char* p = base + o;
@@ -134,7 +144,7 @@ __device__ FxSmem fx_carve(unsigned char* base, const ProbDev& P, int nel, int Q
 __device__ __forceinline__ long long fx_from(double x, int sc) { return __double2ll_rn(scalbn(x, sc)); }
 __device__ __forceinline__ double fx_to(long long X, int sc) { return scalbn((double)X, -sc); }
 __device__ __forceinline__ long long fx_other(long long x) { return __shfl_xor_sync(kFull, x, 1); }
-__device__ void fx_setup(const FxSmem& S, const ProbDev& P, int herm) {
+__device__ __forceinline__ void fx_setup(const FxSmem& S, const ProbDev& P, int herm) {
   if (threadIdx.x == 0) {
     load_hdr(*S.hdr, P);
     S.hdr->herm = herm;
@@ -185,7 +195,7 @@ __device__ __forceinline__ unsigned fx_slots_max(const unsigned* w, int nwarps) 
 }
 
 // CTA maximum of a double's magnitude bits
-__device__ unsigned long long fx_cta_max(const FxSmem& S, unsigned long long m) {
+__device__ __forceinline__ unsigned long long fx_cta_max(const FxSmem& S, unsigned long long m) {
   unsigned long long* w = S.mx;
   m = warp_max_u64(m);
   if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = m;
@@ -224,7 +234,7 @@ template <>
 struct FxPlan<0> {};
 
 template <int QT>
-__device__ void fx_plan(FxPlan<QT>& pl, const FxSmem& S, const ProbDev& P, int v) {
+__device__ __forceinline__ void fx_plan(FxPlan<QT>& pl, const FxSmem& S, const ProbDev& P, int v) {
   const Hdr& H = *S.hdr;
   const bool ok = v < H.V;
   const Fx zero{0, 0};
@@ -349,32 +359,36 @@ __device__ __forceinline__ FxPR fx_pr_tab(const Fx* __restrict__ z, int4 ck, int
   return fx_pr(z[2 * s], z[-2 * sN], z[-2 * s], z[2 * sN], Fx{ck.x, ck.y}, Fx{cl.x, cl.y}, Fx{ck.z, ck.w},
                Fx{cl.z, cl.w});
 }
-// (not inlined: the element loops call it once per element; everything it
-// needs comes in registers)
+// (not inlined: the element loops call it once per element.  Everything it
+// needs comes in registers, shared memory as offsets from its start: of a
+// pointer the callee could not tell that it is shared memory.)
 template <bool ADJ>
-__device__ __noinline__ Cx fx_apply_tab(const Fx* __restrict__ z, const FxSub* __restrict__ sub,
-                                        const int4* __restrict__ ck, const int4* __restrict__ cl,
-                                        const Fx* __restrict__ cj, const int4* __restrict__ ctl, int QN, uint32_t kd,
+__device__ __noinline__ Cx fx_apply_tab(int zo, int subo, int cko, int clo, int cjo, int ctlo, int QN, uint32_t kd,
                                         uint32_t ld) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Fx* const z = reinterpret_cast<const Fx*>(smem + zo);
   // QN: Q | N << 8 | bits of a digit << 24
   const int Q = QN & 0xff, N = (QN >> 8) & 0xffff, dm = (1 << (QN >> 24)) - 1;
   Cx r{0, 0};
 #pragma unroll 1
   for (int q = 0; q < Q; ++q) {
-    const FxSub b = sub[q];
+    const FxSub b = *reinterpret_cast<const FxSub*>(smem + subo + q * sizeof(FxSub));
     const int sh = (b.n_sh >> 8) & 0xff, s = b.s, sN = s * N;
     const int nk = (kd >> sh) & dm, nl = (ld >> sh) & dm;
-    const FxPR p = fx_pr_tab(z, ck[b.co + nk], cl[b.co + nl], s, sN);
+    const int4 ck = *reinterpret_cast<const int4*>(smem + cko + (b.co + nk) * sizeof(int4));
+    const int4 cl = *reinterpret_cast<const int4*>(smem + clo + (b.co + nl) * sizeof(int4));
+    const int4 t = *reinterpret_cast<const int4*>(smem + ctlo + q * sizeof(int4));
+    const FxPR p = fx_pr_tab(z, ck, cl, s, sN);
     const bool dec = b.n_sh >> 16;
     Fx c5{0, 0}, x5{0, 0};
     if (dec) {
-      c5 = cj[b.jo + nk * (b.n_sh & 0xff) + nl];
+      c5 = *reinterpret_cast<const Fx*>(smem + cjo + (b.jo + nk * (b.n_sh & 0xff) + nl) * sizeof(Fx));
       x5 = z[ADJ ? -2 * (s + sN) : 2 * (s + sN)];
     }
     if (ADJ)
-      fx_unit_adj(r.x, r.y, p, ctl[q], dec, c5, x5);
+      fx_unit_adj(r.x, r.y, p, t, dec, c5, x5);
     else
-      fx_unit(r.x, r.y, p, ctl[q], dec, c5, x5);
+      fx_unit(r.x, r.y, p, t, dec, c5, x5);
   }
   return r;
 }
@@ -471,7 +485,7 @@ __device__ __forceinline__ void fx_put_d(double2* a, int v, int m, bool im, long
 }
 
 template <int E, int QT>
-__device__ void fx_init(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P) {
+__device__ __forceinline__ void fx_init(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P) {
   const Hdr& H = *S.hdr;
   const double hh = 0.5 * H.h;
   st.cap = QT > 0 ? min(P.pred_order, kFxOrder) : P.pred_order;
@@ -506,7 +520,7 @@ __device__ void fx_init(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P) {
 }
 // the predictor's ring of this launch (QT == 0) in `ring`, `ph`, `fu` of the workspace
 template <int E, int QT>
-__device__ void fx_ring(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, double2* ring, double2* ph, double2* fu,
+__device__ __forceinline__ void fx_ring(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, double2* ring, double2* ph, double2* fu,
                         size_t base) {
   if constexpr (QT == 0) {
     st.pr.ring = reinterpret_cast<long long*>(ring + base);
@@ -526,7 +540,7 @@ __device__ void fx_ring(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, d
 // Load this state's elements from FP64 values, setting the scale; returns
 // false on NaN or Inf.
 template <int E, int QT, class F>
-__device__ bool fx_load(FxState<E, QT>& st, const FxSmem& S, F&& val) {
+__device__ __forceinline__ bool fx_load(FxState<E, QT>& st, const FxSmem& S, F&& val) {
   const Hdr& H = *S.hdr;
   unsigned long long mx = 0;
 #pragma unroll
@@ -554,7 +568,7 @@ __device__ bool fx_load(FxState<E, QT>& st, const FxSmem& S, F&& val) {
 
 // Load this state's elements from a chunk boundary (fixed point, with its scale).
 template <int E, int QT>
-__device__ void fx_load_fixed(FxState<E, QT>& st, const FxSmem& S, const longlong2* x, int sc) {
+__device__ __forceinline__ void fx_load_fixed(FxState<E, QT>& st, const FxSmem& S, const longlong2* x, int sc) {
   const Hdr& H = *S.hdr;
   st.sc = sc;
 #pragma unroll
@@ -616,7 +630,7 @@ __device__ __noinline__ long long fx_ring_sum(const long long* __restrict__ ring
 // in, so that threads may still read that z until the next barrier.
 // jnext: the step after this one (< 0: none), whose control row is fetched.
 template <int E, int QT, bool ADJ>
-__device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, int jnext, bool pred, FxCount& cnt,
+__device__ __forceinline__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, int jnext, bool pred, FxCount& cnt,
                         int& cur, unsigned& qtop, long long& zr, long long& cr) {
   const Hdr& H = *S.hdr;
   const int V = H.V, cq = H.cq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -685,6 +699,7 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
   for (int it = 0; it < maxit; ++it) {
     const Fx* __restrict__ zc = cur ? S.zb1 : S.zb0;
     Fx* __restrict__ zn = cur ? S.zb0 : S.zb1;
+    const int zo = S.off(zc), ctlo = S.off(ctl);
     unsigned* ds = S.slots + 64 * (it & 1) + 32;
     unsigned dm = 0;
     if constexpr (QT > 0) {
@@ -709,7 +724,8 @@ __device__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, const ProbDev& P, i
         int4 d = make_int4(0, 0, 0, 0);
         Cx p{0, 0};
         if (ok) {
-          r = fx_apply_tab<ADJ>(zc + 2 * v + im, S.sub, S.ck, S.cl, ADJ ? S.ja : S.jf, ctl, qn, st.kd[e], st.ld[e]);
+          r = fx_apply_tab<ADJ>(zo + (2 * v + im) * (int)sizeof(Fx), S.off(S.sub), S.off(S.ck), S.off(S.cl),
+                                S.off(ADJ ? S.ja : S.jf), ctlo, qn, st.kd[e], st.ld[e]);
           d = S.dsm[fx_u<E, QT>(e)];
           if (pred && st.frame) p = st.pr.ph[v];
         }
@@ -795,7 +811,7 @@ __device__ __forceinline__ void fx_commit(FxState<E, QT>& st, const FxSmem& S, l
 
 // scale the state (and its predictor) by 2^-s
 template <int E, int QT>
-__device__ void fx_scale_by(FxState<E, QT>& st, const FxSmem& S, int s, bool pred) {
+__device__ __forceinline__ void fx_scale_by(FxState<E, QT>& st, const FxSmem& S, int s, bool pred) {
   const Hdr& H = *S.hdr;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -835,7 +851,7 @@ __device__ __forceinline__ void fx_rescale(FxState<E, QT>& st, const FxSmem& S, 
 // q += src (FP64, each lane's component): the scale follows the sum's largest
 // entry first, which a source may raise by any factor in one step (all threads)
 template <int E, int QT>
-__device__ void fx_add_source(FxState<E, QT>& st, const FxSmem& S, const double (&src)[E], bool pred) {
+__device__ __forceinline__ void fx_add_source(FxState<E, QT>& st, const FxSmem& S, const double (&src)[E], bool pred) {
   unsigned long long mx = 0;
 #pragma unroll
   for (int e = 0; e < E; ++e) mx = umax64(mx, abs_bits(fx_to(st.q[e], st.sc) + src[e]));
@@ -865,7 +881,7 @@ __device__ __forceinline__ void fx_update(FxState<E, QT>& st, const FxSmem& S, c
 }
 
 // deterministic CTA sum of one double per thread, to every thread
-__device__ double fx_cta_sum(const FxSmem& S, double x) {
+__device__ __forceinline__ double fx_cta_sum(const FxSmem& S, double x) {
   double* w = reinterpret_cast<double*>(S.mx);
   x = warp_sum(x);
   if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = x;

@@ -16,6 +16,8 @@
 // correction is not stored by the iteration: c = (I - dt/2 D) z - q recovers it
 // to the rounding of z.
 
+#include <algorithm>
+
 #include "lb_grid.cuh"
 #include "lb_fixed.cuh"
 
@@ -25,6 +27,7 @@ namespace {
 
 constexpr int kGxWarps = kGridThreads / 32;
 constexpr int kGxBlocks = 2;  // blocks per SM
+constexpr int kApplyBlocks = 3;  // ... of the product alone, and of its launch (12 per SM: their table set-ups took 3%)
 
 // kernel parameter: what the element loops need of the system, in the
 // constant bank (the subsystem loop is unrolled for QN > 0)
@@ -1076,7 +1079,7 @@ __global__ void k_apply_split(const double2* __restrict__ x, int V, const unsign
   }
 }
 template <bool ADJ, int QN>
-__global__ void __launch_bounds__(kGridThreads, 3)
+__global__ void __launch_bounds__(kGridThreads, kApplyBlocks)
     k_apply_gx(const ProbDev* __restrict__ pp, const __grid_constant__ GxParams gp, int step,
                const double2* __restrict__ x, const int4* __restrict__ z, const unsigned* __restrict__ slots,
                double2* __restrict__ y, int n_vec) {
@@ -1109,9 +1112,11 @@ __global__ void __launch_bounds__(kGridThreads, 3)
   }
   __syncthreads();
   const double inv = 2.0 / H.h;
-  const long long n = (long long)n_vec * V, nt = (long long)gridDim.x * blockDim.x;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += nt) {
-    const int b = (int)(e / V), v = (int)(e - (long long)b * V), k = v % N, l = v / N;
+  const long long n = (long long)n_vec * V;
+  const int nt = gridDim.x * blockDim.x;
+  for (GIter it_(*S.g, (long long)blockIdx.x * blockDim.x + threadIdx.x); it_.e < n; it_.next(*S.g, nt)) {
+    const long long e = it_.e;
+    const int b = it_.b, v = it_.i, l = (int)((unsigned)v / (unsigned)N), k = v - l * N;
     const uint32_t kd = __ldg(P.digits + k), ld = __ldg(P.digits + l);
     const unsigned h = __ldg(slots + b);
     double cr = 0.0, ci = 0.0;
@@ -1211,7 +1216,12 @@ cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h, int adjoint
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const long long nb = ((long long)n_vec * h.V + kGridThreads - 1) / kGridThreads;
-  const unsigned blocks = (unsigned)(nb < 152 * 12 ? nb : 152 * 12);  // the tables are set up once per block
+  // the blocks the device holds at once: the tables are set up once per block
+  int dev = 0, nsm = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const unsigned blocks = (unsigned)std::min<long long>(nb, (long long)nsm * kApplyBlocks);
   const size_t smem = gx_smem_bytes(h.ncoef, h.njcoef, h.M);
   if (adjoint)
     run_apply<true>(h.Q, blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
