@@ -51,11 +51,13 @@ struct GxSmem {
   int* flag;      // [0] decision, [1] stopping factor (float bits)
   int* sc;        // [M] scale of each state
   int* sh;        // [M] the commit's change of it
+  unsigned long long* due;  // arrivals that end the last barrier
+  int* passed;              // ... and whether it did
 };
 
 __host__ __device__ inline size_t gx_smem_bytes(int ncoef, int njcoef, int M) {
   return align16(sizeof(GridHdr)) + sizeof(int4) * ncoef + 2 * align16(sizeof(Fx) * njcoef) + sizeof(int4) * LB_MAXQ +
-         align16(sizeof(unsigned) * 4 * kGxWarps) + sizeof(longlong2) * 12 * kGxWarps + 16 + 2 * align16(sizeof(int) * M);
+         align16(sizeof(unsigned) * 4 * kGxWarps) + sizeof(longlong2) * 12 * kGxWarps + 32 + 2 * align16(sizeof(int) * M);
 }
 
 __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, int herm) {
@@ -74,9 +76,12 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
   S.red = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * 4 * kGxWarps));
   S.gs = reinterpret_cast<longlong2*>(take(sizeof(longlong2) * 12 * kGxWarps));
   S.flag = reinterpret_cast<int*>(take(16));
+  S.due = reinterpret_cast<unsigned long long*>(take(16));
+  S.passed = reinterpret_cast<int*>(S.due + 1);
   S.sc = reinterpret_cast<int*>(take(sizeof(int) * P.M));
   S.sh = reinterpret_cast<int*>(take(sizeof(int) * P.M));
   if (threadIdx.x == 0) {
+    *S.due = 0;
     load_hdr(S.g->h, P);
     S.g->M = nstates;
     S.g->herm = herm;
@@ -99,6 +104,35 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
   for (int i = threadIdx.x; i < P.M; i += blockDim.x) S.sc[i] = S.sh[i] = 0;
   __syncthreads();
   return S;
+}
+
+// Grid barrier with a bounded wait, as grid_sync (lb_grid.cuh) in fewer round
+// trips to L2: one counter that only grows (zeroed before the launch), so an
+// arrival is one atomic whose value already ends the wait of the last block,
+// and a poll is one load with nothing between two of them.  (grid_sync reads the
+// generation, resets the count, reads the error word beside every poll and
+// sleeps: one state of 3240 elements, 1000 steps forward and back, 36.0 ms with it,
+// 30.5 with this one; three states of vec 65536, 400 steps, 35.3 and 31.0 ms.)
+// The top bit is set by a wait that gave up; the counter is short of the
+// barrier's arrivals then, so no block that looks later passes it.
+constexpr unsigned long long kGxGaveUp = 1ull << 63;
+__device__ __forceinline__ bool gx_sync(const GxSmem& S, GridBar* bar, long long limit) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned long long due = *S.due + gridDim.x;
+    *S.due = due;
+    __threadfence();
+    unsigned long long v = atomicAdd(&bar->arrived, 1ull) + 1;
+    long long spins = 0;
+    while (v < due) {
+      if (++spins > limit) v = atomicOr(&bar->arrived, kGxGaveUp) | kGxGaveUp;
+      else v = *(volatile unsigned long long*)&bar->arrived;
+    }
+    __threadfence();
+    *S.passed = v < kGxGaveUp;
+  }
+  __syncthreads();
+  return *S.passed != 0;
 }
 
 __device__ __forceinline__ int4 gx_pack(Cx z) {
@@ -455,7 +489,7 @@ __device__ int gx_solve(const ProbDev& P, const GxParams& gp, const GxSmem& S, c
   unsigned* qbank = qslots + (solve & 1) * M;
   const long long limit = P.spin_limit > 0 ? P.spin_limit : kSpinLimit;
   gx_ctl<ADJ>(S, P, G.h.Q, G.h.cq, j);
-  if (!grid_sync(P.bar, gridDim.x, limit)) return -3;
+  if (!gx_sync(S, P.bar, limit)) return -3;
   if (S.flag[2]) return -1;
   // the previous solve's |q| bank is free again: clear it for the next solve
   if (blockIdx.x == 0)
@@ -469,7 +503,7 @@ __device__ int gx_solve(const ProbDev& P, const GxParams& gp, const GxSmem& S, c
       gx_pass<ADJ, true, QN>(P, gp, S, e0, e1, rhs, zc, zn, bank);
     else
       gx_pass<ADJ, false, QN>(P, gp, S, e0, e1, rhs, zc, zn, bank);
-    if (!grid_sync(P.bar, gridDim.x, limit)) return -3;
+    if (!gx_sync(S, P.bar, limit)) return -3;
     // bank of iteration it_global + 2 is no longer read by anyone: clear it
     if (blockIdx.x == 0)
       for (int b = threadIdx.x; b < M; b += blockDim.x) slots[((it_global + 2) % 3) * M + b] = 0;
@@ -530,7 +564,7 @@ __device__ int gx_load(const ProbDev& P, const GxSmem& S, double2* q, F&& val) {
     sm.add(g.b, m ? max((unsigned)(m >> 32), 1u) : 0u, slots);
   }
   sm.push(slots, S.red);
-  if (!grid_sync(P.bar, gridDim.x, limit)) return -3;
+  if (!gx_sync(S, P.bar, limit)) return -3;
   bool bad = false;
   if (threadIdx.x < 32) {
     for (int b = threadIdx.x; b < M; b += 32) {
@@ -545,7 +579,7 @@ __device__ int gx_load(const ProbDev& P, const GxSmem& S, double2* q, F&& val) {
   __syncthreads();
   bad = S.flag[0] != 0;
   // every block has read the slots before block 0 clears them for the next load
-  if (!grid_sync(P.bar, gridDim.x, limit)) return -3;
+  if (!gx_sync(S, P.bar, limit)) return -3;
   if (blockIdx.x == 0)
     for (int b = threadIdx.x; b < M; b += blockDim.x) slots[b] = 0;
   if (bad) return 0;
@@ -558,7 +592,8 @@ __device__ int gx_load(const ProbDev& P, const GxSmem& S, double2* q, F&& val) {
 }
 
 __device__ void gx_fail(const ProbDev& P, int code, int step) {
-  if (threadIdx.x == 0 && blockIdx.x == 0)
+  // a wait may give up in one block while the others pass the launch's last barrier
+  if (threadIdx.x == 0 && (blockIdx.x == 0 || code == -3))
     record_error(P.status, code == -3 ? LB_ECUDA : (code == 0 ? LB_ENAN : LB_ENOTCONV), step);
 }
 
@@ -940,7 +975,7 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
       }
       if (failed) break;
       // every block reads the adjoint's scales and the segment's stage scales block 0 wrote
-      if (!grid_sync(P.bar, gridDim.x, limit)) {
+      if (!gx_sync(S, P.bar, limit)) {
         gx_fail(P, -3, j0);
         failed = true;
         break;
@@ -987,7 +1022,7 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
       __syncthreads();
       for (int b = threadIdx.x; b < G.M; b += blockDim.x) S.sc[b] -= S.sh[b];
       // the first pass below writes zA, whose neighbours other blocks may still be reading
-      if (!grid_sync(P.bar, gridDim.x, limit)) {
+      if (!gx_sync(S, P.bar, limit)) {
         gx_fail(P, -3, j);
         failed = true;
         break;

@@ -28,6 +28,7 @@ struct GridBar {
   unsigned int gen;    // generation counter
   int err;             // set when a wait gave up
   int pad;
+  unsigned long long arrived;  // blocks arrived since the launch; top bit: a wait gave up (fixed-point sweeps)
 };
 
 // Everything a kernel needs to know about one system, in device memory.
