@@ -122,6 +122,18 @@ typedef struct lb_system_desc {
   int64_t n_steps;             /* N_T >= 1; dt = T/N_T (uniform grid, Appendix A) */
 } lb_system_desc;
 
+/* Arithmetic of the sweeps (chosen per call from the controls in effect).
+ * LB_ARITH_FIXED: states, iterates and gradient sums are 64-bit integers with
+ * one power of two per state, on the integer pipe; for the Jacobi iteration
+ * while every step's iteration matrix is bounded by 0.24 (the grid sweep: 1/16,
+ * no coupling, no running penalty) and the step's diagonal phases are small.
+ * Closer to the exact solution of the step than FP64.  The predictor's order
+ * counts up to 8 for the states it keeps in registers.  A call recorded into
+ * a CUDA graph, and a workspace without these sweeps' tables (smaller than
+ * lb_workspace_bytes says), run LB_ARITH_F64. */
+#define LB_ARITH_F64 0
+#define LB_ARITH_FIXED 1
+
 /* Solver statistics of the last lb_forward / lb_gradient / lb_propagate.
  * Phases: 0 = forward sweep, 1 = stage vectors of the checkpoint segments, 2 =
  * adjoint steps (which also evaluate the gradient pieces of eq. reducedgradient).
@@ -142,7 +154,7 @@ typedef struct lb_stats {
   int32_t ckpt_every;       /* checkpoint interval in effect (0 = every stage vector kept) */
   int32_t symmetry;         /* LB_SYM_HERMITIAN when the sweep iterated k <= l only */
   int32_t states_integrated; /* states the sweeps integrated (conjugate pairs count once, lb_set_pairing) */
-  int32_t pad;
+  int32_t arithmetic;       /* LB_ARITH_* the forward and adjoint sweeps ran in */
   int64_t phase_diff_iterations[3]; /* of phase_iterations: difference iterations in single precision
                                        (grid sweeps, lb_set_difference_iterations) */
 } lb_stats;
@@ -198,7 +210,8 @@ int lb_objective_set_gate(lb_system* sys, int32_t kind, const double* V, double 
  * (rho_j >= 1/2, or the Neumann iteration); max_iter caps the
  * iterations of one step (LB_ENOTCONV beyond); ckpt_every = K >= 1 stores the
  * forward state every K steps and recomputes each K-step segment in the
- * backward sweep; K = 0 stores every stage vector z^j instead (no recompute);
+ * backward sweep (the fixed-point sweeps keep the last one from the forward
+ * sweep); K = 0 stores every stage vector z^j instead (no recompute);
  * K = LB_CKPT_AUTO keeps every stage vector when that tape takes at most
  * 8 GiB (M * N_T * N^2 * 16 bytes) and checkpoints every 100 steps otherwise.
  * Defaults: LB_SOLVER_AUTO, 1e-15, 200, 100.  Call before lb_workspace_bytes. */
@@ -280,7 +293,7 @@ int lb_get_predictor(const lb_system* sys, int32_t* restart, int32_t* order);
 
 /* Bound of the grid sweeps' barrier waits (failure detection; the paper has
  * no counterpart).  Each block polls the grid barrier at most `polls` times
- * (about 64 ns apart) before it gives up; a wait that gives up makes every
+ * (some 100 ns apart) before it gives up; a wait that gives up makes every
  * block of the launch return, and the call reports LB_ECUDA with the time
  * step ("a grid barrier wait gave up at time step j").  The handle stays
  * usable: the next call clears the barrier.  0 restores the default
@@ -288,7 +301,8 @@ int lb_get_predictor(const lb_system* sys, int32_t* restart, int32_t* order);
  * the new bound is uploaded on the bind stream, which is synchronised. */
 int lb_set_wait_limit(lb_system* sys, int64_t polls);
 
-/* Single-precision difference iterations of the grid sweeps' Jacobi solves
+/* Single-precision difference iterations of the grid sweeps' Jacobi solves in
+ * FP64 (LB_ARITH_F64; the fixed-point sweeps have none)
  * (on = 1, the default; 0 = every inner iteration in FP64).  The implicit
  * midpoint step (I - dt/2 M) z = q (Appendix A, eqs. IMR, linsystem_primal) is solved by
  * z_{k+1} = (I - dt/2 D)^-1 (q + c(z_k)), c(z) = (dt/2) O z, O the
@@ -425,7 +439,8 @@ int lb_propagate(lb_system* sys, void* stream, int32_t adjoint, int64_t j0, int6
 
 /* y = M^{j+1/2} x (adjoint = 0) or y = (M^{j+1/2})^+ x (adjoint = 1) for
  * n_vec device vectors (Appendix A, eq. mastereq_vectorized), with
- * M^{j+1/2} = M(t_j + dt/2); x and y must not overlap. */
+ * M^{j+1/2} = M(t_j + dt/2); x and y must not overlap.  Many elements at once
+ * (grid sweeps, n_vec <= M) pass through the workspace's iteration buffers. */
 int lb_apply(lb_system* sys, void* stream, int32_t adjoint, int64_t step, const void* x_dev, void* y_dev,
              int32_t n_vec);
 

@@ -36,6 +36,9 @@ LB_SWEEP_RESIDENT = 1
 LB_SWEEP_GRID = 2
 LB_SWEEP_CLUSTER = 3
 
+LB_ARITH_F64 = 0
+LB_ARITH_FIXED = 1
+
 LB_SOLVER_AUTO = 0
 LB_SOLVER_JACOBI = 1
 LB_SOLVER_NEUMANN = 2
@@ -88,7 +91,7 @@ class lb_stats(ctypes.Structure):
         ("ckpt_every", c_int32),
         ("symmetry", c_int32),
         ("states_integrated", c_int32),
-        ("pad", c_int32),
+        ("arithmetic", c_int32),
         ("phase_diff_iterations", c_int64 * 3),
     ]
 

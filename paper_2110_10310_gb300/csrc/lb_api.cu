@@ -363,7 +363,16 @@ bool use_fixed(const lb_system* s, bool herm) {
   if (use_grid(s)) return rho_bound(s) <= lbk::kGridFixedRho;
   return fixed_cfg(s, herm).E > 0 && rho_bound(s) <= lbk::kFixedRho;
 }
-bool use_fixed(const lb_system* s) { return use_fixed(s, s->hp.herm != 0); }
+// ... on this stream: a call recorded into a graph of the caller's may be
+// replayed with controls of any size, which no host check sees then, so it
+// records the FP64 sweeps
+bool use_fixed(const lb_system* s, bool herm, cudaStream_t st) {
+  if (!use_fixed(s, herm)) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap == cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();
+  return true;
+}
 
 // ... and those in chunks: without the Hermitian element plan
 bool use_chunks(const lb_system* s) { return s->hp.chunkL > 0 && s->cluster && !s->hp.herm; }
@@ -1138,7 +1147,7 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.gslots), 0, s->L.gslots.bytes, st), "clear grid slots");
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
       LB_CUDA(cudaEventRecord(a, st), "cudaEventRecord");
-      if (use_fixed(s))
+      if (use_fixed(s, s->hp.herm != 0))
         LB_CUDA(lbk::launch_sweep_gx(s->dp, s->hp, 0, 0, 0, pst, nullptr, s->M, st), "forward grid sweep");
       else
         LB_CUDA(lbk::launch_sweep_grid(s->dp, 0, 1, 0, 0, pst, nullptr, s->M, s->gblocks, s->gsmem, s->hp.ff, st),
@@ -1599,7 +1608,7 @@ static int run_forward(lb_system* s, cudaStream_t st, int tape) {
     LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
     if (s->gamma1 != 0.0) LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.jpen), 0, s->L.jpen.bytes, st), "clear penalty");
     if (s->timing) LB_CUDA(cudaEventRecord(s->ev[0], st), "cudaEventRecord");
-    s->fx_now = use_fixed(s);
+    s->fx_now = use_fixed(s, s->hp.herm != 0, st);
     if (s->fx_now)
       LB_CUDA(lbk::launch_sweep_gx(s->dp, s->hp, 0, tape, 0, s->NT, nullptr, s->M, st), "forward grid sweep");
     else
@@ -1614,7 +1623,7 @@ static int run_forward(lb_system* s, cudaStream_t st, int tape) {
     return LB_OK;
   }
   if (s->timing) LB_CUDA(cudaEventRecord(s->ev[0], st), "cudaEventRecord");
-  s->fx_now = use_fixed(s);
+  s->fx_now = use_fixed(s, s->hp.herm != 0, st);
   if (s->fx_now && use_chunks(s))
     LB_CUDA(lbk::launch_forward_chunks(s->dp, s->hp, tape, fixed_cfg(s, false), st), "forward kernels");
   else if (s->fx_now)
@@ -1648,6 +1657,7 @@ static int finish(lb_system* s, cudaStream_t st, double* G_out, double* grad_out
   LB_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
   int rc = read_status(d, &s->last, s->launches);
   s->last.sweep = use_grid(s) ? LB_SWEEP_GRID : (s->cluster ? LB_SWEEP_CLUSTER : LB_SWEEP_RESIDENT);
+  s->last.arithmetic = s->fx_now ? LB_ARITH_FIXED : LB_ARITH_F64;
   s->last.solver = s->method;
   s->last.ckpt_every = effective_K(s);
   s->last.symmetry = s->hp.herm ? LB_SYM_HERMITIAN : LB_SYM_NONE;
@@ -1869,6 +1879,7 @@ static int propagate_impl(lb_system* s, cudaStream_t st, int adjoint, int64_t j0
   int rc = order_after_uploads(s, st);
   if (rc) return rc;
   s->launches = 0;
+  s->fx_now = use_fixed(s, false, st);
   rc = ensure_ctab(s, st);
   if (rc) return rc;
   LB_CUDA(cudaMemsetAsync(at<DevStatus>(s, s->L.status), 0, sizeof(DevStatus), st), "clear status");
@@ -1878,13 +1889,13 @@ static int propagate_impl(lb_system* s, cudaStream_t st, int adjoint, int64_t j0
       if (n_vec > s->M) return fail(LB_EINVAL, "grid sweeps propagate at most M vectors at a time");
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.gslots), 0, s->L.gslots.bytes, st), "clear grid slots");
       LB_CUDA(cudaMemsetAsync(at<char>(s, s->L.bar), 0, s->L.bar.bytes, st), "clear grid barrier");
-      if (use_fixed(s, false))
+      if (s->fx_now)
         LB_CUDA(lbk::launch_sweep_gx(s->dp, s->hp, adjoint ? 2 : 1, 0, j0, j1, x, n_vec, st), "propagate grid sweep");
       else
         LB_CUDA(lbk::launch_sweep_grid(s->dp, adjoint ? 2 : 1, 0, 0, j0, j1, x, n_vec, s->gblocks, s->gsmem, s->hp.ff,
                                        st),
                 "propagate grid sweep");
-    } else if (use_fixed(s, false)) {
+    } else if (s->fx_now) {
       LB_CUDA(lbk::launch_propagate_fixed(s->dp, adjoint, j0, j1, x, n_vec, fixed_cfg(s, false), st),
               "propagate kernel");
     } else if (s->cluster) {
@@ -2067,7 +2078,7 @@ static std::vector<WorkItem> fx_groups(lb_batch* b, const std::vector<WorkItem>&
 static bool batch_fixed(const lb_batch* b) {
   if (b->fx.empty()) return false;
   for (const lb_system* s : b->sys)
-    if (!use_fixed(s)) return false;
+    if (!use_fixed(s, s->hp.herm != 0)) return false;
   return true;
 }
 

@@ -43,6 +43,7 @@ def _stats_dict(s) -> dict:
             "solver": {1: "jacobi", 2: "neumann", 3: "gmres"}.get(s.solver, s.solver),
             "symmetry": "hermitian" if s.symmetry == L.LB_SYM_HERMITIAN else "none",
             "ckpt_every": s.ckpt_every, "states_integrated": s.states_integrated,
+            "arithmetic": "fixed" if s.arithmetic == L.LB_ARITH_FIXED else "f64",
             "phase_diff_iterations": list(s.phase_diff_iterations)}
 
 

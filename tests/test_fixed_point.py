@@ -255,3 +255,32 @@ def test_last_segment_kept_by_the_forward_sweep(L, levels, sweep, K):
         assert G == G0 and np.array_equal(g, g0)
         st = s.stats()
         assert st["phase_steps"][1] == st["phase_steps"][0] and st["phase_iterations"][1] == st["phase_iterations"][0]
+
+
+# A recorded call serves controls of any size on replay: it is the FP64 sweeps
+# that are recorded, whatever the controls were then.
+@gpu
+@pytest.mark.parametrize("sweep", ["auto", "resident", "grid"])
+def test_recorded_gradient_replays_with_larger_controls(L, sweep):
+    sw = {"auto": L.LB_SWEEP_AUTO, "resident": L.LB_SWEEP_RESIDENT, "grid": L.LB_SWEEP_GRID}[sweep]
+    p = _problem((3, 2), 70, True, 0)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s = _sys(p, sweep=sw)
+        G, g = torch.zeros(1, dtype=torch.float64, device="cuda"), torch.zeros(s.n_params, dtype=torch.float64,
+                                                                               device="cuda")
+        s.gradient()
+        assert s.stats()["arithmetic"] == "fixed"
+        s.set_alpha(p.controls.alpha)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            s.gradient_async(G, g, stream=st)
+        for scale in (1.0, 40.0):
+            s.set_alpha(scale * p.controls.alpha)
+            graph.replay()
+            torch.cuda.synchronize()
+            q = copy.deepcopy(p)
+            q.controls.alpha = scale * p.controls.alpha
+            Go, go = _sys(q, sweep=sw).gradient()
+            assert abs(float(G) - Go) <= 1e-12 * abs(Go) and _rel(g.cpu().numpy(), go) < 1e-11
