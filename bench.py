@@ -307,6 +307,45 @@ def method_flops(V: int, Q: int, st: dict, phase_set) -> float:
     return f
 
 
+def fixed_products(V: int, Q: int, n_decay: int, st: dict, phase_set) -> float:
+    """32 x 32 -> 64 bit multiply-adds of the fixed-point sweeps (three per
+    real product), from the iteration counts.  Per element and inner iteration:
+    36 per subsystem (the neighbours and the control factor), 6 per decaying
+    subsystem and 12 for (I - dt/2 D)^-1.  Per element and step: 12 for the first
+    iterate and 80 for the predictor (its sum of 8, the correction, the frame
+    and its phase).  Adjoint steps: 36 per subsystem for the gradient pieces."""
+    f = 0.0
+    for ph in phase_set:
+        f += V * ((36 * Q + 6 * n_decay + 12) * st["phase_iterations"][ph] + 92 * st["phase_steps"][ph])
+        if ph == 2:
+            f += V * 36 * Q * st["phase_steps"][ph]
+    return f
+
+
+def fixed_peak_tops(dev, sm_mhz: float | None) -> tuple[float, str]:
+    """Rate of the wide integer multiply-add: one warp instruction per 2 cycles
+    and SM sub-partition (measured), 64 per SM and clock."""
+    import torch
+
+    nsm = torch.cuda.get_device_properties(dev).multi_processor_count
+    mhz = sm_mhz or measured_peaks().get("sm_max_mhz") or 2070.0
+    return 64 * nsm * mhz * 1e6 / 1e12, (f"IMAD.WIDE: 64/SM/clk (measured) x {nsm} SMs (queried) x {mhz:.0f} MHz "
+                                         f"({'median sampled in the timed region' if sm_mhz else 'maximum clock'})")
+
+
+def swept_phases(st: dict, n_steps: int) -> dict:
+    """The statistics with phase 1 cut to what the backward sweep recomputes:
+    the fixed-point sweeps keep the last segment from the forward sweep."""
+    K = st["ckpt_every"]
+    if st.get("arithmetic") != "fixed" or K <= 0 or not st["phase_steps"][1]:
+        return st
+    part = (n_steps - 1) // K * K / n_steps
+    cut = dict(st)
+    for key in ("phase_steps", "phase_iterations"):
+        cut[key] = [st[key][0], st[key][1] * part, st[key][2]]
+    return cut
+
+
 BYTES_PER_ELEMENT_ITERATION = 48  # read the iterate and the right-hand side, write the new iterate
 
 
@@ -324,6 +363,8 @@ def kernel_source_digest(path: str) -> str:
 
 
 KERNEL_SOURCES = {
+    "k_backward_gx": ("lb_gridx.cu", "lb_grid.cuh", "lb_fixed.cuh"),
+    "k_backward_fx": ("lb_fixed_backward.cu", "lb_fixed_sweep.cuh", "lb_fixed.cuh"),
     "k_backward_grid": ("lb_grid.cu", "lb_device.cuh"),
     "k_sweep_grid": ("lb_grid.cu", "lb_device.cuh"),
     # the paired-single instantiations (lb_set_precision LB_PREC_F32X2)
@@ -451,6 +492,8 @@ def run_apply(args, rank, world, dev):
     p = W.prefix(W.config5(n_states=n), 40)
     p.ckpt_every = 10
     s = LindbladSystem(p, device=dev)
+    s.forward()
+    fixed = s.stats()["arithmetic"] == "fixed"  # the product follows the sweeps
     lib = _lib.load()
     V = s.N * s.N
     x = torch.from_numpy(colmajor(p.rho0)).to(dev)
@@ -482,7 +525,11 @@ def run_apply(args, rank, world, dev):
     peaks = measured_peaks()
     hbm_peak = peaks.get("hbm_gbs") or 6800.0
     clocks = clk.summary()
-    fp64_peak, src = fp64_peak_tflops(dev, clocks["sm_mhz"] if clocks else None)
+    peak, src = fp64_peak_tflops(dev, clocks["sm_mhz"] if clocks else None)
+    done, unit = flops, "TFLOP/s"
+    if fixed:
+        peak, src = fixed_peak_tops(dev, clocks["sm_mhz"] if clocks else None)
+        done, unit = n * V * (36 * Q + 6 * n_decay), "T wide integer multiply-adds/s"
     if rank == 0:
         line = {
             "metric": "Lindblad apply state-applies/s (FP64)",
@@ -501,12 +548,12 @@ def run_apply(args, rank, world, dev):
                        "l2": "inputs ({:.0f} MB in, {:.0f} MB out) larger than L2".format(nbytes / 2e6, nbytes / 2e6),
                        "flops_per_element": 24 * Q + 4 * n_decay + 10, "bytes_per_element": 32},
             "roofline": {
-                "kernel": "k_apply",
+                "kernel": "k_apply_gx" if fixed else "k_apply",
                 "bound": "alu",
-                "achieved": flops / t / 1e12,
-                "peak": fp64_peak,
-                "unit": "TFLOP/s",
-                "frac": flops / t / 1e12 / fp64_peak,
+                "achieved": done / t / 1e12,
+                "peak": peak,
+                "unit": unit,
+                "frac": done / t / 1e12 / peak,
                 "peak_source": src,
                 "hbm_achieved_gbs": nbytes / t / 1e9,
                 "hbm_peak_gbs": hbm_peak,
@@ -764,12 +811,27 @@ def run_gradient(args, rank, world, dev, dist):
     n_decay = int(sum(1 for t in p.system.t1_us if np.isfinite(t) and t > 0))
     st = sts[-1]
     Ve = s.N * (s.N + 1) // 2 if st["symmetry"] == "hermitian" else V
-    kernel_name = {"grid": "k_backward_grid", "cluster": "k_backward_cl"}.get(st["sweep"], "k_backward_res")
+    fixed = st["arithmetic"] == "fixed"
+    st = swept_phases(st, p.system.n_steps)
+    if fixed:
+        kernel_name = "k_backward_gx" if st["sweep"] == "grid" else "k_backward_fx"
+    else:
+        kernel_name = {"grid": "k_backward_grid", "cluster": "k_backward_cl"}.get(st["sweep"], "k_backward_res")
     bwd_method = method_flops(Ve, Q, st, (1, 2))
     bwd_impl = fp64_flops(Ve, Q, n_decay, st, (1, 2))
     fwd_method = method_flops(Ve, Q, st, (0,))
     fp64_peak, peak_src = fp64_peak_tflops(dev, clocks["sm_mhz"] if clocks else None)
     achieved = bwd_method / (bwd_ms * 1e-3) / 1e12
+    unit, impl_frac = "TFLOP/s", bwd_impl / (bwd_ms * 1e-3) / 1e12 / fp64_peak
+    peak = fp64_peak
+    count = ("method count: (8 + 36 Q) per element per FP64 inner iteration (difference "
+             "iterations not counted) + 28 Q per element per adjoint step (gradient pieces)")
+    if fixed:
+        peak, peak_src = fixed_peak_tops(dev, clocks["sm_mhz"] if clocks else None)
+        achieved = fixed_products(Ve, Q, n_decay, st, (1, 2)) / (bwd_ms * 1e-3) / 1e12
+        unit, impl_frac = "T wide integer multiply-adds/s", achieved / peak
+        count = ("multiply-adds: 36 Q + 6 per decaying subsystem + 12 per element per inner iteration, 92 per "
+                 "element and step, 36 Q more per adjoint step")
     elem_iters = Ve * (st["phase_iterations"][1] + st["phase_iterations"][2])
     hbm_alg = BYTES_PER_ELEMENT_ITERATION * elem_iters
     hbm_peak = measured_peaks().get("hbm_gbs") or 6800.0
@@ -800,7 +862,7 @@ def run_gradient(args, rank, world, dev, dist):
             "higher_is_better": True,
             "scaling": "strong" if world > 1 else "weak",
             "vs_baseline": None,
-            "dtype": "f64" if args.precision == "f64" else "f64+f32x2",
+            "dtype": "f64 (int64 fixed point)" if fixed else "f64" if args.precision == "f64" else "f64+f32x2",
             "data": "synthetic",
             "config": static_config(wl, full),
             "fwd_value": full.M * full.system.n_steps / (fwd_ms * 1e-3),
@@ -816,11 +878,13 @@ def run_gradient(args, rank, world, dev, dist):
                 "autotune": tuned,
                 "inner_iters_per_step": inner,
                 "diff_iters_per_step": diff,
-                "precision": ("FP64 states, corrections, objective, gradient and stopping rule; inner iterations "
+                "arithmetic": "64-bit fixed point on the integer pipe" if fixed else "FP64",
+                "precision": ("64-bit fixed point, one power of two per state; objective, gradient projection and "
+                              "stopping rule FP64" if fixed else "FP64 states, corrections, objective, gradient and stopping rule; inner iterations "
                               "after the first of a step apply O to the single-precision change of the iterate "
                               "once it is below 2^-32 max|q| (lb_set_difference_iterations)"
                               if args.diff_iterations == "on" else "FP64 throughout")
-                             + ("; the other inner iterations apply O in pairs of single-precision numbers "
+                             + ("" if fixed else "; the other inner iterations apply O in pairs of single-precision numbers "
                                 "(about 48 significant bits, lb_set_precision LB_PREC_F32X2)"
                                 if args.precision == "f32x2" else ""),
                 "ms_forward_kernel": statistics.median(ms_fwd),
@@ -833,15 +897,13 @@ def run_gradient(args, rank, world, dev, dist):
                 "kernel": kernel_name,
                 "bound": "alu",
                 "achieved": achieved,
-                "peak": fp64_peak,
-                "unit": "TFLOP/s",
-                "frac": achieved / fp64_peak,
+                "peak": peak,
+                "unit": unit,
+                "frac": achieved / peak,
                 "peak_source": peak_src,
-                "flop_count": ("method count: (8 + 36 Q) per element per FP64 inner iteration (difference "
-                               "iterations not counted) + 28 Q per element per adjoint step (gradient pieces), "
-                               "over the elements the sweep computes "
+                "flop_count": (count + ", over the elements the sweep computes "
                                f"({Ve} per state: {'k <= l under the Hermitian symmetry' if Ve != V else 'all'})"),
-                "frac_instruction_count": bwd_impl / (bwd_ms * 1e-3) / 1e12 / fp64_peak,
+                "frac_instruction_count": impl_frac,
                 "hbm_achieved_gbs": hbm_alg / (bwd_ms * 1e-3) / 1e9,
                 "hbm_peak_gbs": hbm_peak,
                 "hbm_frac": hbm_alg / (bwd_ms * 1e-3) / 1e9 / hbm_peak,
