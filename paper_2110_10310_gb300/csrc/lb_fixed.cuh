@@ -107,6 +107,14 @@ __host__ __device__ __forceinline__ unsigned fx_abs_sat(long long X) {
   const unsigned a = l < 0 ? 0u - (unsigned)l : (unsigned)l;
   return h == (l >> 31) ? a : 0xffffffffu;
 }
+// leading zero bits of h != 0
+__host__ __device__ __forceinline__ int fx_clz(unsigned h) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)h);
+#else
+  return __builtin_clz(h);
+#endif
+}
 // X 2^-s (s < 0: X 2^|s|)
 __host__ __device__ __forceinline__ long long fx_shift(long long X, int s) {
   if (s > 61 || s < -61) return 0;  // (to the left: X is zero there)
@@ -162,6 +170,14 @@ __device__ __forceinline__ long long fx_from_bits(double x, int sc) {
 // start and the scale moved by 2 when it has left [2^58.5, 2^60)
 constexpr int kFxTop = 59;
 constexpr unsigned kFxHigh = 1u << (60 - 32), kFxLow = 94906266u;  // 2^26.5
+
+// The shift that gives a quarter of a state its scale, from the quarter's
+// largest high word: back to the state as it is when that lies in [2^58.5,
+// 2^60), else to a largest entry in [2^59, 2^60).
+__host__ __device__ __forceinline__ int fx_quarter_shift(unsigned top) {
+  if (top == 0 || (top < kFxHigh / 4 && top >= kFxLow / 4)) return -2;
+  return 4 - fx_clz(top);  // the top bit of the high word to bit 27
+}
 
 }  // namespace
 }  // namespace lbk

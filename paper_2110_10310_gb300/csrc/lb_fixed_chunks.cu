@@ -155,8 +155,8 @@ __device__ __forceinline__ int4 fx_split2(Cx q) {
 }
 
 // Take the value of entry threadIdx.x (< V, else ignored) of the next boundary
-// state, plus `add` (ADD): set its scale by its largest entry, keep it split in
-// S.x and store it.
+// state, at the scale sc, plus `add` (ADD): set its scale by its largest entry,
+// keep it split in S.x and store it.
 template <bool ADD>
 __device__ void fx_boundary(const FxCombine& S, const ProbDev& P, Cx q, double2 add, int& sc, int V, size_t b) {
   const int t = threadIdx.x;
@@ -172,8 +172,7 @@ __device__ void fx_boundary(const FxCombine& S, const ProbDev& P, Cx q, double2 
     if ((t & 31) == 0) w[t >> 5] = m;
     __syncthreads();
     const unsigned top = __reduce_max_sync(kFull, (t & 31) < (int)(blockDim.x >> 5) ? w[t & 31] : 0u);
-    // the top bit of the largest high word to bit 27: the largest entry in [2^59, 2^60)
-    if (top && (top >= kFxHigh || top < kFxLow)) s = 4 - __clz(top);
+    s = fx_quarter_shift(top);
   }
   sc -= s;
   if (t < V) {
@@ -189,7 +188,10 @@ __device__ void fx_boundary(const FxCombine& S, const ProbDev& P, Cx q, double2 
   if (t == 0) P.bsc[b] = sc;
   __syncthreads();
 }
-// entry threadIdx.x of the product from the G partial sums (a quarter each)
+// entry threadIdx.x of the product from the G partial sums: a quarter of it.
+// A chunk can raise the largest entry (a uniform superposition turned into a
+// basis state: up to N times), so the sum stays a quarter, its scale 2 less,
+// until fx_boundary has seen its size.
 __device__ __forceinline__ Cx fx_take(const FxCombine& S, int G, int V) {
   Cx q{0, 0};
   if ((int)threadIdx.x < V) {
@@ -198,8 +200,6 @@ __device__ __forceinline__ Cx fx_take(const FxCombine& S, int G, int V) {
       q.x += p.x;
       q.y += p.y;
     }
-    q.x <<= 2;
-    q.y <<= 2;
   }
   return q;
 }
@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(1024) k_boundary_fx(const ProbDev* __restrict_
       S.part[g * V + v] = make_longlong2(re, im);
     }
     __syncthreads();
+    sc -= 2;
     fx_boundary<false>(S, P, fx_take(S, G, V), make_double2(0.0, 0.0), sc, V, (size_t)(c + 1) * M + i);
   }
 }
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(1024) k_boundary_adj_fx(const ProbDev* __restr
     }
     __syncthreads();
     const Cx q = fx_take(S, G, V);
+    sc -= 2;
     if (P.gamma1 != 0.0) {
       // the chunk's response to its own penalty sources
       double2 add = make_double2(0.0, 0.0);

@@ -1,0 +1,88 @@
+"""The fixed-point sweeps at the limits of their arithmetic: states that grow,
+cancel, vanish or decay between two rescalings, peaked states, tables that do
+not fit, and the calls that share their buffers.
+
+Tolerances: the method's accuracy targets against the oracle (states and
+objective 1e-10, gradient 1e-9 of the largest entry) unless a test derives its
+own."""
+
+import copy
+import ctypes
+
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import imr, model
+
+torch = pytest.importorskip("torch")
+gpu = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2110_10310_gb300 import _lib
+
+    _lib.load(build_if_missing=True)
+    return _lib
+
+
+def _rel(a, b):
+    return float(np.max(np.abs(np.asarray(a) - np.asarray(b))) / np.max(np.abs(b)))
+
+
+def _sys(p, **kw):
+    from paper_2110_10310_gb300.system import LindbladSystem
+
+    return LindbladSystem(p, **kw)
+
+
+def _fixed(s):
+    assert s.stats()["arithmetic"] == "fixed"
+    return s
+
+
+def _basis(levels, k, l):
+    N = int(np.prod(levels))
+    r = np.zeros((N, N), dtype=np.complex128)
+    r[k, l] = 1.0
+    return r
+
+
+def _constant_drive(levels, n_steps, h, theta, t1_us=100.0, t2_us=50.0):
+    """Resonant subsystems under constant drives of theta rad per step."""
+    p = W.random_problem(811, levels=levels, n_states=1, n_steps=n_steps, T_ns=h * n_steps, amp=0.01, ckpt_every=0)
+    Q = len(levels)
+    p.system.detuning_ghz[:] = 0.0
+    p.system.selfkerr_ghz[:] = 0.0
+    p.system.crosskerr_ghz[:] = 0.0
+    p.system.t1_us, p.system.t2_us = np.full(Q, t1_us), np.full(Q, t2_us)
+    p.controls.carriers_ghz = [np.zeros(1) for _ in range(Q)]
+    a = np.zeros((Q, 1, p.controls.n_splines, 2))
+    a[..., 0] = theta / (2.0 * np.pi * h)
+    p.controls.alpha = a.reshape(-1)
+    p.weights = None
+    p.rho0 = np.stack([_basis(levels, 0, 0)])
+    return p
+
+
+@gpu
+def test_an_adjoint_state_that_gathers_within_a_chunk(L):
+    """The target is what |00> has spread into over the last chunk's 22 steps,
+    so that the adjoint state gathers into one entry 8.4 times its largest
+    there: 2^63.06 in the scale of the chunk's end."""
+    p = _constant_drive((3, 3), 748, 0.1, 0.0476)
+    m = model.Model(p.system, p.controls)
+    q = model.vec(p.rho0).T.copy()
+    for j in range(726, 748):
+        q, _ = imr.imr_step(m, j, q)
+    p.targets = model.unvec(q[:, 0], 9)[None]
+    p.objective, p.weights = "trace", np.array([1.04])
+    s = _sys(p)
+    G, g = s.gradient()
+    assert _fixed(s).stats()["sweep"] == "cluster"
+    Go, go, _ = imr.gradient(p)
+    assert abs(G - Go) <= 1e-10 * abs(Go)
+    assert _rel(g, go) < 1e-9
