@@ -162,9 +162,14 @@ __device__ void fx_boundary(const FxCombine& S, const ProbDev& P, Cx q, double2 
   const int t = threadIdx.x;
   int s = 0;
   if (ADD) {
-    double2 d = make_double2(0.0, 0.0);
-    if (t < V) d = make_double2(fx_to(q.x, sc) + add.x, fx_to(q.y, sc) + add.y);
-    const unsigned long long mx = fx_block_max(S.mx, t < V ? umax64(abs_bits(d.x), abs_bits(d.y)) : 0ull);
+    // the largest of state, addend and sum: the two may cancel
+    unsigned long long m = 0;
+    if (t < V) {
+      const double2 x = make_double2(fx_to(q.x, sc), fx_to(q.y, sc));
+      m = umax64(umax64(abs_bits(x.x), abs_bits(x.y)), umax64(abs_bits(add.x), abs_bits(add.y)));
+      m = umax64(m, umax64(abs_bits(x.x + add.x), abs_bits(x.y + add.y)));
+    }
+    const unsigned long long mx = fx_block_max(S.mx, m);
     if (mx && mx < kInfBits) s = sc - fx_scale(mx);
   } else {
     unsigned* w = reinterpret_cast<unsigned*>(S.mx);

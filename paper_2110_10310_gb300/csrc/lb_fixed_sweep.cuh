@@ -848,13 +848,18 @@ __device__ __forceinline__ void fx_rescale(FxState<E, QT>& st, const FxSmem& S, 
   if (qtop < kFxHigh && (qtop >= kFxLow || qtop == 0)) return;
   fx_scale_by(st, S, qtop >= kFxHigh ? 1 : -1, pred);
 }
-// q += src (FP64, each lane's component): the scale follows the sum's largest
-// entry first, which a source may raise by any factor in one step (all threads)
+// q += src (FP64, each lane's component): the scale first follows the largest
+// of state, source and sum, which a source may raise by any factor in one step
+// (of the sum alone it would shift a state that the source cancels past 64
+// bits) (all threads)
 template <int E, int QT>
 __device__ __forceinline__ void fx_add_source(FxState<E, QT>& st, const FxSmem& S, const double (&src)[E], bool pred) {
   unsigned long long mx = 0;
 #pragma unroll
-  for (int e = 0; e < E; ++e) mx = umax64(mx, abs_bits(fx_to(st.q[e], st.sc) + src[e]));
+  for (int e = 0; e < E; ++e) {
+    const double x = fx_to(st.q[e], st.sc);
+    mx = umax64(mx, umax64(abs_bits(x + src[e]), umax64(abs_bits(x), abs_bits(src[e]))));
+  }
   mx = fx_cta_max(S, mx);
   if (mx >= kInfBits) return;
   const int sc = fx_scale(mx);

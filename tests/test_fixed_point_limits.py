@@ -86,3 +86,26 @@ def test_an_adjoint_state_that_gathers_within_a_chunk(L):
     Go, go, _ = imr.gradient(p)
     assert abs(G - Go) <= 1e-10 * abs(Go)
     assert _rel(g, go) < 1e-9
+
+
+@gpu
+@pytest.mark.parametrize("n_steps,theta,weight,sweep", [(24, 0.7796, 1.0, "resident"), (64, np.pi / 4.5, 1.06, "cluster")])
+def test_a_penalty_source_that_cancels_the_adjoint_state(L, n_steps, theta, weight, sweep):
+    """A free coherence whose adjoint turns by theta per step while a constant
+    running penalty adds the same source each step: the sum falls to some
+    hundredths of both addends -- after seven sources in the sequential sweep,
+    and where the response of a chunk's eight sources meets the adjoint state."""
+    h = 0.1
+    p = _constant_drive((2,), n_steps, h, 1e-4, t1_us=np.inf, t2_us=np.inf)
+    # the implicit midpoint step turns a phase by 2 atan(h delta / 2)
+    p.system.detuning_ghz[:] = 2.0 * np.tan(0.5 * theta) / h / (2.0 * np.pi)
+    p.rho0 = np.full((1, 2, 2), 0.5, dtype=np.complex128)
+    p.targets = np.array([[[0.0, 0.5], [0.5, 0.0]]], dtype=np.complex128)
+    p.objective, p.penalty_a = "trace", 1e6
+    p.gamma1 = weight * p.penalty_a / h
+    s = _sys(p)
+    G, g = s.gradient()
+    assert _fixed(s).stats()["sweep"] == "cluster" and (s.stats()["kernel_launches"] > 8) == (sweep == "cluster")
+    Go, go, _ = imr.gradient(p)
+    assert abs(G - Go) <= 1e-10 * abs(Go)
+    assert _rel(g, go) < 1e-9
