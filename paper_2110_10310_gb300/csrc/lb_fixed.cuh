@@ -171,6 +171,15 @@ __device__ __forceinline__ long long fx_from_bits(double x, int sc) {
 constexpr int kFxTop = 59;
 constexpr unsigned kFxHigh = 1u << (60 - 32), kFxLow = 94906266u;  // 2^26.5
 
+// Largest change of an iterate that ends a solve: fac (rtol times the step's
+// factor) of the right-hand side's largest entry (its high word), in units of
+// the state; never below one unit, so that a state of zeros and an iterate
+// that a tolerance below the format's resolution asks for are accepted.
+__device__ __forceinline__ unsigned fx_stop(float fac, unsigned qtop) {
+  const float t = fac * (float)qtop * 4294967296.0f;
+  return t >= 4294967040.0f ? 0xffffff00u : (t >= 1.0f ? (unsigned)t : 1u);
+}
+
 // The shift that gives a quarter of a state its scale, from the quarter's
 // largest high word: back to the state as it is when that lies in [2^58.5,
 // 2^60), else to a largest entry in [2^59, 2^60).

@@ -693,9 +693,7 @@ __device__ __forceinline__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, con
   qtop = fx_slots_max(qs, nwarps);
   const int4 last = ctl[cq];
   if (last.y != 0) return -1;
-  // rtol max|rhs| (its high word) times the step's factor, in units of the state
-  const float thf = __int_as_float(last.x) * (float)qtop * 4294967296.0f;
-  const unsigned thr = thf >= 4294967040.0f ? 0xffffff00u : (unsigned)thf;
+  const unsigned thr = fx_stop(__int_as_float(last.x), qtop);
   for (int it = 0; it < maxit; ++it) {
     const Fx* __restrict__ zc = cur ? S.zb1 : S.zb0;
     Fx* __restrict__ zn = cur ? S.zb0 : S.zb1;
@@ -749,7 +747,7 @@ __device__ __forceinline__ int fx_solve(FxState<E, QT>& st, const FxSmem& S, con
     __syncthreads();
     dm = fx_slots_max(ds, nwarps);
     cur ^= 1;
-    if (dm < thr) return it + 1;
+    if (dm <= thr) return it + 1;
   }
   return -1;
 }

@@ -513,9 +513,7 @@ __device__ int gx_solve(const ProbDev& P, const GxParams& gp, const GxSmem& S, c
       const float fac = __int_as_float(S.flag[1]);
       for (int b = threadIdx.x; b < M; b += 32) {
         const unsigned q = __ldcg(qbank + b), d = __ldcg(bank + b);
-        const float thf = fac * (float)q * 4294967296.0f;
-        const unsigned thr = thf >= 4294967040.0f ? 0xffffff00u : (unsigned)thf;
-        if (d > thr) open = true;
+        if (d > fx_stop(fac, q)) open = true;
       }
       open = __any_sync(kFull, open);
       if (!open)

@@ -109,3 +109,44 @@ def test_a_penalty_source_that_cancels_the_adjoint_state(L, n_steps, theta, weig
     Go, go, _ = imr.gradient(p)
     assert abs(G - Go) <= 1e-10 * abs(Go)
     assert _rel(g, go) < 1e-9
+
+
+def _vanishing(levels, n_steps, zero):
+    """Two states, one of which has a zero weight or is zero itself."""
+    p = W.random_problem(813, levels=levels, n_states=2, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.02, ckpt_every=0)
+    p.weights = np.array([1.0, 1.0])
+    if zero == "weight":
+        p.weights[1] = 0.0
+    else:
+        p.rho0[1] = 0.0
+    return p
+
+
+@gpu
+@pytest.mark.parametrize("levels,n_steps,sweep", [((2, 2), 24, 1), ((2, 2), 80, 0), ((3, 2, 3), 10, 1), ((3, 3), 20, 2)])
+@pytest.mark.parametrize("zero", ["weight", "state"])
+def test_states_of_zeros(L, levels, n_steps, sweep, zero):
+    """The one-CTA sweeps (register and table path), the chunks and the grid."""
+    p = _vanishing(levels, n_steps, zero)
+    s = _sys(p, sweep=sweep)
+    G, g = s.gradient()
+    _fixed(s)
+    Go, go, _ = imr.gradient(p)
+    assert abs(G - Go) <= 1e-10 * abs(Go)
+    assert _rel(g, go) < 1e-9
+    x = torch.from_numpy(p.rho0).cuda()
+    x[0] = 0.0
+    for adj in (False, True):
+        assert not s.propagate(x[:1], 0, n_steps, adjoint=adj).any()
+
+
+@gpu
+@pytest.mark.parametrize("levels,n_steps,sweep", [((2, 2), 24, 1), ((2, 2), 80, 0), ((3, 2, 3), 10, 1), ((3, 3), 20, 2)])
+def test_a_tolerance_below_the_resolution(L, levels, n_steps, sweep):
+    p = W.random_problem(814, levels=levels, n_states=2, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.02, ckpt_every=0)
+    s = _sys(p, sweep=sweep, rtol=1e-30)
+    G, g = s.gradient()
+    _fixed(s)
+    Go, go, _ = imr.gradient(p)
+    assert abs(G - Go) <= 1e-10 * abs(Go)
+    assert _rel(g, go) < 1e-9
