@@ -80,6 +80,30 @@ __host__ __device__ __forceinline__ FxAcc fx_acc() {
   s.mid = 0x80000000LL;
   return s;
 }
+// high half of a 32 x 32 bit product
+__host__ __device__ __forceinline__ int fx_mulhi(int a, int b) {
+#ifdef __CUDA_ARCH__
+  return __mulhi(a, b);
+#else
+  return (int)(((long long)a * (long long)b) >> 32);
+#endif
+}
+// A sum of products of two states' entries, hi 2^32 + lo in units of 2^32: each
+// product whole but for its last 32 bits.  A gradient sum adds the products of
+// all entries, and with one large entry among many small ones those small
+// products are the gradient: cut at 2^64 (fx_val) they would carry an error of
+// 2^-56 of the two states' largest entries each.
+struct FxSum {
+  long long hi;
+  unsigned lo;
+};
+__host__ __device__ __forceinline__ void fx_sum_mac(FxSum& s, Fx a, Fx x) {
+  long long mid = fx_madw(a.h, x.l, (long long)fx_mulhi(a.l, x.l));
+  mid = fx_madw(a.l, x.h, mid);
+  const unsigned long long lo = (unsigned long long)s.lo + (unsigned)mid;
+  s.lo = (unsigned)lo;
+  s.hi = fx_madw(a.h, x.h, s.hi) + (mid >> 32) + (long long)(lo >> 32);
+}
 __host__ __device__ __forceinline__ long long fx_join(Fx a) {
   return (long long)((unsigned long long)(unsigned)a.h << 32) + (long long)a.l;
 }

@@ -7,13 +7,20 @@ namespace lbk {
 
 namespace {
 
-// exact sum over the warp of v (|v| < 2^62) in three limbs of 24 bits: sums
-// l0 + l1 2^24 + l2 2^48, to every lane
-__device__ __forceinline__ int3 fx_warp_sum(long long v) {
+// sum over the warp of v, in words of 32 bits from 2^-24 of a product's cut at
+// 2^64 up (exact in limbs of 24 bits, then without the lowest 8), to every lane
+__device__ __forceinline__ int3 fx_warp_sum(const FxSum& v) {
+  const unsigned h0 = (unsigned)v.hi;
+  const unsigned s0 = __reduce_add_sync(kFull, v.lo & 0xffffffu);
+  const unsigned s1 = __reduce_add_sync(kFull, (v.lo >> 24 | h0 << 8) & 0xffffffu);
+  const unsigned s2 = __reduce_add_sync(kFull, (unsigned)(v.hi >> 16) & 0xffffffu);
+  const int s3 = __reduce_add_sync(kFull, (int)(v.hi >> 40));
+  unsigned long long t = (s0 >> 8) + ((unsigned long long)s1 << 16);
   int3 r;
-  r.x = __reduce_add_sync(kFull, (int)((unsigned)v & 0xffffffu));
-  r.y = __reduce_add_sync(kFull, (int)((unsigned)(v >> 24) & 0xffffffu));
-  r.z = __reduce_add_sync(kFull, (int)(v >> 48));
+  r.x = (int)(unsigned)t;
+  t = (t >> 32) + ((unsigned long long)s2 << 8);
+  r.y = (int)(unsigned)t;
+  r.z = s3 + (int)(t >> 32);
   return r;
 }
 
@@ -23,34 +30,30 @@ __device__ __forceinline__ int3 fx_warp_sum(long long v) {
 // +-Z_{1-c} R_c to Im A; the same with P for B).  herm: 0, or under the
 // Hermitian symmetry 1 off and 2 on the diagonal.
 struct FxG {
-  long long ar, ai, br, bi;
+  FxSum ar, ai, br, bi;
 };
-__device__ __forceinline__ long long fx_prod(long long a, long long b) {
-  FxAcc s = fx_acc();
-  fx_mac(s, fx_split(a), fx_split(b));
-  return fx_val(s);
-}
+__device__ __forceinline__ void fx_prod(FxSum& s, long long a, long long b) { fx_sum_mac(s, fx_split(a), fx_split(b)); }
 __device__ __forceinline__ void fx_grad_acc(FxG& g, const FxPR& p, long long Zc, long long Zo, bool im, int herm) {
   // Im A = Zy Rx - Zx Ry
   const long long Zs = im ? -Zo : Zo;
   if (herm == 0) {
-    g.ar += fx_prod(Zc, p.r);
-    g.ai += fx_prod(Zs, p.r);
-    g.br += fx_prod(Zc, p.p);
-    g.bi += fx_prod(Zs, p.p);
+    fx_prod(g.ar, Zc, p.r);
+    fx_prod(g.ai, Zs, p.r);
+    fx_prod(g.br, Zc, p.p);
+    fx_prod(g.bi, Zs, p.p);
   } else if (herm == 1) {
     // the element and its mirror add A - conj(B) to the g_a sum
-    g.ar += fx_prod(Zc, p.r - p.p);
-    g.ai += fx_prod(Zs, p.r + p.p);
+    fx_prod(g.ar, Zc, p.r - p.p);
+    fx_prod(g.ai, Zs, p.r + p.p);
   } else {
-    g.ar += fx_prod(Zc, p.r);
-    g.ai += fx_prod(Zs, p.r);
+    fx_prod(g.ar, Zc, p.r);
+    fx_prod(g.ai, Zs, p.r);
   }
 }
 
 // Gradient pieces of one step (eq. reducedgradient): per subsystem A = sum Z
 // conj(R) and B = sum Z conj(P) of zhat (scaled 2^-kc and by both scales).
-// The warps' exact sums go to shared memory; fx_grad_store adds them after
+// The warps' sums go to shared memory; fx_grad_store adds them after
 // the next barrier.  Z0: the lane's element of the stage vector (QT > 0).
 template <int E, int QT>
 __device__ __forceinline__ void fx_grad(const FxState<E, QT>& st, const FxSmem& S, const Fx* __restrict__ zh,
@@ -77,7 +80,7 @@ __device__ __forceinline__ void fx_grad(const FxState<E, QT>& st, const FxSmem& 
 #pragma unroll
     for (int q = 0; q < QT; ++q)
       if (q < st.pl.nq) {
-        FxG g{0, 0, 0, 0};
+        FxG g{};
         if (st.v[0] < V) {
           const FxPR p = fx_pr(ldb(zh, st.pl.o[q][0]), ldb(zh, st.pl.o[q][1]), ldb(zh, st.pl.o[q][2]),
                                ldb(zh, st.pl.o[q][3]), st.pl.c[q][0], st.pl.c[q][1], st.pl.c[q][2], st.pl.c[q][3]);
@@ -87,7 +90,7 @@ __device__ __forceinline__ void fx_grad(const FxState<E, QT>& st, const FxSmem& 
       }
   } else {
     for (int q = 0; q < Q; ++q) {
-      FxG g{0, 0, 0, 0};
+      FxG g{};
       const FxSub b = S.sub[q];
       const int sh = (b.n_sh >> 8) & 0xff, s = b.s, sN = s * H.N, dm = H.dm;
       const int4 *ck = S.ck + b.co, *cl = S.cl + b.co;
@@ -115,15 +118,24 @@ __device__ __forceinline__ void fx_grad_store(const FxSmem& S, const ProbDev& P,
   const bool flip = H.herm && c == 2;
   if (H.herm) c &= 1;
   const int* w = S.gred + (step & 1) * (4 * Q * kFxWarps * 3) + (q * 4 + c) * (kFxWarps * 3);
-  long long lo = 0, hi = 0;
+  unsigned long long a = 0, b = 0;
+  long long hi = 0;
   for (int i = 0; i < nwarps; ++i) {
-    lo += (long long)w[3 * i] + ((long long)w[3 * i + 1] << 24);
+    a += (unsigned)w[3 * i];
+    b += (unsigned)w[3 * i + 1];
     hi += w[3 * i + 2];
   }
-  // the sum is hi 2^48 + lo
-  hi += lo >> 48;
-  lo &= (1LL << 48) - 1;
-  double t = scalbn(fma((double)hi, 281474976710656.0, (double)lo), P.kc[q] - ssum);
+  // the sum is hi 2^64 + lo in units of 2^-24
+  b += a >> 32;
+  hi += (long long)(b >> 32);
+  unsigned long long lo = b << 32 | (a & 0xffffffffull);
+  const bool neg = hi < 0;
+  if (neg) {
+    lo = 0ull - lo;
+    hi = ~hi + (lo == 0);
+  }
+  double t = scalbn(fma((double)hi, 18446744073709551616.0, (double)lo), P.kc[q] - ssum - 24);
+  if (neg) t = -t;
   if (flip) t = -t;
   double* o = reinterpret_cast<double*>(g + q * 2);
   const int d = threadIdx.x & 3;

@@ -744,22 +744,12 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
 // Gradient pieces of one step over a block's chunk (eq. reducedgradient),
 // kGxQP subsystems from q0 per pass: per subsystem A = sum Z conj(R), B = sum
 // Z conj(P) of zhat, scaled by 2^-kc and both states' scales.  Everything is
-// summed in integers -- each product's value in two halves, so that any number
-// of elements fits, every state's sums brought to the smallest scale eref -- and
+// summed in 128-bit integers -- each product to 32 bits below its cut at 2^64
+// (FxSum, lb_fixed.cuh), every state's sums brought to the smallest scale eref -- and
 // added over the blocks by 64-bit integer atomics: exact, whatever their order.
 // (Summed in FP64 and over the blocks by block 0, these sums took 55 us of
 // an adjoint step of three states of vec 65536, the elements' products 12.)
 constexpr int kGxQP = 3;
-__device__ __forceinline__ void gx_addsum(long long& hi, long long& lo, long long h, long long l, int s) {
-  if (s) {
-    // (h 2^32 + l) >> s, rounded
-    const __int128 v = (((__int128)h << 32) + l + (((__int128)1 << s) >> 1)) >> s;
-    h = (long long)(v >> 32);
-    l = (long long)((unsigned long long)v & 0xffffffffull);
-  }
-  hi += h;
-  lo += l;
-}
 template <bool PK>
 __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, const GxSmem& S, long long e0,
                                         long long e1, const int4* __restrict__ zh, const double2* __restrict__ tape,
@@ -768,19 +758,20 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
   const GridHdr& G = *S.g;
   const int N = G.h.N;
   constexpr int NS = PK ? 2 : 4;  // sums per subsystem
-  long long hi[kGxQP][NS], lo[kGxQP][NS], th[kGxQP][NS], tl[kGxQP][NS];
+  // the current state's sums and, at the scale eref, those of the states before
+  __int128 cs[kGxQP][NS], ts[kGxQP][NS];
 #pragma unroll
   for (int u = 0; u < kGxQP; ++u)
 #pragma unroll
-    for (int c = 0; c < NS; ++c) hi[u][c] = lo[u][c] = th[u][c] = tl[u][c] = 0;
+    for (int c = 0; c < NS; ++c) cs[u][c] = ts[u][c] = 0;
   auto leave = [&](int b) {
-    const int s = min(zsc[(size_t)b * 2 * G.h.NT] + S.sc[b] - eref, 100);
+    const int s = min(zsc[(size_t)b * 2 * G.h.NT] + S.sc[b] - eref, 120);
 #pragma unroll
     for (int u = 0; u < kGxQP; ++u)
 #pragma unroll
       for (int c = 0; c < NS; ++c) {
-        gx_addsum(th[u][c], tl[u][c], hi[u][c], lo[u][c], s);
-        hi[u][c] = lo[u][c] = 0;
+        ts[u][c] += s ? (cs[u][c] + (((__int128)1 << s) >> 1)) >> s : cs[u][c];
+        cs[u][c] = 0;
       }
   };
   int bcur = -1;
@@ -794,13 +785,11 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
     const uint32_t kd = __ldg(P.digits + g.k), ld = __ldg(P.digits + g.l);
     const Cx Z = gx_ld(tape + ((size_t)g.b * tslabs + trow) * G.Vh + g.i);
     const Fx zx = fx_split(Z.x), zy = fx_split(Z.y), nzx = fx_split(-Z.x);
-    auto add = [&](long long& h, long long& l, Fx a, long long x, Fx b, long long y) {
-      FxAcc s = fx_acc();
-      fx_mac(s, a, fx_split(x));
-      fx_mac(s, b, fx_split(y));
-      const Fx v = fx_split(fx_val(s));
-      h += v.h;
-      l += v.l;
+    auto add = [&](__int128& t, Fx a, long long x, Fx b, long long y) {
+      FxSum v{0, 0u};
+      fx_sum_mac(v, a, fx_split(x));
+      fx_sum_mac(v, b, fx_split(y));
+      t += ((__int128)v.hi << 32) | v.lo;
     };
 #pragma unroll
     for (int u = 0; u < kGxQP; ++u)
@@ -808,16 +797,16 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
         const GxSub& b = gp.sub[q0 + u];
         const GxPR p = gx_pr<PK>(zh + base, b, S.cc, g.i, g.k, g.l, N, (kd >> b.sh) & gp.dm, (ld >> b.sh) & gp.dm);
         if constexpr (!PK) {
-          add(hi[u][0], lo[u][0], zx, p.rr, zy, p.ri);
-          add(hi[u][1], lo[u][1], zy, p.rr, nzx, p.ri);
-          add(hi[u][2], lo[u][2], zx, p.pr, zy, p.pi);
-          add(hi[u][3], lo[u][3], zy, p.pr, nzx, p.pi);
+          add(cs[u][0], zx, p.rr, zy, p.ri);
+          add(cs[u][1], zy, p.rr, nzx, p.ri);
+          add(cs[u][2], zx, p.pr, zy, p.pi);
+          add(cs[u][3], zy, p.pr, nzx, p.pi);
         } else {
           // Hermitian Z and zhat: an off-diagonal element and its mirror add
           // A - conj(B) to the g_a sum, a diagonal one A
           const bool od = g.vm >= 0;
-          add(hi[u][0], lo[u][0], zx, od ? p.rr - p.pr : p.rr, zy, od ? p.ri - p.pi : p.ri);
-          add(hi[u][1], lo[u][1], zy, od ? p.rr + p.pr : p.rr, nzx, od ? p.ri + p.pi : p.ri);
+          add(cs[u][0], zx, od ? p.rr - p.pr : p.rr, zy, od ? p.ri - p.pi : p.ri);
+          add(cs[u][1], zy, od ? p.rr + p.pr : p.rr, nzx, od ? p.ri + p.pi : p.ri);
         }
       }
   }
@@ -828,15 +817,17 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
   for (int u = 0; u < kGxQP; ++u)
 #pragma unroll
     for (int c = 0; c < NS; ++c) {
-      // in limbs of 24, 24 and the rest of the bits: exact in 32-bit warp sums
-      const long long h = th[u][c] + (tl[u][c] >> 32);
-      const unsigned l = (unsigned)tl[u][c];
-      const int r0 = __reduce_add_sync(kFull, (int)(l & 0xffffffu));
-      const int r1 = __reduce_add_sync(kFull, (int)((l >> 24) | (((unsigned)h & 0xffffu) << 8)));
-      const int r2 = __reduce_add_sync(kFull, (int)(h >> 16));
+      // in limbs of 27, 27, 27 and the rest of the bits: exact in 32-bit warp sums
+      const unsigned long long l = (unsigned long long)ts[u][c];
+      const long long h = (long long)(ts[u][c] >> 64);
+      const unsigned r0 = __reduce_add_sync(kFull, (unsigned)l & 0x7ffffffu);
+      const unsigned r1 = __reduce_add_sync(kFull, (unsigned)(l >> 27) & 0x7ffffffu);
+      const unsigned r2 = __reduce_add_sync(kFull, (unsigned)(l >> 54 | (unsigned long long)h << 10) & 0x7ffffffu);
+      const int r3 = __reduce_add_sync(kFull, (int)(h >> 17));
       if (lane == 0) {
-        // value = sum r0 + r1 2^24 + r2 2^48
-        S.gs[(u * 4 + c) * kGxWarps + warp] = make_longlong2((long long)r0 + ((long long)r1 << 24), r2);
+        // value = r0 + r1 2^27 + (r2 + r3 2^27) 2^54
+        S.gs[(u * 4 + c) * kGxWarps + warp] = make_longlong2((long long)r0 + ((long long)r1 << 27),
+                                                             (long long)r2 + (long long)r3 * (1LL << 27));
       }
     }
   __syncthreads();
@@ -849,9 +840,9 @@ __device__ __forceinline__ void gx_grad(const ProbDev& P, const GxParams& gp, co
         a += v.x;
         b += v.y;
       }
-      // 48 bits in the low part: the blocks' low parts add up without overflow
-      b += a >> 48;
-      a &= (1LL << 48) - 1;
+      // 54 bits in the low part: the low parts of up to 512 blocks add up without overflow
+      b += a >> 54;
+      a &= (1LL << 54) - 1;
       atomicAdd(acc + ((q0 + u) * 4 + c) * 2, (unsigned long long)a);
       atomicAdd(acc + ((q0 + u) * 4 + c) * 2 + 1, (unsigned long long)b);
     }
@@ -1034,9 +1025,9 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
         const bool flip = G.herm && c == 2;
         if (G.herm) c &= 1;
         long long lo = (long long)__ldcg(acc + (q * 4 + c) * 2), hi = (long long)__ldcg(acc + (q * 4 + c) * 2 + 1);
-        hi += lo >> 48;
-        lo &= (1LL << 48) - 1;
-        double t = scalbn(fma((double)hi, 281474976710656.0, (double)lo), 64 - eref + P.kc[q]);
+        hi += lo >> 54;
+        lo &= (1LL << 54) - 1;
+        double t = scalbn(fma((double)hi, 18014398509481984.0, (double)lo), 32 - eref + P.kc[q]);
         if (flip) t = -t;
         double* gg = reinterpret_cast<double*>(P.gproj + ((size_t)j * H.Q + q) * 2);
         const int d = threadIdx.x & 3;
@@ -1210,6 +1201,7 @@ const void* backward_kernel(int Q) {
 // Blocks of a launch: all the device holds at once, but no more than give each
 // kGxMinElems elements (a barrier costs with every block that arrives).
 constexpr int kGxMinElems = 64;
+constexpr int kGxMaxBlocks = 512;  // gx_grad's sums over the blocks
 cudaError_t gx_launch(const void* k, long long elements, size_t smem, void** args, cudaStream_t s) {
   int dev = 0, nsm = 0, per = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1220,7 +1212,7 @@ cudaError_t gx_launch(const void* k, long long elements, size_t smem, void** arg
   long long n = (long long)nsm * per;
   const long long few = (elements + kGxMinElems - 1) / kGxMinElems;
   if (n > few) n = few;
-  if (n > kMaxGridBlocks) n = kMaxGridBlocks;
+  if (n > kGxMaxBlocks) n = kGxMaxBlocks;
   return cudaLaunchCooperativeKernel(k, dim3((unsigned)n), dim3(kGridThreads), args, smem, s);
 }
 

@@ -6,14 +6,19 @@ Tolerances: the method's accuracy targets against the oracle (states and
 objective 1e-10, gradient 1e-9 of the largest entry) unless a test derives its
 own."""
 
-import copy
-import ctypes
+import importlib
+import os
+import random
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
 
 import workloads as W
 from oracle import imr, model
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 torch = pytest.importorskip("torch")
 gpu = pytest.mark.gpu
@@ -150,3 +155,152 @@ def test_a_tolerance_below_the_resolution(L, levels, n_steps, sweep):
     Go, go, _ = imr.gradient(p)
     assert abs(G - Go) <= 1e-10 * abs(Go)
     assert _rel(g, go) < 1e-9
+
+
+HARNESS = r"""
+#include <cstdio>
+#include "lb_fixed.cuh"
+int main() {
+  long long a, x, b, y;
+  while (std::scanf("%lld %lld %lld %lld", &a, &x, &b, &y) == 4) {
+    lbk::FxSum s{0, 0u};
+    lbk::fx_sum_mac(s, lbk::fx_split(a), lbk::fx_split(x));
+    lbk::fx_sum_mac(s, lbk::fx_split(b), lbk::fx_split(y));
+    std::printf("%lld %u\n", s.hi, s.lo);
+  }
+  return 0;
+}
+"""
+
+
+def test_sums_of_products_keep_32_bits_below_the_cut(tmp_path):
+    """Each product is whole but for its last 32 bits (rounded down)."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    B = importlib.import_module("paper_2110_10310_gb300.build")
+    src, exe = tmp_path / "h.cu", str(tmp_path / "h")
+    src.write_text(HARNESS)
+    r = subprocess.run([nvcc, "-std=c++17", "-O2", "-I", B.CSRC, "-o", exe, str(src)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    rng = random.Random(6)
+    top = 1 << 61
+    cases = [(top, -top, top, top - 1), (-1, 1, 0, 5), (-top, -top, -top, -top), (2**31, 2**31, -2**31, 2**31 - 1)]
+    for _ in range(2000):
+        cases.append(tuple(rng.randrange(-top, top) >> rng.randrange(0, 60) for _ in range(4)))
+    inp = "\n".join(" ".join(str(v) for v in c) for c in cases)
+    out = subprocess.run([exe], input=inp, capture_output=True, text=True, timeout=60).stdout.split("\n")
+    for (a, x, b, y), line in zip(cases, out):
+        hi, lo = (int(v) for v in line.split())
+        assert 0 <= a * x + b * y - ((hi << 32) + lo) * 2**32 < 2 * 2**32
+
+
+def _long_gradient(p):
+    """G's pieces and the gradient of one state in extended precision (numpy's
+    longdouble): the matrix form, each stage by the Jacobi iteration."""
+    ld, cld = np.longdouble, np.clongdouble
+    m = model.Model(p.system, p.controls)
+    lev, Q, N = p.system.levels, len(p.system.levels), m.N
+    NT, h = p.system.n_steps, ld(p.system.T_ns / p.system.n_steps)
+    dig = np.stack(np.unravel_index(np.arange(N), lev))
+    num = [d.astype(ld) for d in dig]
+    st = [int(np.prod(lev[q + 1:])) for q in range(Q)]
+    # row k of a X is sqrt(n_q + 1) times row k + st of X; of a^+ X sqrt(n_q) times row k - st
+    up = [np.where(dig[q] + 1 < lev[q], np.sqrt(num[q] + 1), ld(0)) for q in range(Q)]
+    dn = [np.sqrt(num[q]) for q in range(Q)]
+
+    def left(X, q, dag):
+        return dn[q][:, None] * np.roll(X, st[q], 0) if dag else up[q][:, None] * np.roll(X, -st[q], 0)
+
+    def right(X, q, dag):
+        return np.roll(X, -st[q], 1) * up[q] if dag else np.roll(X, st[q], 1) * dn[q]
+
+    def comm(X, q):
+        return left(X, q, False) - right(X, q, False), left(X, q, True) - right(X, q, True)
+
+    one = np.ones((N, N), dtype=ld)
+    E = sum(ld(2 * np.pi * p.system.detuning_ghz[q]) * num[q]
+            - ld(np.pi * p.system.selfkerr_ghz[q]) * num[q] * (num[q] - 1) for q in range(Q))
+    for q in range(Q):
+        for r in range(q):
+            E = E - ld(2 * np.pi * p.system.crosskerr_ghz[r, q]) * num[r] * num[q]
+    g1 = [ld(1.0 / (1000.0 * t)) for t in p.system.t1_us]
+    g2 = [ld(1.0 / (1000.0 * t)) for t in p.system.t2_us]
+    D = (-1j * (E[:, None] - E[None, :])).astype(cld)
+    for q in range(Q):
+        d = num[q][:, None] - num[q][None, :]
+        D = D - (g2[q] * d * d + g1[q] * (num[q][:, None] + num[q][None, :])) / 2 * one
+    t = [m.t_half(j) for j in range(NT)]
+    amp = np.array([model.control_amplitudes(p.controls, x, p.system.T_ns) for x in t])
+
+    def off(X, j, adj):
+        Y = np.zeros_like(X)
+        for q in range(Q):
+            P, R = comm(X, q)
+            Y = Y + (1j if adj else -1j) * (cld(amp[j][q]) * P + cld(np.conj(amp[j][q])) * R)
+            Y = Y + g1[q] * right(left(X, q, adj), q, not adj)
+        return Y
+
+    def stage(x, j, adj):
+        d = D.conj() if adj else D
+        inv = 1 / (1 - h / 2 * d)
+        z = inv * x
+        for _ in range(60):
+            z, old = inv * (x + h / 2 * off(z, j, adj)), z
+            if np.abs(z - old).max() <= ld(1e-22) * np.abs(x).max():
+                break
+        return z
+
+    rho, zs = p.rho0[0].astype(cld), []
+    for j in range(NT):
+        zs.append(stage(rho, j, False))
+        rho = 2 * zs[-1] - rho
+    lam = rho - p.targets[0].astype(cld)
+    lmax = float(np.abs(lam).max())
+    grad = np.zeros(p.controls.n_params, dtype=ld)
+    for j in range(NT - 1, -1, -1):
+        zh = stage(lam, j, True)
+        lam = 2 * zh - lam
+        for q in range(Q):
+            P, R = comm(zs[j], q)
+            pr = np.real((zh.conj() * (-1j * (P + R))).sum()), np.real((zh.conj() * (P - R)).sum())
+            for f, om in enumerate(p.controls.carriers_ghz[q]):
+                ph = ld(2 * np.pi * om * t[j])
+                for s in range(p.controls.n_splines):
+                    S = ld(model.bspline_basis(s, t[j], p.controls.n_splines, p.system.T_ns)) * 2 * ld(np.pi) * h
+                    k = model.alpha_index(p.controls, q, f, s)
+                    grad[k] += S * (np.cos(ph) * pr[0] + np.sin(ph) * pr[1])
+                    grad[k + 1] += S * (np.cos(ph) * pr[1] - np.sin(ph) * pr[0])
+    return grad, lmax
+
+
+@gpu
+@pytest.mark.parametrize("levels,sweep,symmetry", [
+    ((4, 4), 1, 0), ((4, 4), 1, 1), ((4, 4, 4), 1, 0), ((4, 4, 4), 1, 1), ((3, 3, 3), 2, 0), ((4, 4, 4), 2, 0),
+    ((4, 4, 4), 2, 1)])
+def test_gradient_of_a_peaked_state(L, levels, sweep, symmetry):
+    """One large entry among thousands below 1e-3 in the state and in the
+    target: the gradient comes from products with the small ones.  One step,
+    solved to the format's resolution (rtol 1e-19): an entry of either stage
+    vector, or of its neighbour combinations, is off by at most 8 units of 2^-59
+    of its state's largest; each error meets the other state's entries, whose
+    magnitudes sum to below 2 of its largest one, with ladder factors of at
+    most 4 sqrt(3) in all."""
+    N = int(np.prod(levels))
+    p = W.random_problem(815, levels=levels, n_states=1, n_steps=1, T_ns=0.01, amp=0.004, ckpt_every=0)
+    rng = np.random.default_rng(816)
+
+    def peaked(k):
+        v = 1e-3 * W.random_pure_state(rng, N)
+        v[k] = 1.0
+        return W.synthetic.pure_density(v)[None]
+
+    p.rho0, p.targets, p.weights = peaked(0), peaked(N - 1), None
+    s = _sys(p, sweep=sweep, symmetry=symmetry, rtol=1e-19)
+    _, g = s.gradient()
+    _fixed(s)
+    go, lmax = _long_gradient(p)
+    unit = 2.0**-59 * lmax * 2.0 * np.pi * p.system.T_ns
+    err, tol = float(np.abs(g - go).max()), unit * 2 * 8 * 2 * 4 * np.sqrt(3.0) + 4e-16 * float(np.abs(go).max())
+    print(levels, sweep, symmetry, "error", err, "bound", tol)
+    assert err < tol
