@@ -304,3 +304,15 @@ def test_gradient_of_a_peaked_state(L, levels, sweep, symmetry):
     err, tol = float(np.abs(g - go).max()), unit * 2 * 8 * 2 * 4 * np.sqrt(3.0) + 4e-16 * float(np.abs(go).max())
     print(levels, sweep, symmetry, "error", err, "bound", tol)
     assert err < tol
+
+
+@gpu
+@pytest.mark.parametrize("sweep", [0, 1, 2])
+def test_a_cross_kerr_that_is_not_a_number_is_reported(L, sweep):
+    p = W.random_problem(817, levels=(2, 2), n_states=1, n_steps=80, T_ns=0.8, amp=0.02, ckpt_every=0)
+    p.system.crosskerr_ghz[0, 1] = np.nan
+    s = _sys(p, sweep=sweep)
+    for call in (s.forward, s.gradient):
+        with pytest.raises(L.LBError) as e:
+            call()
+        assert e.value.code in (L.LB_ENAN, L.LB_ENOTCONV)
