@@ -539,6 +539,8 @@ __device__ int gx_solve(const ProbDev& P, const GxParams& gp, const GxSmem& S, c
   return -1;
 }
 
+constexpr int kGxZeroScale = 1 << 13;  // larger than any scale of a state that is not zero
+
 __device__ __forceinline__ double gx_to(long long X, int sc) { return scalbn((double)X, -sc); }
 __device__ __forceinline__ long long gx_from(double x, int sc) { return __double2ll_rn(scalbn(x, sc)); }
 
@@ -569,7 +571,8 @@ __device__ int gx_load(const ProbDev& P, const GxSmem& S, double2* q, F&& val) {
       const unsigned h = __ldcg(slots + b);
       if (h >= 0x7ff00000u) bad = true;
       const int e = (int)(h >> 20);
-      S.sc[b] = h ? kFxTop - (e ? e - 1023 : -1022) : kFxTop;
+      // a state of zeros: above every other's, to which it is to say nothing
+      S.sc[b] = h ? kFxTop - (e ? e - 1023 : -1022) : kGxZeroScale;
     }
     bad = __any_sync(kFull, bad);
     if (threadIdx.x == 0) S.flag[0] = bad;

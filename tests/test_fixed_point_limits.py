@@ -316,3 +316,21 @@ def test_a_cross_kerr_that_is_not_a_number_is_reported(L, sweep):
         with pytest.raises(L.LBError) as e:
             call()
         assert e.value.code in (L.LB_ENAN, L.LB_ENOTCONV)
+
+
+@gpu
+@pytest.mark.parametrize("hermitian,K", [(True, 0), (False, 4)])
+def test_a_zero_adjoint_state_beside_a_small_one(L, hermitian, K):
+    """The grid sweep brings every state's gradient sums to one scale: a state
+    of weight zero must not set it.  With the other's weight 2^-40 the integers
+    are the same as with weight 1, so the gradient is 2^-40 of that one, bitwise."""
+    p = W.random_problem(819, levels=(3, 3), n_states=2, n_steps=12, T_ns=0.12, amp=0.02, hermitian=hermitian, ckpt_every=K)
+    res = []
+    for w in (1.0, 2.0**-40):
+        p.weights = np.array([w, 0.0])
+        s = _sys(p, sweep=L.LB_SWEEP_GRID)
+        res.append(s.gradient())
+        _fixed(s)
+    assert res[1][0] == res[0][0] * 2.0**-40 and np.array_equal(res[1][1], res[0][1] * 2.0**-40)
+    Go, go, _ = imr.gradient(p)
+    assert _rel(res[1][1], go) < 1e-9
