@@ -2069,7 +2069,12 @@ static std::vector<WorkItem> fx_groups(lb_batch* b, const std::vector<WorkItem>&
       N = std::max(N, s->N);
       out.push_back(keyed[e].second);
     }
-    b->fx.push_back({(int)i, (int)(e - i), lbk::fixed_config(nel, V, Q, units, nc, nj, N, units)});
+    const lbk::FixedConfig fc = lbk::fixed_config(nel, V, Q, units, nc, nj, N, units);
+    if (fc.E <= 0) {  // each fits, but not the largest tables of all with the largest state
+      b->fx.clear();
+      return {};
+    }
+    b->fx.push_back({(int)i, (int)(e - i), fc});
     i = e;
   }
   return out;

@@ -193,11 +193,13 @@ cudaError_t launch_propagate_resident(const ProbDev* d_prob, int adjoint, int64_
 
 // one-CTA-per-state sweeps in fixed point (lb_fixed.cu)
 constexpr int kFxChunkV = 128;      // largest N^2 of the chunked sweep
+constexpr size_t kFxMaxSmem = 227 * 1024;  // shared memory of one CTA
 constexpr double kFixedRho = 0.24;  // largest iteration-matrix bound rho_j they take
 struct FixedConfig {
   int threads, E, QT;  // CTA size, elements per thread (0: not applicable), units of the register plan (E = 1)
   size_t smem;
 };
+// the configuration for a launch, E == 0 when its tables do not fit one CTA.
 // nel: elements a CTA computes; units: subsystems plus Jaynes-Cummings pairs
 // (maxima over the launch's problems)
 FixedConfig fixed_config(int nel, int V, int Q, int units, int ncoef, int njcoef, int N, int cq);

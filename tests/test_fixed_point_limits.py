@@ -334,3 +334,38 @@ def test_a_zero_adjoint_state_beside_a_small_one(L, hermitian, K):
     assert res[1][0] == res[0][0] * 2.0**-40 and np.array_equal(res[1][1], res[0][1] * 2.0**-40)
     Go, go, _ = imr.gradient(p)
     assert _rel(res[1][1], go) < 1e-9
+
+
+def _mode(n_steps, levels=(64,), n_states=2, hermitian=False):
+    """One mode of many levels, its phases and decay small."""
+    p = W.random_problem(818, levels=levels, n_states=n_states, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.004,
+                         hermitian=hermitian, ckpt_every=0)
+    Q = len(levels)
+    p.system.detuning_ghz[:] = 0.01
+    p.system.selfkerr_ghz[:] = 1e-4
+    p.system.crosskerr_ghz[:] = 0.0
+    p.system.t1_us, p.system.t2_us = np.full(Q, 40.0), np.full(Q, 30.0)
+    return p
+
+
+@gpu
+@pytest.mark.parametrize("n,hermitian", [(64, False), (64, True), (60, False), (56, True), (56, False)])
+def test_one_mode_of_many_levels_in_one_cta(L, n, hermitian):
+    """Its decay tables beside the state may not fit one CTA: those calls keep
+    the FP64 sweep.  Against the Neumann iteration (FP64), alone and in a batch
+    with a system whose tables are smaller."""
+    from paper_2110_10310_gb300.system import LindbladBatch
+
+    p = _mode(4, (n,), hermitian=hermitian)
+    s = _sys(p, sweep=L.LB_SWEEP_RESIDENT)
+    G, g = s.gradient()
+    Gn, gn = _sys(p, sweep=L.LB_SWEEP_RESIDENT, solver=L.LB_SOLVER_NEUMANN).gradient()
+    assert abs(G - Gn) <= 1e-12 * abs(Gn) and _rel(g, gn) < 1e-11
+    x = torch.from_numpy(p.rho0).cuda()
+    assert _rel(s.propagate(x, 0, 4).cpu().numpy(), _sys(p, sweep=L.LB_SWEEP_GRID).propagate(x, 0, 4).cpu().numpy()) < 1e-13
+    q = _mode(4, (2, 32), hermitian=hermitian)
+    t = _sys(q, sweep=L.LB_SWEEP_RESIDENT)
+    Gq, gq = t.gradient()
+    Gb, gb = LindbladBatch([s, t]).gradient()
+    assert abs(Gb[0] - G) <= 1e-12 * abs(G) and abs(Gb[1] - Gq) <= 1e-12 * abs(Gq)
+    assert _rel(gb[:s.n_params], g) < 1e-11 and _rel(gb[s.n_params:], gq) < 1e-11
