@@ -341,20 +341,24 @@ bool fixed_possible(const lb_system* s) {
   return fixed_cfg(s, true).E > 0;
 }
 
-// Chunked sweeps (lb_fixed_chunks.cu) of the small states the cluster sweep
-// took one cluster each: with the full stage tape, at least kChunkMinSteps
-// steps, and N^2 <= 128, where N (N + 1) / 2 columns per chunk cost less than the idle
-// SMs.  A chunk starts its predictor cold, so a step takes more iterations
-// there: max_iter must leave room for a cold start at rho = 0.24.
-constexpr int kChunkMinSteps = 64, kChunkMinIter = 64;
-bool chunks_possible(const lb_system* s) {
-  return !use_grid(s) && s->V <= lbk::kFxChunkV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&
-         s->sweep != LB_SWEEP_RESIDENT && fixed_cfg(s, false).QT > 0;
-}
 // steps per chunk: the chunks of steps run at the same time, the C boundary
 // products one after another, so about the square root of the step count
 int chunk_steps(const lb_system* s) {
   return std::max(8, (int)std::lround(0.8 * std::sqrt((double)s->NT)));
+}
+// Chunked sweeps (lb_fixed_chunks.cu) of the small states the cluster sweep
+// took one cluster each: with the full stage tape, at least kChunkMinSteps
+// steps, and N^2 <= 128, where N (N + 1) / 2 columns per chunk cost less than the idle
+// SMs.  A chunk starts its predictor cold, so a step takes more iterations
+// there: max_iter must leave room for a cold start at rho = 0.24.  The
+// propagators' entries are kept to 2^-62 of the largest possible, the states to
+// 2^-60: an entry that decays by more than kChunkDecay e-folds within a
+// chunk would fall below the state's resolution, so such systems run step by step.
+constexpr int kChunkMinSteps = 64, kChunkMinIter = 64;
+constexpr double kChunkDecay = 1.0;
+bool chunks_possible(const lb_system* s) {
+  return !use_grid(s) && s->V <= lbk::kFxChunkV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&
+         chunk_steps(s) * s->h * largest_decay(s) <= kChunkDecay && s->sweep != LB_SWEEP_RESIDENT && fixed_cfg(s, false).QT > 0;
 }
 
 // Whether this call runs the fixed-point sweeps: the Jacobi iteration with

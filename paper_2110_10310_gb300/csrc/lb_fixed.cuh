@@ -191,7 +191,7 @@ __device__ __forceinline__ long long fx_from_bits(double x, int sc) {
 }
 
 // headroom of a state's scale: the largest entry is set to [2^59, 2^60) at the
-// start and the scale moved by 2 when it has left [2^58.5, 2^60)
+// start and the scale moved when it has left [2^58.5, 2^60)
 constexpr int kFxTop = 59;
 constexpr unsigned kFxHigh = 1u << (60 - 32), kFxLow = 94906266u;  // 2^26.5
 
@@ -202,6 +202,13 @@ constexpr unsigned kFxHigh = 1u << (60 - 32), kFxLow = 94906266u;  // 2^26.5
 __device__ __forceinline__ unsigned fx_stop(float fac, unsigned qtop) {
   const float t = fac * (float)qtop * 4294967296.0f;
   return t >= 4294967040.0f ? 0xffffff00u : (t >= 1.0f ? (unsigned)t : 1u);
+}
+
+// The shift that brings a state's largest entry back to [2^59, 2^60) from its
+// high word (by more than one bit at once: a decay may halve a state and more
+// each step); 0 while it lies in [2^58.5, 2^60) and for a state of zeros.
+__host__ __device__ __forceinline__ int fx_rescale_shift(unsigned qtop) {
+  return qtop < kFxHigh && (qtop >= kFxLow || qtop == 0) ? 0 : 4 - fx_clz(qtop);
 }
 
 // The shift that gives a quarter of a state its scale, from the quarter's

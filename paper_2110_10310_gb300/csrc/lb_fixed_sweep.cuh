@@ -843,8 +843,8 @@ __device__ __forceinline__ void fx_scale_by(FxState<E, QT>& st, const FxSmem& S,
 // the last right-hand side's largest magnitude (uniform over the CTA).
 template <int E, int QT>
 __device__ __forceinline__ void fx_rescale(FxState<E, QT>& st, const FxSmem& S, unsigned qtop, bool pred) {
-  if (qtop < kFxHigh && (qtop >= kFxLow || qtop == 0)) return;
-  fx_scale_by(st, S, qtop >= kFxHigh ? 1 : -1, pred);
+  const int s = fx_rescale_shift(qtop);
+  if (s) fx_scale_by(st, S, s, pred);
 }
 // q += src (FP64, each lane's component): the scale first follows the largest
 // of state, source and sum, which a source may raise by any factor in one step

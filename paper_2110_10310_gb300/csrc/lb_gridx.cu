@@ -455,11 +455,6 @@ __device__ __forceinline__ Cx gx_commit(const ProbDev& P, const GEl& g, size_t o
   return qn;
 }
 
-// per-state change of scale from a solve's largest magnitude
-__device__ __forceinline__ int gx_shift_of(unsigned qtop) {
-  return qtop >= kFxHigh ? 1 : (qtop < kFxLow && qtop ? -1 : 0);
-}
-
 // this solve's control row (all threads; visible after the next block barrier)
 template <bool ADJ>
 __device__ __forceinline__ void gx_ctl(const GxSmem& S, const ProbDev& P, int Q, int cq, int j) {
@@ -518,7 +513,7 @@ __device__ int gx_solve(const ProbDev& P, const GxParams& gp, const GxSmem& S, c
       open = __any_sync(kFull, open);
       if (!open)
         for (int b = threadIdx.x; b < M; b += 32) {
-          const int s = gx_shift_of(__ldcg(qbank + b));
+          const int s = fx_rescale_shift(__ldcg(qbank + b));
           S.sh[b] = s;
           S.sc[b] -= s;
         }

@@ -369,3 +369,38 @@ def test_one_mode_of_many_levels_in_one_cta(L, n, hermitian):
     Gb, gb = LindbladBatch([s, t]).gradient()
     assert abs(Gb[0] - G) <= 1e-12 * abs(G) and abs(Gb[1] - Gq) <= 1e-12 * abs(Gq)
     assert _rel(gb[:s.n_params], g) < 1e-11 and _rel(gb[s.n_params:], gq) < 1e-11
+
+
+@gpu
+@pytest.mark.parametrize("levels,n_steps,sweep", [((2,), 300, 1), ((2,), 300, 0), ((2, 5), 120, 1), ((2, 5), 120, 0),
+                                                  ((3, 2, 3), 80, 1), ((3,), 300, 2), ((3, 2, 2), 100, 2)])
+def test_a_coherence_that_halves_and_more_each_step(L, levels, n_steps, sweep):
+    """A dephasing first subsystem, the slowest decay of its coherences 0.4 of
+    themselves per step: hundreds of powers of ten over the run, far below
+    2^-60 within the length of a chunk.  Every solve keeps the state's own scale."""
+    p = W.random_problem(820, levels=levels, n_states=1, n_steps=n_steps, T_ns=float(n_steps), amp=0.0,
+                         hermitian=False, ckpt_every=0)
+    Q = len(levels)
+    p.system.detuning_ghz[:] = 1e-4
+    p.system.selfkerr_ghz[:] = 1e-4
+    p.system.crosskerr_ghz[:] = 0.0
+    n = levels[0] - 1
+    p.system.t1_us = np.full(Q, np.inf)
+    p.system.t2_us = np.r_[1e-3 * 0.5 * n * n / 0.85, np.full(Q - 1, np.inf)]  # decay h n^2 / (2 T2) = 0.85
+    p.controls.alpha[:] = 0.0
+    N = int(np.prod(levels))
+    p.rho0 = np.zeros((1, N, N), dtype=np.complex128)
+    p.rho0[0, 0, N - 1] = 0.3  # levels 0 and n of the first subsystem
+    p.weights = None
+    s = _sys(p, sweep=sweep)
+    _, rho = s.forward(want_states=True)
+    _fixed(s)
+    h = 1.0
+    m = _torch_model(p)
+    d = complex(m.D.reshape(N, N)[0, N - 1])
+    want = 0.3 * ((1 + 0.5 * h * d) / (1 - 0.5 * h * d)) ** n_steps
+    assert 0.0 < abs(want) < 1e-25
+    assert abs(complex(rho[0, 0, N - 1]) - want) <= 1e-12 * abs(want)
+    x = torch.from_numpy(p.rho0).cuda()
+    y = s.propagate(x, 0, n_steps, adjoint=True)
+    assert abs(complex(y[0, 0, N - 1]) - np.conj(want / 0.3) * 0.3) <= 1e-12 * abs(want)
