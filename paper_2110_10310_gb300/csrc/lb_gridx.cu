@@ -1113,10 +1113,17 @@ __global__ void __launch_bounds__(kGridThreads, kApplyBlocks)
   const int V = H.V, N = H.N;
   const double2* ct = P.ctab + (size_t)step * H.cq;
   if (threadIdx.x == 0) {
-    // the largest power of two that keeps every factor below 0.45 (decay: below 2^-ka there)
-    double m = 0.0;
-    for (int q = 0; q < gp.Q; ++q) m = fmax(m, scalbn(fmax(fabs(ct[q].x), fabs(ct[q].y)), P.kc[q]));
-    for (int i = 0; i < P.njcoef; ++i) m = fmax(m, fmax(P.jf[i], P.ja[i]));
+    // the largest power of two that keeps every factor below 0.45, and those
+    // that one sum of gx_apply takes (both control factors and a decay factor)
+    // below 0.75 together: its middle part adds each factor's high half times a
+    // low half of 2^31 and each one's low half times a high half of 2^28
+    double m = 0.0, c = 0.0, d = 0.0;
+    for (int q = 0; q < gp.Q; ++q) {
+      m = fmax(m, scalbn(fmax(fabs(ct[q].x), fabs(ct[q].y)), P.kc[q]));
+      c = fmax(c, scalbn(fabs(ct[q].x) + fabs(ct[q].y), P.kc[q]));
+    }
+    for (int i = 0; i < P.njcoef; ++i) d = fmax(d, fmax(P.jf[i], P.ja[i]));
+    m = fmax(fmax(m, d), 0.6 * (c + d));
     s_ka = m > 0.0 ? min(20, ilogb(0.45 / m)) : 20;
   }
   __syncthreads();

@@ -370,6 +370,36 @@ def test_one_mode_of_many_levels_in_one_cta(L, n, hermitian):
     assert abs(Gb[0] - G) <= 1e-12 * abs(G) and abs(Gb[1] - Gq) <= 1e-12 * abs(Gq)
     assert _rel(gb[:s.n_params], g) < 1e-11 and _rel(gb[s.n_params:], gq) < 1e-11
 
+def _torch_model(p):
+    """The operator of a problem in plain torch: perf.cases' 64-bit matrix form."""
+    from perf.cases import _Model
+
+    return _Model(p, "cuda")
+
+
+def _apply_ref(p, x, step, adj):
+    """M x and the sum of the magnitudes of its terms, entry by entry."""
+    m = _torch_model(p)
+    X = x.reshape((-1,) + tuple(m.lev) * 2)
+    y = m.off(X, step, adj) + m.diag(adj) * X
+    return y.reshape(x.shape)
+
+
+def _term_bound(p, x, step):
+    """A bound of the sum of the magnitudes of the terms of an entry of M x, per
+    vector: twice the row sums' bound times the vector's largest entry."""
+    m = _torch_model(p)
+    row = float(m.D.abs().max())
+    for q, n in enumerate(m.lev):
+        row += abs(complex(m.d[q][step])) * 2.0 * (np.sqrt(n - 1.0) + np.sqrt(n - 2.0)) + m.g1[q] * (n - 1.0)
+    return 2.0 * row * x.abs().amax(dim=(1, 2))
+
+
+def _vectors(n, N, seed=5):
+    g = torch.Generator().manual_seed(seed)
+    a = torch.randn((n, N, N), dtype=torch.complex128, generator=g)
+    return a.cuda()
+
 
 @gpu
 @pytest.mark.parametrize("levels,n_steps,sweep", [((2,), 300, 1), ((2,), 300, 0), ((2, 5), 120, 1), ((2, 5), 120, 0),
@@ -404,3 +434,20 @@ def test_a_coherence_that_halves_and_more_each_step(L, levels, n_steps, sweep):
     x = torch.from_numpy(p.rho0).cuda()
     y = s.propagate(x, 0, n_steps, adjoint=True)
     assert abs(complex(y[0, 0, N - 1]) - np.conj(want / 0.3) * 0.3) <= 1e-12 * abs(want)
+
+
+@gpu
+def test_products_where_control_and_decay_factors_are_alike(L):
+    """Drives as weak as the decay: scaled up together, the two control factors
+    and the decay factor of one sum must not pass 64 bits.  The bound is that of
+    test_large_products_match_fp64."""
+    p = _mode(3, (4, 4, 4, 4))
+    Q = 4
+    p.controls.carriers_ghz = [np.zeros(1) for _ in range(Q)]
+    # (dt/2) 2 pi |d| 2^3 (the ladder's scale) = (dt/2) 3 / T1
+    p.controls.alpha = np.full(2 * p.controls.n_splines * Q, 3.0 / 40e3 / (2.0 * np.pi * 8.0))
+    s = _sys(p, sweep=L.LB_SWEEP_GRID)
+    x = _vectors(2, 256)
+    for adj in (False, True):
+        y, ref = s.apply(x, 1, adjoint=adj), _apply_ref(p, x, 1, adj)
+        assert bool(((y - ref).abs().amax(dim=(1, 2)) <= 2.0**-50 * _term_bound(p, x, 1)).all())
