@@ -17,6 +17,7 @@
 // to the rounding of z.
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lb_grid.cuh"
 #include "lb_fixed.cuh"
@@ -60,7 +61,8 @@ __host__ __device__ inline size_t gx_smem_bytes(int ncoef, int njcoef, int M) {
          align16(sizeof(unsigned) * 4 * kGxWarps) + sizeof(longlong2) * 12 * kGxWarps + 32 + 2 * align16(sizeof(int) * M);
 }
 
-__device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, int herm) {
+// M: the states whose scales it keeps (none in the product alone)
+__device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, int herm, int M) {
   GxSmem S;
   size_t o = 0;
   auto take = [&](size_t b) {
@@ -78,8 +80,8 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
   S.flag = reinterpret_cast<int*>(take(16));
   S.due = reinterpret_cast<unsigned long long*>(take(16));
   S.passed = reinterpret_cast<int*>(S.due + 1);
-  S.sc = reinterpret_cast<int*>(take(sizeof(int) * P.M));
-  S.sh = reinterpret_cast<int*>(take(sizeof(int) * P.M));
+  S.sc = reinterpret_cast<int*>(take(sizeof(int) * M));
+  S.sh = reinterpret_cast<int*>(take(sizeof(int) * M));
   if (threadIdx.x == 0) {
     *S.due = 0;
     load_hdr(S.g->h, P);
@@ -101,7 +103,7 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
     S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 64)));
     S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 64)));
   }
-  for (int i = threadIdx.x; i < P.M; i += blockDim.x) S.sc[i] = S.sh[i] = 0;
+  for (int i = threadIdx.x; i < M; i += blockDim.x) S.sc[i] = S.sh[i] = 0;
   __syncthreads();
   return S;
 }
@@ -627,7 +629,7 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
                double2* __restrict__ x, int nstates) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
-  const GxSmem S = gx_setup(smem, P, nstates, mode == 0 ? P.herm : 0);
+  const GxSmem S = gx_setup(smem, P, nstates, mode == 0 ? P.herm : 0, P.M);
   const GridHdr& G = *S.g;
   const Hdr& H = G.h;
   const int V = H.V;
@@ -857,7 +859,7 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
     k_backward_gx(const ProbDev* __restrict__ pp, const __grid_constant__ GxParams gp) {
   extern __shared__ __align__(16) unsigned char smem[];
   const ProbDev& P = *pp;
-  const GxSmem S = gx_setup(smem, P, P.M, P.herm);
+  const GxSmem S = gx_setup(smem, P, P.M, P.herm, P.M);
   const GridHdr& G = *S.g;
   const Hdr& H = G.h;
   const int V = H.V;
@@ -1108,7 +1110,7 @@ __global__ void __launch_bounds__(kGridThreads, kApplyBlocks)
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_ka;
   const ProbDev& P = *pp;
-  const GxSmem S = gx_setup(smem, P, n_vec, 0);
+  const GxSmem S = gx_setup(smem, P, n_vec, 0, 0);
   const Hdr& H = S.g->h;
   const int V = H.V, N = H.N;
   const double2* ct = P.ctab + (size_t)step * H.cq;
@@ -1221,14 +1223,15 @@ cudaError_t gx_launch(const void* k, long long elements, size_t smem, void** arg
   return cudaLaunchCooperativeKernel(k, dim3((unsigned)n), dim3(kGridThreads), args, smem, s);
 }
 
-template <bool ADJ>
-void run_apply(int Q, unsigned blocks, size_t smem, cudaStream_t s, const ProbDev* p, const GxParams& gp, int step,
-               const double2* x, const int4* z, const unsigned* slots, double2* y, int n_vec) {
-  switch (Q) {
-    case 4: k_apply_gx<ADJ, 4><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec); break;
-    case 6: k_apply_gx<ADJ, 6><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec); break;
-    default: k_apply_gx<ADJ, 0><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec); break;
-  }
+template <bool ADJ, int QN>
+cudaError_t run_apply(unsigned blocks, size_t smem, cudaStream_t s, const ProbDev* p, const GxParams& gp, int step,
+                      const double2* x, const int4* z, const unsigned* slots, double2* y, int n_vec) {
+  // (above 48 KB for one mode of some 55 levels and more)
+  cudaError_t e =
+      cudaFuncSetAttribute(k_apply_gx<ADJ, QN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_apply_gx<ADJ, QN><<<blocks, kGridThreads, smem, s>>>(p, gp, step, x, z, slots, y, n_vec);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1252,12 +1255,16 @@ cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h, int adjoint
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)std::min<long long>(nb, (long long)nsm * kApplyBlocks);
-  const size_t smem = gx_smem_bytes(h.ncoef, h.njcoef, h.M);
-  if (adjoint)
-    run_apply<true>(h.Q, blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
-  else
-    run_apply<false>(h.Q, blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
-  return cudaGetLastError();
+  const size_t smem = gx_smem_bytes(h.ncoef, h.njcoef, 0);
+  auto run = [&](auto adj) {
+    constexpr bool ADJ = decltype(adj)::value;
+    switch (h.Q) {
+      case 4: return run_apply<ADJ, 4>(blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
+      case 6: return run_apply<ADJ, 6>(blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
+      default: return run_apply<ADJ, 0>(blocks, smem, s, d_prob, gp, (int)step, x, z, slots, y, n_vec);
+    }
+  };
+  return adjoint ? run(std::true_type{}) : run(std::false_type{});
 }
 
 cudaError_t launch_sweep_gx(const ProbDev* d_prob, const ProbDev& h, int mode, int tape, int64_t j0, int64_t j1,

@@ -451,3 +451,33 @@ def test_products_where_control_and_decay_factors_are_alike(L):
     for adj in (False, True):
         y, ref = s.apply(x, 1, adjoint=adj), _apply_ref(p, x, 1, adj)
         assert bool(((y - ref).abs().amax(dim=(1, 2)) <= 2.0**-50 * _term_bound(p, x, 1)).all())
+
+
+# edges of the product's dispatch: 2^17 elements and just below, the unrolled
+# loops (4 and 6 subsystems) and the general one, odd N, tables above 48 KB of
+# shared memory, fewer vectors than states
+@gpu
+@pytest.mark.parametrize("levels,M,n", [
+    ((4, 4, 4, 4), 2, 2), ((4, 4, 4, 4), 2, 1), ((3, 3, 3, 3, 3), 3, 3), ((3,) * 6, 1, 1), ((5, 5, 5), 9, 9),
+    ((5, 5, 5), 9, 8), ((7, 3, 7), 7, 7), ((2, 2, 56), 3, 3), ((2, 64), 8, 8)])
+@pytest.mark.parametrize("decay", [True, False])
+def test_large_products_match_fp64(L, levels, M, n, decay):
+    """FP64's and the integers' rounding of at most 2^-50 of the terms."""
+    p = _mode(3, levels, n_states=M)
+    if not decay:
+        p.system.t1_us[:] = np.inf
+    s = _sys(p, sweep=L.LB_SWEEP_GRID)
+    N = int(np.prod(levels))
+    x = _vectors(n, N)
+    x[0] *= 1e-200
+    if n > 2:
+        x[1] *= 1e150
+        x[2] = 0.0
+    for adj in (False, True):
+        y, ref = s.apply(x, 1, adjoint=adj), _apply_ref(p, x, 1, adj)
+        err = (y - ref).abs().amax(dim=(1, 2))
+        assert bool((err <= 2.0**-50 * _term_bound(p, x, 1)).all())
+    if n > 2:
+        x[2, 1, 1] = complex(float("nan"), 0.0)
+        y = s.apply(x, 1)
+        assert bool(torch.isnan(y[2]).any()) and bool(torch.isfinite(y[[0, 1]].abs()).all())
