@@ -439,8 +439,8 @@ int lb_propagate(lb_system* sys, void* stream, int32_t adjoint, int64_t j0, int6
 
 /* y = M^{j+1/2} x (adjoint = 0) or y = (M^{j+1/2})^+ x (adjoint = 1) for
  * n_vec device vectors (Appendix A, eq. mastereq_vectorized), with
- * M^{j+1/2} = M(t_j + dt/2); x and y must not overlap.  Many elements at once
- * (grid sweeps, n_vec <= M) pass through the workspace's iteration buffers. */
+ * M^{j+1/2} = M(t_j + dt/2); x and y must not overlap.  May run beside a
+ * sweep or another lb_apply of this system on another stream. */
 int lb_apply(lb_system* sys, void* stream, int32_t adjoint, int64_t step, const void* x_dev, void* y_dev,
              int32_t n_vec);
 

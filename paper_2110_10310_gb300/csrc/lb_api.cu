@@ -49,7 +49,7 @@ struct Region {
 struct Layout {
   Region prob, status, items, sysp, cu, cd, jf, ja, digits, D, Dinv, alpha, carriers, ctab, q0, tar, wgt, qT, ckpt, seg,
       gproj, gsum, sfac, pen, qb, jpen, mpart, pmap, Ginv, hgp, hgm, fgp, fgm, dfA, dfB, Dinvf, zsA, zsB, J, G, grad, gateV, emap, efull, zA, zB, lam, qf, partials, gslots, bar, hist, histf,
-      hkl, ctabx, fxs, pmat, bst, bsc, jpart, fxd, fxh, fxu, gsc;
+      hkl, ctabx, fxs, pmat, bst, bsc, jpart, fxd, fxh, fxu, gsc, apx, apm;
   size_t total = 0;
 };
 
@@ -125,6 +125,7 @@ struct lb_system {
   size_t ws_bytes = 0;
   cudaStream_t bind_stream = nullptr;
   cudaEvent_t upload_done = nullptr;
+  cudaEvent_t apply_done = nullptr;  // the last fixed-point lb_apply
   Layout L;
   ProbDev hp{};
   ProbDev* dp = nullptr;
@@ -368,16 +369,16 @@ bool use_fixed(const lb_system* s, bool herm) {
   if (use_grid(s)) return rho_bound(s) <= lbk::kGridFixedRho;
   return fixed_cfg(s, herm).E > 0 && rho_bound(s) <= lbk::kFixedRho;
 }
+bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();
+  return false;
+}
 // ... on this stream: a call recorded into a graph of the caller's may be
 // replayed with controls of any size, which no host check sees then, so it
 // records the FP64 sweeps
-bool use_fixed(const lb_system* s, bool herm, cudaStream_t st) {
-  if (!use_fixed(s, herm)) return false;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap == cudaStreamCaptureStatusNone;
-  (void)cudaGetLastError();
-  return true;
-}
+bool use_fixed(const lb_system* s, bool herm, cudaStream_t st) { return use_fixed(s, herm) && !is_capturing(st); }
 
 // ... and those in chunks: without the Hermitian element plan
 bool use_chunks(const lb_system* s) { return s->hp.chunkL > 0 && s->cluster && !s->hp.herm; }
@@ -514,6 +515,9 @@ Layout make_layout(const lb_system* s, int fixed) {
   take(L.fxh, fixed && grid ? sizeof(int4) * V : 0);
   take(L.fxu, fixed && grid ? sizeof(longlong2) * V : 0);
   take(L.gsc, fixed && grid ? sizeof(int32_t) * M : 0);
+  // lb_apply's own, not the sweeps': it may run beside one on another stream
+  take(L.apx, fixed && grid ? sizeof(int4) * M * V : 0);
+  take(L.apm, fixed && grid ? sizeof(uint32_t) * M : 0);
   const bool chunks = fixed == 2 && chunks_possible(s);
   const size_t C = chunks ? (NT + chunk_steps(s) - 1) / chunk_steps(s) : 0;
   take(L.pmat, sizeof(int4) * C * ((size_t)s->N * (s->N + 1) / 2) * V);
@@ -891,6 +895,8 @@ void fill_prob(lb_system* s) {
     P.fxh = at<int4>(s, s->L.fxh);
     P.fxu = at<longlong2>(s, s->L.fxu);
     P.gsc = at<int32_t>(s, s->L.gsc);
+    P.apx = at<int4>(s, s->L.apx);
+    P.apm = at<uint32_t>(s, s->L.apm);
   }
   if (s->fx_ws == 2 && chunks_possible(s)) {
     P.chunkL = chunk_steps(s);
@@ -1021,6 +1027,7 @@ int lb_system_create(const lb_system_desc* d, lb_system** out) {
 void lb_system_destroy(lb_system* s) {
   if (!s) return;
   if (s->upload_done) cudaEventDestroy(s->upload_done);
+  if (s->apply_done) cudaEventDestroy(s->apply_done);
   for (cudaEvent_t e : s->ev)
     if (e) cudaEventDestroy(e);
   delete s;
@@ -1932,13 +1939,18 @@ int lb_apply(lb_system* s, void* stream, int32_t adjoint, int64_t step, const vo
   if (rc) return rc;
   rc = ensure_ctab(s, st);
   if (rc) return rc;
-  // many elements: the off-diagonal part in fixed point, split into the sweeps'
-  // iterate buffer of M states (every control factor within its range)
+  // many elements: the off-diagonal part in fixed point, the vectors split into
+  // a buffer of M states (every control factor within its range); a recorded
+  // call may be replayed beside another one, which would share that buffer
   if (use_grid(s) && s->fx_ws && n_vec <= s->M && (long long)n_vec * s->V >= lbk::kApplyFixedElements &&
-      rho_bound(s) <= lbk::kFixedRho) {
+      rho_bound(s) <= lbk::kFixedRho && !is_capturing(st)) {
+    // after the last such product, whichever stream that was on
+    if (!s->apply_done) LB_CUDA(cudaEventCreateWithFlags(&s->apply_done, cudaEventDisableTiming), "cudaEventCreate");
+    LB_CUDA(cudaStreamWaitEvent(st, s->apply_done, 0), "cudaStreamWaitEvent");
     LB_CUDA(lbk::launch_apply_gx(s->dp, s->hp, adjoint, step, static_cast<const double2*>(x_dev),
                                  static_cast<double2*>(y_dev), n_vec, st),
             "apply kernels");
+    LB_CUDA(cudaEventRecord(s->apply_done, st), "cudaEventRecord");
     return LB_OK;
   }
   LB_CUDA(lbk::launch_apply(s->dp, s->hp, adjoint, step, static_cast<const double2*>(x_dev), static_cast<double2*>(y_dev),

@@ -1070,7 +1070,7 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
 // ---------------------------------------------------------------------------
 // y = M x on many elements (lb_apply): the off-diagonal part on the integer pipe.
 // The vectors are split once (k_apply_split, scaled by each one's largest entry)
-// into the sweeps' iterate buffer; the control factors are scaled up by a
+// into a buffer of the product's own; the control factors are scaled up by a
 // common 2^ka so that the small sums keep 2^-60 of the largest entry times
 // 2^-ka.  The diagonal and the result are FP64.
 
@@ -1239,8 +1239,8 @@ cudaError_t run_apply(unsigned blocks, size_t smem, cudaStream_t s, const ProbDe
 cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h, int adjoint, int64_t step, const double2* x,
                             double2* y, int n_vec, cudaStream_t s) {
   const GxParams gp = gx_params(h);
-  unsigned* slots = reinterpret_cast<unsigned*>(h.gslots);
-  int4* z = reinterpret_cast<int4*>(h.zA);
+  unsigned* slots = h.apm;
+  int4* z = h.apx;
   cudaError_t e = cudaMemsetAsync(slots, 0, sizeof(unsigned) * n_vec, s);
   if (e != cudaSuccess) return e;
   const unsigned bx = (unsigned)((h.V + 8 * 256 - 1) / (8 * 256));

@@ -133,6 +133,8 @@ struct ProbDev {
   int4* fxh;                 // [V] dt/2 D, split
   longlong2* fxu;            // [V] the frame's factor per step, a quarter of the unit-modulus part of g
   int32_t* gsc;              // [M] the adjoint states' scales during a recompute
+  int4* apx;                 // [M][V] lb_apply: the vectors, split
+  uint32_t* apm;             // [M] ... their largest magnitudes
   int4* ctabx;               // [NT][cq + 1] the rows of ctab split for them, last the stopping factor and range flag
   int32_t* fxs;              // [M][2 NT] scales of the stage vectors and the checkpoints
   float4* zsA;               // [M*V] the iterates zA / zB split into single-precision pairs (x_hi, x_lo, y_hi, y_lo)

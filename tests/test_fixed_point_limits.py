@@ -481,3 +481,49 @@ def test_large_products_match_fp64(L, levels, M, n, decay):
         x[2, 1, 1] = complex(float("nan"), 0.0)
         y = s.apply(x, 1)
         assert bool(torch.isnan(y[2]).any()) and bool(torch.isfinite(y[[0, 1]].abs()).all())
+
+
+@gpu
+def test_products_beside_a_gradient_and_each_other_on_other_streams(L):
+    """Products on two streams while a gradient runs on a third: all as alone."""
+    p = W.prefix(W.config4(n_states=3), 60)
+    s = _sys(p)
+    x, x2 = _vectors(3, 256, 6), _vectors(3, 256, 7)
+    G, g = s.gradient()
+    _fixed(s)
+    y, y2 = s.apply(x, 7), s.apply(x2, 9)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    Gd = torch.zeros(1, dtype=torch.float64, device="cuda")
+    gd = torch.zeros(s.n_params, dtype=torch.float64, device="cuda")
+    bufs = [t.transpose(1, 2).contiguous() for t in (x, x2)]
+    outs = [[torch.zeros_like(b) for _ in range(6)] for b in bufs]
+    torch.cuda.synchronize()
+    s.gradient_async(Gd, gd, stream=streams[0])
+    for k in range(6):
+        for i in range(2):
+            L.check(s.lib.lb_apply(s.h, streams[1 + i].cuda_stream, 0, (7, 9)[i], bufs[i].data_ptr(),
+                                   outs[i][k].data_ptr(), 3))
+    torch.cuda.synchronize()
+    assert float(Gd) == G and np.array_equal(gd.cpu().numpy(), g)
+    for i, want in enumerate((y, y2)):
+        for o in outs[i]:
+            assert torch.equal(o.transpose(1, 2), want)
+
+
+@gpu
+def test_a_recorded_product_is_replayed(L):
+    """Recorded, the product is FP64 (its own buffer would be shared by replays)."""
+    p = W.prefix(W.config4(n_states=3), 20)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        s = _sys(p)
+        x = _vectors(3, 256, 6).transpose(1, 2).contiguous()
+        y, z = torch.zeros_like(x), torch.zeros_like(x)
+        L.check(s.lib.lb_apply(s.h, st.cuda_stream, 0, 7, x.data_ptr(), y.data_ptr(), 3))
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            L.check(s.lib.lb_apply(s.h, st.cuda_stream, 0, 7, x.data_ptr(), z.data_ptr(), 3))
+        graph.replay()
+        torch.cuda.synchronize()
+    assert _rel(z.cpu().numpy(), y.cpu().numpy()) < 1e-14
