@@ -320,8 +320,9 @@ int lb_set_wait_limit(lb_system* sys, int64_t polls);
  * bind stream, which is synchronised. */
 int lb_set_difference_iterations(lb_system* sys, int32_t on);
 
-/* Arithmetic of the grid sweeps' FP64 inner iterations (the first of every
- * step and any before the difference iterations take over).
+/* Arithmetic of the FP64 grid sweeps' inner iterations (the first of every
+ * step and any before the difference iterations take over); calls that run in
+ * fixed point (LB_ARITH_FIXED) are the same for both values.
  *   LB_PREC_F64 (default): the off-diagonal apply c = (dt/2) O z in FP64.
  *   LB_PREC_F32X2: the apply in pairs of single-precision numbers (hi + lo,
  *     about 48 significant bits): every iterate is also stored split into
@@ -341,6 +342,12 @@ int lb_set_difference_iterations(lb_system* sys, int32_t on);
 #define LB_PREC_F64 0
 #define LB_PREC_F32X2 1
 int lb_set_precision(lb_system* sys, int32_t precision);
+
+/* LB_ARITH_FIXED (default): fixed point where it applies (see LB_ARITH_*);
+ * LB_ARITH_F64: the FP64 sweeps always, whose products of small entries keep
+ * their own 53 bits.  lb_get_stats reports what a call ran in.  Call before
+ * lb_workspace_bytes. */
+int lb_set_arithmetic(lb_system* sys, int32_t arithmetic);
 
 /* Jaynes-Cummings coupling of the system Hamiltonian (Sec. II):
  *   sum_{p<q} g_pq (e^{i eta_pq t} a_p^+ a_q + e^{-i eta_pq t} a_p a_q^+),

@@ -108,6 +108,7 @@ struct lb_system {
   long long spin_limit = 0;  // polls of a grid-barrier wait (0: the kernels' default; lb_set_wait_limit)
   int diffit = 1;            // single-precision difference iterations in the grid sweeps (lb_set_difference_iterations)
   int precision = LB_PREC_F64;  // arithmetic of the grid sweeps' FP64 iterations (lb_set_precision)
+  int arith = LB_ARITH_FIXED;  // the sweeps' arithmetic within its range (lb_set_arithmetic)
   double gamma1 = 0.0, pen_a = 1.0;  // running penalty (one CTA per state)
   bool rho_herm = false;  // every initial state exactly Hermitian
   bool tar_herm = false;  // every explicit target exactly Hermitian (gate targets: always)
@@ -337,7 +338,7 @@ int fixed_forward_pred(const lb_system* s) { return !(s->cluster && effective_K(
 
 // whether the workspace should hold the fixed-point sweeps' tables
 bool fixed_possible(const lb_system* s) {
-  if (s->method != LB_SOLVER_JACOBI || !fixed_phase_ok(s)) return false;
+  if (s->arith == LB_ARITH_F64 || s->method != LB_SOLVER_JACOBI || !fixed_phase_ok(s)) return false;
   if (use_grid(s)) return gridx_possible(s);
   return fixed_cfg(s, true).E > 0;
 }
@@ -1454,6 +1455,14 @@ int lb_set_precision(lb_system* s, int32_t precision) {
   if (s->ws) return fail(LB_EINVAL, "choose the precision before binding a workspace");
   if (precision != LB_PREC_F64 && precision != LB_PREC_F32X2) return fail(LB_EINVAL, "unknown precision");
   s->precision = precision;
+  return LB_OK;
+}
+
+int lb_set_arithmetic(lb_system* s, int32_t arithmetic) {
+  if (!s) return fail(LB_EINVAL, "null system handle");
+  if (s->ws) return fail(LB_EINVAL, "choose the arithmetic before binding a workspace");
+  if (arithmetic != LB_ARITH_F64 && arithmetic != LB_ARITH_FIXED) return fail(LB_EINVAL, "unknown arithmetic");
+  s->arith = arithmetic;
   return LB_OK;
 }
 

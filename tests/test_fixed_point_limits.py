@@ -527,3 +527,32 @@ def test_a_recorded_product_is_replayed(L):
         graph.replay()
         torch.cuda.synchronize()
     assert _rel(z.cpu().numpy(), y.cpu().numpy()) < 1e-14
+
+
+@gpu
+@pytest.mark.parametrize("levels,sweep", [((3, 3), 0), ((3, 3), 1), ((3, 2, 3), 1), ((3, 3), 2), ((4, 4, 4), 2)])
+def test_fp64_sweeps_on_request(L, levels, sweep):
+    """The FP64 Jacobi sweeps at full length beside the fixed-point ones."""
+    p = W.random_problem(822, levels=levels, n_states=2, n_steps=150, T_ns=1.5, amp=0.02, ckpt_every=0)
+    s, f = _sys(p, sweep=sweep), _sys(p, sweep=sweep, arithmetic=L.LB_ARITH_F64)
+    G, g = _fixed_after(s)
+    Gf, gf = f.gradient()
+    assert f.stats()["arithmetic"] == "f64" and f.workspace_bytes <= s.workspace_bytes
+    assert abs(G - Gf) <= 1e-12 * abs(Gf) and _rel(g, gf) < 1e-11
+    with pytest.raises(L.LBError):
+        L.check(f.lib.lb_set_arithmetic(f.h, L.LB_ARITH_FIXED))  # a workspace is bound
+
+
+def _fixed_after(s):
+    r = s.gradient()
+    _fixed(s)
+    return r
+
+
+def test_arithmetic_values():
+    from paper_2110_10310_gb300 import _lib as L
+
+    if not os.path.exists(L.lib_path()):
+        pytest.skip("library not built")
+    lib = L.load()
+    assert lib.lb_set_arithmetic(None, L.LB_ARITH_F64) == L.LB_EINVAL
