@@ -327,6 +327,10 @@ __global__ void __launch_bounds__(T)
         const double sr = st.v[0] < V ? source(0) : 0.0;
         const unsigned long long mx = fx_cta_max(S, abs_bits(sr));
         if (j > j0) fx_ctl(S, P, H.cq, j - 1, cnt.step);
+        if (mx >= kInfBits && j > 0) {
+          if (threadIdx.x == 0) record_error(P.status, LB_ENAN, j - 1);
+          return;
+        }
         if (mx == 0 || mx >= kInfBits) continue;
         st.sc = fx_scale(mx);
         st.q[0] = fx_from(sr, st.sc);
@@ -358,7 +362,12 @@ __global__ void __launch_bounds__(T)
         double src[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) src[e] = fx_v(st, S, H, e) < V ? source(e) : 0.0;
-        fx_add_source(st, S, src, true);
+        // (the state before step 0 is not used)
+        if (!fx_add_source(st, S, src, true) && j > 0) {
+          if (threadIdx.x == 0) record_error(P.status, LB_ENAN, j - 1);
+          stats.flush(P.status);
+          return;
+        }
       } else {
         fx_rescale(st, S, qtop, true);
       }

@@ -849,9 +849,9 @@ __device__ __forceinline__ void fx_rescale(FxState<E, QT>& st, const FxSmem& S, 
 // q += src (FP64, each lane's component): the scale first follows the largest
 // of state, source and sum, which a source may raise by any factor in one step
 // (of the sum alone it would shift a state that the source cancels past 64
-// bits) (all threads)
+// bits) (all threads).  False when state or source is not finite.
 template <int E, int QT>
-__device__ __forceinline__ void fx_add_source(FxState<E, QT>& st, const FxSmem& S, const double (&src)[E], bool pred) {
+__device__ __forceinline__ bool fx_add_source(FxState<E, QT>& st, const FxSmem& S, const double (&src)[E], bool pred) {
   unsigned long long mx = 0;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -859,11 +859,12 @@ __device__ __forceinline__ void fx_add_source(FxState<E, QT>& st, const FxSmem& 
     mx = umax64(mx, umax64(abs_bits(x + src[e]), umax64(abs_bits(x), abs_bits(src[e]))));
   }
   mx = fx_cta_max(S, mx);
-  if (mx >= kInfBits) return;
+  if (mx >= kInfBits) return false;
   const int sc = fx_scale(mx);
   if (mx && (sc < st.sc || sc > st.sc + 1)) fx_scale_by(st, S, st.sc - sc, pred);
 #pragma unroll
   for (int e = 0; e < E; ++e) st.q[e] += fx_from(src[e], st.sc);
+  return true;
 }
 
 // q <- 2 z - q for the lane's elements, z from the solve (zr for QT > 0); the

@@ -556,3 +556,14 @@ def test_arithmetic_values():
         pytest.skip("library not built")
     lib = L.load()
     assert lib.lb_set_arithmetic(None, L.LB_ARITH_F64) == L.LB_EINVAL
+
+
+@gpu
+@pytest.mark.parametrize("n_steps,sweep", [(24, 1), (80, 0)])
+def test_a_penalty_source_that_overflows_is_reported(L, n_steps, sweep):
+    p = W.random_problem(821, levels=(2, 2), n_states=1, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.02, ckpt_every=0)
+    p.gamma1, p.penalty_a = 1.7e308, 1e-3
+    s = _sys(p, sweep=sweep)
+    with pytest.raises(L.LBError) as e:
+        s.gradient()
+    assert e.value.code == L.LB_ENAN
