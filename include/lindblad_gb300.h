@@ -466,7 +466,11 @@ int lb_get_stats(lb_system* sys, lb_stats* out);
  * (lb_get_predictor reports it).  Synchronises
  * `stream`.  choice_out (nullable, [3]) receives the chosen LB_SWEEP_*,
  * LB_SOLVER_* and the threads per CTA (resident), CTAs per cluster (cluster)
- * or blocks (grid).  LB_ENOTCONV when no candidate converges. */
+ * or blocks (grid).  Within the fixed-point sweeps' range the Jacobi iteration
+ * is one candidate, and a system of the cluster sweep then keeps that sweep
+ * (its chunks) or one CTA per state, whichever runs lb_forward faster;
+ * choice_out[2] is then the number of chunks or the threads per CTA.
+ * LB_ENOTCONV when no candidate converges. */
 int lb_autotune(lb_system* sys, void* stream, int32_t probe_steps, int32_t* choice_out);
 
 /* on != 0: record CUDA events around the sweep kernels on the launching

@@ -1035,6 +1035,34 @@ void lb_system_destroy(lb_system* s) {
 }
 
 static int propagate_impl(lb_system* s, cudaStream_t st, int adjoint, int64_t j0, int64_t j1, double2* x, int n_vec);
+static int run_forward(lb_system* s, cudaStream_t st, int tape);
+
+// The bound system's small-state sweep: cluster (with its chunks in fixed
+// point) or one CTA per state; the caller uploads s->hp.
+static void choose_cluster(lb_system* s, bool cluster) {
+  s->cluster = cluster;
+  s->hp.gM = gproj_used(s);
+  s->hp.fxfwd = fixed_forward_pred(s);
+  s->hp.herm = use_symmetry(s) ? 1 : 0;
+}
+
+// Device time of a forward call (ms; the second of two), negative when it
+// fails to converge.
+static int time_forward(lb_system* s, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, float* ms) {
+  for (int k = 0; k < 2; ++k) {
+    LB_CUDA(cudaEventRecord(e0, st), "cudaEventRecord");
+    const int rc = run_forward(s, st, 0);
+    if (rc) return rc;
+    LB_CUDA(cudaEventRecord(e1, st), "cudaEventRecord");
+  }
+  DevStatus d{};
+  LB_CUDA(cudaMemcpyAsync(&d, at<DevStatus>(s, s->L.status), sizeof(DevStatus), cudaMemcpyDeviceToHost, st),
+          "read status");
+  LB_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+  LB_CUDA(cudaEventElapsedTime(ms, e0, e1), "cudaEventElapsedTime");
+  if (d.code || d.late) *ms = -1.0f;
+  return LB_OK;
+}
 
 int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice_out) {
   int rc = check_ready(s, true);
@@ -1050,7 +1078,17 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
   // grid sweeps, GMRES runs one CTA per state
   const bool grid0 = use_grid(s);
   const int methods[3] = {LB_SOLVER_JACOBI, LB_SOLVER_NEUMANN, LB_SOLVER_GMRES};
+  // in fixed point steps on vectors run one kernel, whatever shape the FP64
+  // sweeps would take
+  const int bound_method = s->method;
+  s->method = LB_SOLVER_JACOBI;
+  const bool fixed = !grid0 && use_fixed(s, false, st);
+  s->method = bound_method;
   for (int m : methods) {
+    if (fixed && m == LB_SOLVER_JACOBI) {
+      cands.push_back({LB_SWEEP_RESIDENT, m, s->rc.E});
+      continue;
+    }
     if (grid0) {
       if (m != LB_SOLVER_GMRES) cands.push_back({LB_SWEEP_GRID, m, 0});
       continue;
@@ -1079,11 +1117,8 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
   for (const Cand& c : cands) {
     s->method = c.method;
     s->hp.method = c.method;
-    s->cluster = c.sweep == LB_SWEEP_CLUSTER;
-    if (s->cluster) s->cc = cluster_cfg(s, c.E != 0);
-    s->hp.gM = gproj_used(s);
-    s->hp.fxfwd = fixed_forward_pred(s);
-    s->hp.herm = use_symmetry(s) ? 1 : 0;
+    if (c.sweep == LB_SWEEP_CLUSTER) s->cc = cluster_cfg(s, c.E != 0);
+    choose_cluster(s, c.sweep == LB_SWEEP_CLUSTER);
     if (c.sweep == LB_SWEEP_RESIDENT) {
       s->rc = lbk::resident_config(s->V, s->Q, n_coef(s), n_jcoef(s), s->N, s->jp.empty(), kry_elems(s));
       const int threads = ((s->V + c.E - 1) / c.E + 31) / 32 * 32;
@@ -1115,26 +1150,42 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
       win = c;
     }
   }
+  const bool fixed_won = fixed && win.method == LB_SOLVER_JACOBI;
+  if (fixed_won) {
+    // the sweeps of the whole horizon: in chunks (the cluster sweep's systems)
+    // against one CTA per state, by a forward call each; a tie, or neither: as bound
+    s->rc = rc0;
+    s->cc = cc0;
+    s->method = s->hp.method = win.method;
+    win.sweep = cl0 ? LB_SWEEP_CLUSTER : LB_SWEEP_RESIDENT;
+    float ms[2] = {-1.0f, -1.0f};
+    for (int cl = 0; cl < 2 && cc0.C > 0; ++cl) {
+      choose_cluster(s, cl != 0);
+      LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
+      rc = time_forward(s, st, e0, e1, &ms[cl]);
+      if (rc) {
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        return rc;
+      }
+    }
+    if (ms[1] >= 0.0f && (ms[0] < 0.0f || ms[1] < ms[0])) win.sweep = LB_SWEEP_CLUSTER;
+    else if (ms[0] >= 0.0f && (ms[1] < 0.0f || ms[0] < ms[1])) win.sweep = LB_SWEEP_RESIDENT;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (win.sweep < 0) {
     s->rc = rc0;
-    s->cluster = cl0;
     s->cc = cc0;
     s->method = s->hp.method = m0;
-    s->hp.gM = gproj_used(s);
-    s->hp.fxfwd = fixed_forward_pred(s);
-    s->hp.herm = use_symmetry(s) ? 1 : 0;
+    choose_cluster(s, cl0);
     LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
     return fail(LB_ENOTCONV, "no candidate's inner solve converged on the probe steps");
   }
   s->method = s->hp.method = win.method;
-  s->cluster = win.sweep == LB_SWEEP_CLUSTER;
-  s->cc = s->cluster ? cluster_cfg(s, win.E != 0) : cc0;
-  s->hp.gM = gproj_used(s);
-  s->hp.fxfwd = fixed_forward_pred(s);
-  s->hp.herm = use_symmetry(s) ? 1 : 0;
-  if (win.sweep == LB_SWEEP_RESIDENT) {
+  s->cc = win.sweep == LB_SWEEP_CLUSTER && !fixed_won ? cluster_cfg(s, win.E != 0) : cc0;
+  choose_cluster(s, win.sweep == LB_SWEEP_CLUSTER);
+  if (win.sweep == LB_SWEEP_RESIDENT && !fixed_won) {
     s->rc = lbk::resident_config(s->V, s->Q, n_coef(s), n_jcoef(s), s->N, s->jp.empty(), kry_elems(s));
     s->rc.E = win.E;
     s->rc.threads = ((s->V + win.E - 1) / win.E + 31) / 32 * 32;
@@ -1189,6 +1240,8 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
     choice_out[0] = win.sweep;
     choice_out[1] = win.method;
     choice_out[2] = win.sweep == LB_SWEEP_RESIDENT ? s->rc.threads : (s->cluster ? s->cc.C : s->gblocks);
+    if (fixed_won)
+      choice_out[2] = use_chunks(s) ? s->hp.chunkC : fixed_cfg(s, s->hp.herm != 0).threads;
   }
   return LB_OK;
 }

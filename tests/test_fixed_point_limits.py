@@ -567,3 +567,24 @@ def test_a_penalty_source_that_overflows_is_reported(L, n_steps, sweep):
     with pytest.raises(L.LBError) as e:
         s.gradient()
     assert e.value.code == L.LB_ENAN
+
+
+@gpu
+@pytest.mark.parametrize("levels,n_steps,K,sweep", [((3, 3), 2000, 0, "cluster"), ((2,), 2000, 0, "cluster"),
+                                                     ((3, 3), 300, 25, "resident")])
+def test_autotune_within_the_fixed_point_range(L, levels, n_steps, K, sweep):
+    """The kernels that run are the ones timed: chunks over a long horizon; with
+    checkpoints one CTA per state, whose forward sweep predicts.  choice[2] is
+    theirs: chunks of about 0.8 sqrt(steps), or two threads per element."""
+    p = W.random_problem(823, levels=levels, n_states=2, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.01, ckpt_every=K)
+    s = _sys(p)
+    G, g = s.gradient()
+    c = s.autotune(probe_steps=20)
+    assert (c["sweep"], c["solver"]) == (sweep, "jacobi")
+    if sweep == "cluster":
+        per = round(0.8 * np.sqrt(n_steps))
+        assert c["shape"] == -(-n_steps // per)
+    else:
+        assert c["shape"] == (2 * 45 + 31) // 32 * 32
+    Gt, gt = _fixed_after(s)
+    assert abs(Gt - G) <= 1e-12 * abs(G) and _rel(gt, g) < 1e-11
