@@ -147,7 +147,8 @@ FixedConfig fixed_config(int nel, int V, int Q, int units, int ncoef, int njcoef
     if (fc.threads < 64) fc.threads = 64;  // the first 4 Q and cq + 1 threads have work of their own
   }
   fc.smem = fx_smem_bytes(ncoef, njcoef, N, V, Q, cq, fc.E * (fc.threads / 2), fc.QT);
-  // (one mode of 58 to 64 levels: its decay tables take up to 64 KB beside the state's 128)
+  // (one mode of 59 levels and more, 63 under the Hermitian symmetry: its decay
+  // tables take up to 64 KB beside the state's 128; the FP64 sweep ends at 58)
   return fc.smem <= kFxMaxSmem ? fc : FixedConfig{};
 }
 
