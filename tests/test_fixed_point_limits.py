@@ -565,7 +565,7 @@ def test_arithmetic_values():
 @pytest.mark.parametrize("n_steps,sweep", [(24, 1), (80, 0)])
 def test_a_penalty_source_that_overflows_is_reported(L, n_steps, sweep):
     p = W.random_problem(821, levels=(2, 2), n_states=1, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.02, ckpt_every=0)
-    p.gamma1, p.penalty_a = 1.7e308, 1e-3
+    p.gamma1, p.penalty_a, p.weights = 1.7e308, 0.1, np.array([1e5])
     s = _sys(p, sweep=sweep)
     with pytest.raises(L.LBError) as e:
         s.gradient()
@@ -591,3 +591,67 @@ def test_autotune_within_the_fixed_point_range(L, levels, n_steps, K, sweep):
         assert c["shape"] == (2 * 45 + 31) // 32 * 32
     Gt, gt = _fixed_after(s)
     assert abs(Gt - G) <= 1e-12 * abs(G) and _rel(gt, g) < 1e-11
+
+
+def _large(state, n_states=1):
+    """Four four-level qudits (N^2 = 65536) from and to peaked or spread matrices."""
+    p = W.prefix(W.config4(n_states=n_states), 12)
+    if state != "spread":
+        p.rho0 = np.stack([_basis((4,) * 4, 0, k) for k in range(n_states)])
+        if state == "peaked":
+            p.targets = np.stack([_basis((4,) * 4, 255, 254 - k) for k in range(n_states)])
+    return p
+
+
+@gpu
+def test_peaked_states_of_large_systems_keep_fp64(L):
+    """Entries are rounded to their state's largest: on the large grids a state
+    of one entry is served by FP64, and is its results; small systems and spread
+    states stay in fixed point.  The caller's vectors decide for lb_propagate."""
+    for state, want in (("spread", "fixed"), ("peaked", "f64"), ("from", "f64")):
+        p = _large(state)
+        s, f = _sys(p), _sys(p, arithmetic=L.LB_ARITH_F64)
+        G, g = s.gradient()
+        assert s.stats()["arithmetic"] == want
+        Gf, gf = f.gradient()
+        assert abs(G - Gf) <= 1e-12 * abs(Gf) and _rel(g, gf) < 1e-9
+        if want == "f64":
+            assert G == Gf and np.array_equal(g, gf)
+    s = _sys(_large("spread", 3))
+    x = _vectors(3, 256)
+    s.propagate(x, 0, 3)
+    assert s.stats()["arithmetic"] == "fixed"
+    x[1] = torch.from_numpy(_basis((4,) * 4, 3, 7)).cuda()
+    y = s.propagate(x, 0, 3, adjoint=True)
+    assert s.stats()["arithmetic"] == "f64"
+    f = _sys(_large("spread", 3), arithmetic=L.LB_ARITH_F64)
+    assert torch.equal(y, f.propagate(x, 0, 3, adjoint=True))
+    q = W.random_problem(824, levels=(4, 4, 4), n_states=1, n_steps=5, T_ns=0.05, amp=0.02, ckpt_every=0)
+    q.rho0 = _basis((4, 4, 4), 0, 0)[None]
+    t = _sys(q, sweep=L.LB_SWEEP_GRID)
+    t.gradient()
+    _fixed(t)
+
+
+@gpu
+def test_products_of_peaked_vectors(L):
+    """Per vector: one of spread entries, one of a single large entry among
+    entries of 1e-13, whose products keep their own 53 bits away from it."""
+    p = _large("spread", 2)
+    s = _sys(p)
+    x = _vectors(2, 256)
+    x[1] *= 1e-13
+    x[1, 0, 0] = 1.0
+    for adj in (False, True):
+        y, ref = s.apply(x, 5, adjoint=adj), _apply_ref(p, x, 5, adj)
+        err = (y - ref).abs()
+        assert float(err[0].amax()) <= 2.0**-50 * float(_term_bound(p, x, 5)[0])
+        # entries that neither the large one nor its neighbours reach
+        small = x.clone()
+        small[1, 0, 0] = 0.0
+        far = torch.ones(256, 256, dtype=torch.bool, device="cuda")
+        far[0, :] = far[:, 0] = False
+        far[:, :2] = far[:2, :] = False
+        for st in (1, 4, 16, 64):
+            far[st, :] = far[:, st] = False
+        assert float(err[1][far].amax()) <= 2.0**-48 * float(_term_bound(p, small, 5)[1])
