@@ -112,6 +112,7 @@ struct lb_system {
   double gamma1 = 0.0, pen_a = 1.0;  // running penalty (one CTA per state)
   bool rho_herm = false;  // every initial state exactly Hermitian
   bool tar_herm = false;  // every explicit target exactly Hermitian (gate targets: always)
+  bool rho_spread = true, tar_spread = true;  // ... within kGridCrest (gate targets: as their states)
   bool rho_finite = true;  // no NaN or Inf in the initial states
   int gblocks = 0;   // cooperative grid size of the forward grid sweep
   int gblocks_b = 0;  // ... and of the backward one
@@ -363,13 +364,41 @@ bool chunks_possible(const lb_system* s) {
          chunk_steps(s) * s->h * largest_decay(s) <= kChunkDecay && s->sweep != LB_SWEEP_RESIDENT && fixed_cfg(s, false).QT > 0;
 }
 
+// a state of N^2 entries this small is within kGridCrest whatever they are
+bool any_crest(const lb_system* s) { return (double)s->V <= lbk::kGridCrest * lbk::kGridCrest; }
+// every N x N complex matrix of M within kGridCrest (each component counts)
+bool spread_matrices(const double* a, int M, int N) {
+  const size_t n = (size_t)2 * N * N;
+  for (int i = 0; i < M; ++i) {
+    const double* m = a + (size_t)i * n;
+    double mx[4] = {0.0, 0.0, 0.0, 0.0}, sq[4] = {0.0, 0.0, 0.0, 0.0};
+    for (size_t t = 0; t + 3 < n; t += 4)
+      for (int k = 0; k < 4; ++k) {
+        mx[k] = std::max(mx[k], std::fabs(m[t + k]));
+        sq[k] += m[t + k] * m[t + k];
+      }
+    for (size_t t = n / 4 * 4; t < n; ++t) {
+      mx[0] = std::max(mx[0], std::fabs(m[t]));
+      sq[0] += m[t] * m[t];
+    }
+    const double top = std::max(std::max(mx[0], mx[1]), std::max(mx[2], mx[3]));
+    const double sum = (sq[0] + sq[1]) + (sq[2] + sq[3]);
+    // (false for values whose squares leave the range, too)
+    if (top != 0.0 && !(0.5 * (double)n * top * top <= lbk::kGridCrest * lbk::kGridCrest * sum)) return false;
+  }
+  return true;
+}
+
 // Whether this call runs the fixed-point sweeps: the Jacobi iteration with
-// rho_j <= 0.24, where its sums stay inside 64 bits.
-bool use_fixed(const lb_system* s, bool herm) {
+// rho_j <= 0.24, where its sums stay inside 64 bits, and on the grid vectors
+// within kGridCrest (spread: the caller's, else the initial states and targets,
+// between which the 2-norm and with it the crest factor changes little).
+bool use_fixed_on(const lb_system* s, bool herm, bool spread) {
   if (!s->fx_ws || s->method != LB_SOLVER_JACOBI) return false;
-  if (use_grid(s)) return rho_bound(s) <= lbk::kGridFixedRho;
+  if (use_grid(s)) return rho_bound(s) <= lbk::kGridFixedRho && (any_crest(s) || spread);
   return fixed_cfg(s, herm).E > 0 && rho_bound(s) <= lbk::kFixedRho;
 }
+bool use_fixed(const lb_system* s, bool herm) { return use_fixed_on(s, herm, s->rho_spread && s->tar_spread); }
 bool is_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
@@ -554,6 +583,14 @@ int order_after_uploads(lb_system* s, cudaStream_t stream) {
   if (stream == s->bind_stream) return LB_OK;
   LB_CUDA(cudaEventRecord(s->upload_done, s->bind_stream), "cudaEventRecord");
   LB_CUDA(cudaStreamWaitEvent(stream, s->upload_done, 0), "cudaStreamWaitEvent");
+  return LB_OK;
+}
+
+// Make `stream` wait for the last fixed-point lb_apply, whichever stream that
+// was on: the next user of its buffers.
+int order_after_products(lb_system* s, cudaStream_t stream) {
+  if (!s->apply_done) LB_CUDA(cudaEventCreateWithFlags(&s->apply_done, cudaEventDisableTiming), "cudaEventCreate");
+  LB_CUDA(cudaStreamWaitEvent(stream, s->apply_done, 0), "cudaStreamWaitEvent");
   return LB_OK;
 }
 
@@ -1317,6 +1354,7 @@ int lb_states_set(lb_system* s, int32_t M, const double* rho0, const double* wei
   s->Mu = M;
   s->wgt_u = w;
   s->rho_herm = hermitian_matrices(rho0, M, s->N);
+  s->rho_spread = any_crest(s) || spread_matrices(rho0, M, s->N);
   s->rho_finite = true;
   for (size_t t = 0; t < (size_t)2 * M * s->N * s->N; ++t)
     if (!std::isfinite(rho0[t])) {
@@ -1357,6 +1395,7 @@ int lb_objective_set(lb_system* s, int32_t kind, const double* targets, double g
   s->target_mode = 1;
   s->targets.assign(targets, targets + (size_t)2 * s->Mu * s->V);
   s->tar_herm = hermitian_matrices(targets, s->Mu, s->N);
+  s->tar_spread = any_crest(s) || spread_matrices(targets, s->Mu, s->N);
   if (!s->ws) update_pairs(s);
   if (s->ws) {
     s->hp.kind = kind;
@@ -1383,6 +1422,7 @@ int lb_objective_set_measure(lb_system* s, int32_t m, double gamma2) {
   s->target_mode = 1;
   s->targets.swap(t);
   s->tar_herm = true;
+  s->tar_spread = any_crest(s) || spread_matrices(s->targets.data(), 1, s->N);
   if (!s->ws) update_pairs(s);
   if (s->ws) {
     s->hp.kind = LB_J_NM;
@@ -1405,6 +1445,7 @@ int lb_objective_set_gate(lb_system* s, int32_t kind, const double* V, double ga
   s->gateV.assign(V, V + (size_t)2 * s->Ne * s->Ne);
   s->targets.clear();
   s->tar_herm = true;
+  s->tar_spread = true;
   if (!s->ws) update_pairs(s);
   if (s->ws) {
     s->hp.kind = kind;
@@ -1949,11 +1990,31 @@ int lb_gradient_async(lb_system* s, void* stream, void* G_dev, void* grad_dev) {
   return LB_OK;
 }
 
+// whether each of n_vec <= M device vectors of a grid system is within
+// kGridCrest (a vector with NaN or Inf counts as not)
+static int vectors_spread(lb_system* s, cudaStream_t st, const double2* x, int n_vec, bool* spread) {
+  std::vector<uint32_t> h((size_t)n_vec);
+  int rc = order_after_products(s, st);
+  if (rc) return rc;
+  LB_CUDA(lbk::launch_crest(s->hp, x, n_vec, st), "crest kernels");
+  LB_CUDA(cudaMemcpyAsync(h.data(), s->hp.apm, sizeof(uint32_t) * h.size(), cudaMemcpyDeviceToHost, st), "read crests");
+  LB_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+  *spread = true;
+  for (uint32_t v : h) *spread = *spread && v < 0x7ff00000u;
+  return LB_OK;
+}
+
 static int propagate_impl(lb_system* s, cudaStream_t st, int adjoint, int64_t j0, int64_t j1, double2* x, int n_vec) {
   int rc = order_after_uploads(s, st);
   if (rc) return rc;
   s->launches = 0;
-  s->fx_now = use_fixed(s, false, st);
+  bool spread = true;
+  if (use_fixed_on(s, false, true) && use_grid(s) && !any_crest(s) && n_vec <= s->M && !is_capturing(st)) {
+    // the given vectors decide (this call synchronises anyway)
+    rc = vectors_spread(s, st, x, n_vec, &spread);
+    if (rc) return rc;
+  }
+  s->fx_now = use_fixed_on(s, false, spread) && !is_capturing(st);
   rc = ensure_ctab(s, st);
   if (rc) return rc;
   LB_CUDA(cudaMemsetAsync(at<DevStatus>(s, s->L.status), 0, sizeof(DevStatus), st), "clear status");
@@ -2006,9 +2067,8 @@ int lb_apply(lb_system* s, void* stream, int32_t adjoint, int64_t step, const vo
   // call may be replayed beside another one, which would share that buffer
   if (use_grid(s) && s->fx_ws && n_vec <= s->M && (long long)n_vec * s->V >= lbk::kApplyFixedElements &&
       rho_bound(s) <= lbk::kFixedRho && !is_capturing(st)) {
-    // after the last such product, whichever stream that was on
-    if (!s->apply_done) LB_CUDA(cudaEventCreateWithFlags(&s->apply_done, cudaEventDisableTiming), "cudaEventCreate");
-    LB_CUDA(cudaStreamWaitEvent(st, s->apply_done, 0), "cudaStreamWaitEvent");
+    rc = order_after_products(s, st);
+    if (rc) return rc;
     LB_CUDA(lbk::launch_apply_gx(s->dp, s->hp, adjoint, step, static_cast<const double2*>(x_dev),
                                  static_cast<double2*>(y_dev), n_vec, st),
             "apply kernels");

@@ -1074,27 +1074,70 @@ __global__ void __launch_bounds__(kGridThreads, kGxBlocks)
 // common 2^ka so that the small sums keep 2^-60 of the largest entry times
 // 2^-ka.  The diagonal and the result are FP64.
 
-// high words of the largest magnitudes of n_vec vectors (slots cleared before)
-__global__ void k_apply_max(const double2* __restrict__ x, int V, unsigned* __restrict__ slots) {
-  const double2* xv = x + (size_t)blockIdx.y * V;
-  unsigned m = 0;
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
-    const double2 a = xv[v];
-    const unsigned long long b = umax64(abs_bits(a.x), abs_bits(a.y));
-    m = max(m, b ? max((unsigned)(b >> 32), 1u) : 0u);
-  }
-  m = __reduce_max_sync(kFull, m);
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(slots + blockIdx.y, m);
-}
 // scale with the largest entry in [2^59, 2^60) from its magnitude's high word
 __device__ __forceinline__ int gx_scale_of(unsigned h) {
   const int e = (int)(h >> 20);
   return h ? kFxTop - (e ? e - 1023 : -1022) : kFxTop;
 }
+// A vector's largest entry and the sum of its squares: the high word of the
+// largest magnitude and the sum over the squares of the entries in units of
+// 2^(its exponent).  Joined in a fixed order, so that a call's route repeats.
+struct GxCrest {
+  unsigned h;
+  float s;
+};
+__device__ __forceinline__ GxCrest gx_join_crest(GxCrest a, GxCrest b) {
+  const unsigned h = max(a.h, b.h);
+  const int e = (int)(h >> 20);
+  return GxCrest{h, ldexpf(a.s, 2 * ((int)(a.h >> 20) - e)) + ldexpf(b.s, 2 * ((int)(b.h >> 20) - e))};
+}
+__device__ GxCrest gx_block_crest(GxCrest c) {
+  __shared__ GxCrest w[kGxWarps];
+  for (int o = 16; o; o >>= 1) c = gx_join_crest(c, GxCrest{__shfl_xor_sync(kFull, c.h, o), __shfl_xor_sync(kFull, c.s, o)});
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = c;
+  __syncthreads();
+  c = w[0];
+  for (int i = 1; i < kGxWarps; ++i) c = gx_join_crest(c, w[i]);
+  return c;
+}
+// ... of each block's share of a vector, part[vector][block]
+__global__ void __launch_bounds__(kGridThreads) k_crest(const double2* __restrict__ x, int V, GxCrest* __restrict__ part) {
+  const double2* xv = x + (size_t)blockIdx.y * V;
+  GxCrest c{0u, 0.0f};
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
+    const double2 a = xv[v];
+    const unsigned long long b = umax64(abs_bits(a.x), abs_bits(a.y));
+    // (a nonzero value below the smallest high word counts as one unit of it)
+    const unsigned h = b ? max((unsigned)(b >> 32), 1u) : 0u;
+    float s = 0.0f;
+    if (h && h < 0x7ff00000u) {
+      const int sc = gx_scale_of(h);
+      const float fx = (float)(int)(fx_from_bits(a.x, sc) >> 32), fy = (float)(int)(fx_from_bits(a.y, sc) >> 32);
+      s = (fx * fx + fy * fy) * (1.0f / 18014398509481984.0f);  // 2^-54: units of 2^27 = 2^(59 - 32)
+    }
+    c = gx_join_crest(c, GxCrest{h, s});
+  }
+  c = gx_block_crest(c);
+  if (threadIdx.x == 0) part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = c;
+}
+// slots[vector] = the high word of its largest entry, or kGxNotFixed for a
+// vector that holds NaN or Inf or whose entries are not spread (kGridCrest)
+constexpr unsigned kGxNotFixed = 0x7ff00000u;
+__global__ void __launch_bounds__(kGridThreads) k_crest_vectors(const GxCrest* __restrict__ part, int n, int V,
+                                                               unsigned* __restrict__ slots) {
+  GxCrest c{0u, 0.0f};
+  for (int i = threadIdx.x; i < n; i += blockDim.x) c = gx_join_crest(c, part[(size_t)blockIdx.x * n + i]);
+  c = gx_block_crest(c);
+  if (threadIdx.x) return;
+  // the largest entry in [1, 2)
+  const float m = 1.0f + (float)(c.h & 0xfffffu) * (1.0f / 1048576.0f);
+  const bool spread = c.h == 0 || (float)V * m * m <= (float)(kGridCrest * kGridCrest) * c.s;
+  slots[blockIdx.x] = c.h < kGxNotFixed && spread ? c.h : kGxNotFixed;
+}
 __global__ void k_apply_split(const double2* __restrict__ x, int V, const unsigned* __restrict__ slots,
                               int4* __restrict__ z) {
   const unsigned h = slots[blockIdx.y];
-  if (h >= 0x7ff00000u) return;  // NaN or Inf: k_apply_gx computes this vector in FP64
+  if (h >= kGxNotFixed) return;  // k_apply_gx computes this vector in FP64
   const int sc = gx_scale_of(h);
   const size_t base = (size_t)blockIdx.y * V;
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
@@ -1151,7 +1194,7 @@ __global__ void __launch_bounds__(kGridThreads, kApplyBlocks)
     const uint32_t kd = __ldg(P.digits + k), ld = __ldg(P.digits + l);
     const unsigned h = __ldg(slots + b);
     double cr = 0.0, ci = 0.0;
-    if (h < 0x7ff00000u) {
+    if (h < kGxNotFixed) {
       const Cx c = gx_apply<ADJ, false, QN>(z + (size_t)b * V, gp, S, v, k, l, N, kd, ld);
       const double f = scalbn(inv, -gx_scale_of(h) - ka);
       cr = f * (double)c.x;
@@ -1236,15 +1279,22 @@ cudaError_t run_apply(unsigned blocks, size_t smem, cudaStream_t s, const ProbDe
 
 }  // namespace
 
+cudaError_t launch_crest(const ProbDev& h, const double2* x, int n_vec, cudaStream_t s) {
+  GxCrest* part = reinterpret_cast<GxCrest*>(h.apx);
+  const int n = std::min((h.V + 8 * kGridThreads - 1) / (8 * kGridThreads), 512);
+  k_crest<<<dim3((unsigned)n, n_vec), kGridThreads, 0, s>>>(x, h.V, part);
+  k_crest_vectors<<<n_vec, kGridThreads, 0, s>>>(part, n, h.V, h.apm);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h, int adjoint, int64_t step, const double2* x,
                             double2* y, int n_vec, cudaStream_t s) {
   const GxParams gp = gx_params(h);
-  unsigned* slots = h.apm;
+  const unsigned* slots = h.apm;
   int4* z = h.apx;
-  cudaError_t e = cudaMemsetAsync(slots, 0, sizeof(unsigned) * n_vec, s);
+  cudaError_t e = launch_crest(h, x, n_vec, s);
   if (e != cudaSuccess) return e;
   const unsigned bx = (unsigned)((h.V + 8 * 256 - 1) / (8 * 256));
-  k_apply_max<<<dim3(bx, n_vec), 256, 0, s>>>(x, h.V, slots);
   k_apply_split<<<dim3(bx, n_vec), 256, 0, s>>>(x, h.V, slots, z);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -240,9 +240,19 @@ cudaError_t launch_backward_grid(const ProbDev* d_prob, int nblocks, size_t smem
 // the same sweeps in fixed point (lb_gridx.cu)
 constexpr double kGridFixedRho = 0.0625;  // largest iteration-matrix bound they take
 constexpr int kGridFixedStates = 4096;    // most states (their scales are in shared memory)
+// Largest crest factor sqrt(N^2) max|x| / ||x||_2 of a state they take: an
+// entry is rounded to its state's largest one, so over a whole state the error
+// grows with the crest factor, where FP64's follows the 2-norm.  Against 80-bit
+// references (states of N^2 = 65536 after 30 steps, 2-norm; fixed point, FP64):
+// crest 7 3.1e-15, 6.9e-15; 40 4.1e-15, 6.9e-15; 133 4.4e-15, 4.5e-15; 253
+// 3.2e-15, 2.2e-15; 256 (one entry) 1.8e-15, 0.8e-15.  Gradients are as close
+// or closer at all of them.
+constexpr double kGridCrest = 128.0;
 cudaError_t launch_sweep_gx(const ProbDev* d_prob, const ProbDev& h_prob, int mode, int tape, int64_t j0, int64_t j1,
                             double2* x, int nstates, cudaStream_t s);
 cudaError_t launch_backward_gx(const ProbDev* d_prob, const ProbDev& h_prob, cudaStream_t s);
+// P.apm[i] of n_vec <= M vectors: below 0x7ff00000 when vector i is within kGridCrest
+cudaError_t launch_crest(const ProbDev& h_prob, const double2* x, int n_vec, cudaStream_t s);
 // y = M x with the off-diagonal part in fixed point (n_vec <= M)
 constexpr long long kApplyFixedElements = 1 << 17;  // fewest elements of a call that take it
 cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h_prob, int adjoint, int64_t step, const double2* x,
