@@ -258,7 +258,7 @@ int check_predictor(const lb_system* s) {
 bool recompute_predicts(const lb_system* s) { return effective_K(s) > 0 && effective_pred(s) > 0; }
 
 // the largest phase |h (E_k - E_l)| an element's free evolution turns by in
-// one step (H_sys, Sec. II); infinite when a frequency is not finite
+// one step (H_sys, Sec. II)
 double largest_phase(const lb_system* s) {
   double lo = 0.0, hi = 0.0;
   for (int k = 0; k < s->N; ++k) {
@@ -272,7 +272,6 @@ double largest_phase(const lb_system* s) {
       E += s->det[q] * d[q] - 0.5 * s->kerr[q] * d[q] * (d[q] - 1.0);
       for (int p = 0; p < q; ++p) E -= s->xkerr[p * s->Q + q] * d[p] * d[q];
     }
-    if (!std::isfinite(E)) return INFINITY;
     lo = k ? std::min(lo, E) : E;
     hi = k ? std::max(hi, E) : E;
   }

@@ -307,18 +307,6 @@ def test_gradient_of_a_peaked_state(L, levels, sweep, symmetry):
 
 
 @gpu
-@pytest.mark.parametrize("sweep", [0, 1, 2])
-def test_a_cross_kerr_that_is_not_a_number_is_reported(L, sweep):
-    p = W.random_problem(817, levels=(2, 2), n_states=1, n_steps=80, T_ns=0.8, amp=0.02, ckpt_every=0)
-    p.system.crosskerr_ghz[0, 1] = np.nan
-    s = _sys(p, sweep=sweep)
-    for call in (s.forward, s.gradient):
-        with pytest.raises(L.LBError) as e:
-            call()
-        assert e.value.code in (L.LB_ENAN, L.LB_ENOTCONV)
-
-
-@gpu
 @pytest.mark.parametrize("hermitian,K", [(True, 0), (False, 4)])
 def test_a_zero_adjoint_state_beside_a_small_one(L, hermitian, K):
     """The grid sweep brings every state's gradient sums to one scale: a state
