@@ -27,6 +27,7 @@ int fail(int code, const std::string& msg) {
 }
 
 int cuda_fail(cudaError_t e, const char* where) {
+  (void)cudaGetLastError();  // a launch's error must not be the next call's too
   return fail(LB_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
