@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(T)
         const unsigned long long mx = fx_cta_max(S, abs_bits(sr));
         if (j > j0) fx_ctl(S, P, H.cq, j - 1, cnt.step);
         if (mx >= kInfBits && j > 0) {
-          if (threadIdx.x == 0) record_error(P.status, LB_ENAN, j - 1);
+          fx_overflow(P.status, j - 1, chunked);
           return;
         }
         if (mx == 0 || mx >= kInfBits) continue;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(T)
         for (int e = 0; e < E; ++e) src[e] = fx_v(st, S, H, e) < V ? source(e) : 0.0;
         // (the state before step 0 is not used)
         if (!fx_add_source(st, S, src, true) && j > 0) {
-          if (threadIdx.x == 0) record_error(P.status, LB_ENAN, j - 1);
+          fx_overflow(P.status, j - 1, chunked);
           stats.flush(P.status);
           return;
         }

@@ -587,6 +587,16 @@ __device__ __forceinline__ void fx_fail(DevStatus* st, int j, bool chunked) {
     record_error(st, LB_ENOTCONV, j);
 }
 
+// an adjoint state that a source before step j made infinite; chunks run at the
+// same time: the latest step, which a step-by-step sweep meets first, counts
+__device__ __forceinline__ void fx_overflow(DevStatus* st, int j, bool chunked) {
+  if (threadIdx.x) return;
+  if (!chunked)
+    record_error(st, LB_ENAN, j);
+  else if (const int c = atomicCAS(&st->code, 0, LB_ENAN); c == 0 || c == LB_ENAN)
+    atomicMax(&st->step, j);
+}
+
 // steps of a launch so far (they select buffers)
 struct FxCount {
   unsigned step = 0;

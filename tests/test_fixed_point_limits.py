@@ -557,7 +557,7 @@ def test_a_penalty_source_that_overflows_is_reported(L, n_steps, sweep):
     s = _sys(p, sweep=sweep)
     with pytest.raises(L.LBError) as e:
         s.gradient()
-    assert e.value.code == L.LB_ENAN
+    assert e.value.code == L.LB_ENAN and str(e.value).endswith(f"time step {n_steps - 2}")
 
 
 @gpu
