@@ -432,25 +432,25 @@ def test_products_where_control_and_decay_factors_are_alike(L):
     """Drives as weak as the decay: scaled up together, the two control factors
     and the decay factor of one sum must not pass 64 bits.  The bound is that of
     test_large_products_match_fp64."""
-    p = _mode(3, (4, 4, 4, 4))
+    p = _mode(3, (4, 4, 4, 4), n_states=6)
     Q = 4
     p.controls.carriers_ghz = [np.zeros(1) for _ in range(Q)]
     # (dt/2) 2 pi |d| 2^3 (the ladder's scale) = (dt/2) 3 / T1
     p.controls.alpha = np.full(2 * p.controls.n_splines * Q, 3.0 / 40e3 / (2.0 * np.pi * 8.0))
     s = _sys(p, sweep=L.LB_SWEEP_GRID)
-    x = _vectors(2, 256)
+    x = _vectors(6, 256)
     for adj in (False, True):
         y, ref = s.apply(x, 1, adjoint=adj), _apply_ref(p, x, 1, adj)
         assert bool(((y - ref).abs().amax(dim=(1, 2)) <= 2.0**-50 * _term_bound(p, x, 1)).all())
 
 
-# edges of the product's dispatch: 2^17 elements and just below, the unrolled
+# edges of the product's dispatch: 3 2^17 elements and just below, the unrolled
 # loops (4 and 6 subsystems) and the general one, odd N, tables above 48 KB of
 # shared memory, fewer vectors than states
 @gpu
 @pytest.mark.parametrize("levels,M,n", [
-    ((4, 4, 4, 4), 2, 2), ((4, 4, 4, 4), 2, 1), ((3, 3, 3, 3, 3), 3, 3), ((3,) * 6, 1, 1), ((5, 5, 5), 9, 9),
-    ((5, 5, 5), 9, 8), ((7, 3, 7), 7, 7), ((2, 2, 56), 3, 3), ((2, 64), 8, 8)])
+    ((4, 4, 4, 4), 6, 6), ((4, 4, 4, 4), 6, 5), ((3, 3, 3, 3, 3), 7, 7), ((3,) * 6, 1, 1), ((5, 5, 5), 26, 26),
+    ((5, 5, 5), 26, 25), ((7, 3, 7), 20, 19), ((2, 2, 56), 8, 8), ((2, 64), 24, 24)])
 @pytest.mark.parametrize("decay", [True, False])
 def test_large_products_match_fp64(L, levels, M, n, decay):
     """FP64's and the integers' rounding of at most 2^-50 of the terms."""
@@ -477,9 +477,9 @@ def test_large_products_match_fp64(L, levels, M, n, decay):
 @gpu
 def test_products_beside_a_gradient_and_each_other_on_other_streams(L):
     """Products on two streams while a gradient runs on a third: all as alone."""
-    p = W.prefix(W.config4(n_states=3), 60)
+    p = W.prefix(W.config4(n_states=6), 60)
     s = _sys(p)
-    x, x2 = _vectors(3, 256, 6), _vectors(3, 256, 7)
+    x, x2 = _vectors(6, 256, 6), _vectors(6, 256, 7)
     G, g = s.gradient()
     _fixed(s)
     y, y2 = s.apply(x, 7), s.apply(x2, 9)
@@ -493,7 +493,7 @@ def test_products_beside_a_gradient_and_each_other_on_other_streams(L):
     for k in range(6):
         for i in range(2):
             L.check(s.lib.lb_apply(s.h, streams[1 + i].cuda_stream, 0, (7, 9)[i], bufs[i].data_ptr(),
-                                   outs[i][k].data_ptr(), 3))
+                                   outs[i][k].data_ptr(), 6))
     torch.cuda.synchronize()
     assert float(Gd) == G and np.array_equal(gd.cpu().numpy(), g)
     for i, want in enumerate((y, y2)):
@@ -504,17 +504,17 @@ def test_products_beside_a_gradient_and_each_other_on_other_streams(L):
 @gpu
 def test_a_recorded_product_is_replayed(L):
     """Recorded, the product is FP64 (its own buffer would be shared by replays)."""
-    p = W.prefix(W.config4(n_states=3), 20)
+    p = W.prefix(W.config4(n_states=6), 20)
     st = torch.cuda.Stream()
     with torch.cuda.stream(st):
         s = _sys(p)
-        x = _vectors(3, 256, 6).transpose(1, 2).contiguous()
+        x = _vectors(6, 256, 6).transpose(1, 2).contiguous()
         y, z = torch.zeros_like(x), torch.zeros_like(x)
-        L.check(s.lib.lb_apply(s.h, st.cuda_stream, 0, 7, x.data_ptr(), y.data_ptr(), 3))
+        L.check(s.lib.lb_apply(s.h, st.cuda_stream, 0, 7, x.data_ptr(), y.data_ptr(), 6))
         torch.cuda.synchronize()
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph, stream=st):
-            L.check(s.lib.lb_apply(s.h, st.cuda_stream, 0, 7, x.data_ptr(), z.data_ptr(), 3))
+            L.check(s.lib.lb_apply(s.h, st.cuda_stream, 0, 7, x.data_ptr(), z.data_ptr(), 6))
         graph.replay()
         torch.cuda.synchronize()
     assert _rel(z.cpu().numpy(), y.cpu().numpy()) < 1e-14
@@ -625,9 +625,9 @@ def test_peaked_states_of_large_systems_keep_fp64(L):
 def test_products_of_peaked_vectors(L):
     """Per vector: one of spread entries, one of a single large entry among
     entries of 1e-13, whose products keep their own 53 bits away from it."""
-    p = _large("spread", 2)
+    p = _large("spread", 6)
     s = _sys(p)
-    x = _vectors(2, 256)
+    x = _vectors(6, 256)
     x[1] *= 1e-13
     x[1, 0, 0] = 1.0
     for adj in (False, True):
