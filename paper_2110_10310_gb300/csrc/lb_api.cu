@@ -345,19 +345,24 @@ bool fixed_possible(const lb_system* s) {
 }
 
 // steps per chunk: the chunks of steps run at the same time, the C boundary
-// products one after another, so about the square root of the step count
+// products one after another, so about the square root of the step count (the
+// factor 0.6, 0.8, 1, 1.3: qubit, 1000 steps, 0.371, 0.338, 0.391, 0.419 ms; CNOT,
+// 10000 steps, 6.15, 5.84, 5.56, 5.29 ms)
 int chunk_steps(const lb_system* s) {
   return std::max(8, (int)std::lround(0.8 * std::sqrt((double)s->NT)));
 }
 // Chunked sweeps (lb_fixed_chunks.cu) of the small states the cluster sweep
 // took one cluster each: with the full stage tape, at least kChunkMinSteps
-// steps, and N^2 <= 128, where N (N + 1) / 2 columns per chunk cost less than the idle
-// SMs.  A chunk starts its predictor cold, so a step takes more iterations
+// steps (gradients in ms, chunks / one CTA per state / the FP64 cluster sweep:
+// CNOT 16 steps 0.255 / 0.212 / 0.231, 24 steps 0.255 / 0.258 / 0.260, 63 steps
+// 0.328 / 0.446 / 0.418; 11 levels 0.280 / 0.259 / 0.319, 0.300 / 0.320 / 0.423
+// and 0.409 / 0.566 / 0.922), and N^2 <= 128, where N (N + 1) / 2 columns per chunk
+// cost less than the idle SMs.  A chunk starts its predictor cold, so a step takes more iterations
 // there: max_iter must leave room for a cold start at rho = 0.24.  The
 // propagators' entries are kept to 2^-62 of the largest possible, the states to
 // 2^-60: an entry that decays by more than kChunkDecay e-folds within a
 // chunk would fall below the state's resolution, so such systems run step by step.
-constexpr int kChunkMinSteps = 64, kChunkMinIter = 64;
+constexpr int kChunkMinSteps = 24, kChunkMinIter = 64;
 constexpr double kChunkDecay = 1.0;
 bool chunks_possible(const lb_system* s) {
   return !use_grid(s) && s->V <= lbk::kFxChunkV && s->NT >= kChunkMinSteps && s->max_iter >= kChunkMinIter && effective_K(s) == 0 &&

@@ -94,7 +94,7 @@ def test_an_adjoint_state_that_gathers_within_a_chunk(L):
 
 
 @gpu
-@pytest.mark.parametrize("n_steps,theta,weight,sweep", [(24, 0.7796, 1.0, "resident"), (64, np.pi / 4.5, 1.06, "cluster")])
+@pytest.mark.parametrize("n_steps,theta,weight,sweep", [(23, 0.7796, 1.0, "resident"), (64, np.pi / 4.5, 1.06, "cluster")])
 def test_a_penalty_source_that_cancels_the_adjoint_state(L, n_steps, theta, weight, sweep):
     """A free coherence whose adjoint turns by theta per step while a constant
     running penalty adds the same source each step: the sum falls to some
@@ -128,7 +128,7 @@ def _vanishing(levels, n_steps, zero):
 
 
 @gpu
-@pytest.mark.parametrize("levels,n_steps,sweep", [((2, 2), 24, 1), ((2, 2), 80, 0), ((3, 2, 3), 10, 1), ((3, 3), 20, 2)])
+@pytest.mark.parametrize("levels,n_steps,sweep", [((2, 2), 24, 1), ((2, 2), 24, 0), ((2, 2), 80, 0), ((3, 2, 3), 10, 1), ((3, 3), 20, 2)])
 @pytest.mark.parametrize("zero", ["weight", "state"])
 def test_states_of_zeros(L, levels, n_steps, sweep, zero):
     """The one-CTA sweeps (register and table path), the chunks and the grid."""
@@ -643,3 +643,21 @@ def test_products_of_peaked_vectors(L):
         for st in (1, 4, 16, 64):
             far[st, :] = far[:, st] = False
         assert float(err[1][far].amax()) <= 2.0**-48 * float(_term_bound(p, small, 5)[1])
+
+
+@gpu
+@pytest.mark.parametrize("levels,penalty", [((2,), 0.0), ((3, 3), 0.0), ((3, 3), 0.3), ((11,), 0.0)])
+@pytest.mark.parametrize("n_steps", [23, 24, 25, 40])
+def test_the_shortest_horizons_in_chunks(L, levels, penalty, n_steps):
+    """Three chunks of eight steps and around: a last chunk of one step, none."""
+    p = W.random_problem(825, levels=levels, n_states=2, n_steps=n_steps, T_ns=0.01 * n_steps, amp=0.01, hermitian=False,
+                         ckpt_every=0)
+    if levels == (11,):
+        p.system.selfkerr_ghz[:] = 0.01
+    p.gamma1, p.penalty_a = penalty, 0.1
+    s = _sys(p)
+    G, g = s.gradient()
+    assert (_fixed(s).stats()["kernel_launches"] > 8) == (n_steps >= 24)
+    Go, go, _ = imr.gradient(p)
+    assert abs(G - Go) <= 1e-10 * abs(Go)
+    assert _rel(g, go) < 1e-9
