@@ -83,7 +83,7 @@ struct FxSmem {
   uint16_t* hmir;   // [Vh] its mirror, 0xffff on the diagonal
   unsigned* slots;  // [2][2][32]: per step parity the warps' max |rhs|, per iteration parity their max change
   int4* ctl;        // [2][cq + 1] control factors of the step (a, b split), last the stopping factor
-  int* gred;        // [2][Q][4][kFxWarps][3] words of the warps' gradient sums, by step parity
+  int* gred;        // [2][Q][4][kFxWarps][3] limbs of the warps' gradient sums, by step parity
   unsigned long long* mx;  // [kFxWarps] fx_cta_max's
   int4* dsm;        // [nel] (I - dt/2 D)^-1 - 1 (QT == 0)
   Fx* zb0;          // [V][2] iterate, split, component by component
