@@ -371,29 +371,6 @@ bool chunks_possible(const lb_system* s) {
 
 // a state of N^2 entries this small is within kGridCrest whatever they are
 bool any_crest(const lb_system* s) { return (double)s->V <= lbk::kGridCrest * lbk::kGridCrest; }
-// every N x N complex matrix of M within kGridCrest (each component counts)
-bool spread_matrices(const double* a, int M, int N) {
-  const size_t n = (size_t)2 * N * N;
-  for (int i = 0; i < M; ++i) {
-    const double* m = a + (size_t)i * n;
-    double mx[4] = {0.0, 0.0, 0.0, 0.0}, sq[4] = {0.0, 0.0, 0.0, 0.0};
-    for (size_t t = 0; t + 3 < n; t += 4)
-      for (int k = 0; k < 4; ++k) {
-        mx[k] = std::max(mx[k], std::fabs(m[t + k]));
-        sq[k] += m[t + k] * m[t + k];
-      }
-    for (size_t t = n / 4 * 4; t < n; ++t) {
-      mx[0] = std::max(mx[0], std::fabs(m[t]));
-      sq[0] += m[t] * m[t];
-    }
-    const double top = std::max(std::max(mx[0], mx[1]), std::max(mx[2], mx[3]));
-    const double sum = (sq[0] + sq[1]) + (sq[2] + sq[3]);
-    // (false for values whose squares leave the range, too)
-    if (top != 0.0 && !(0.5 * (double)n * top * top <= lbk::kGridCrest * lbk::kGridCrest * sum)) return false;
-  }
-  return true;
-}
-
 // Whether this call runs the fixed-point sweeps: the Jacobi iteration with
 // rho_j <= 0.24, where its sums stay inside 64 bits, and on the grid vectors
 // within kGridCrest (spread: the caller's, else the initial states and targets,
@@ -747,20 +724,42 @@ int upload_targets(lb_system* s, cudaStream_t st) {
 // rounding: each entry within 64 eps max|entry| of the conjugate of its
 // transposed entry (an outer product psi psi^+ formed with fused multiply-adds
 // is Hermitian only to that level)
-bool hermitian_matrices(const double* a, int M, int N) {
+// spread (if given): every matrix within kGridCrest, each component counting
+bool hermitian_matrices(const double* a, int M, int N, bool* spread = nullptr) {
   const size_t NN = (size_t)N * N;
-  for (int i = 0; i < M; ++i) {
+  bool herm = true;
+  if (spread) *spread = true;
+  for (int i = 0; i < M && (herm || (spread && *spread)); ++i) {
     const double* m = a + 2 * (size_t)i * NN;
-    double amax = 0.0;
-    for (size_t t = 0; t < 2 * NN; ++t) amax = std::max(amax, std::fabs(m[t]));
+    // (four partial results: the loop is not a chain)
+    double mx[4] = {0.0, 0.0, 0.0, 0.0}, sq[4] = {0.0, 0.0, 0.0, 0.0};
+    const size_t n4 = 2 * NN / 4 * 4;
+    for (size_t t = 0; t < n4; t += 4)
+      for (int k = 0; k < 4; ++k) {
+        mx[k] = std::max(mx[k], std::fabs(m[t + k]));
+        sq[k] += m[t + k] * m[t + k];
+      }
+    for (size_t t = n4; t < 2 * NN; ++t) {
+      mx[0] = std::max(mx[0], std::fabs(m[t]));
+      sq[0] += m[t] * m[t];
+    }
+    const double amax = std::max(std::max(mx[0], mx[1]), std::max(mx[2], mx[3]));
+    const double sum = (sq[0] + sq[1]) + (sq[2] + sq[3]), top = amax * amax;
+    // (values whose squares leave the range count as not spread)
+    if (spread && amax != 0.0 &&
+        !(top > 1e-280 && sum < 1e300 && (double)NN * top <= lbk::kGridCrest * lbk::kGridCrest * sum))
+      *spread = false;
     const double tol = 64.0 * 2.220446049250313e-16 * amax;
-    for (int l = 0; l < N; ++l)
+    for (int l = 0; l < N && herm; ++l)
       for (int k = 0; k <= l; ++k) {
         const size_t p = (size_t)2 * (k + (size_t)N * l), q = (size_t)2 * (l + (size_t)N * k);
-        if (!(std::fabs(m[p] - m[q]) <= tol) || !(std::fabs(m[p + 1] + m[q + 1]) <= tol)) return false;
+        if (!(std::fabs(m[p] - m[q]) <= tol) || !(std::fabs(m[p + 1] + m[q + 1]) <= tol)) {
+          herm = false;
+          break;
+        }
       }
   }
-  return true;
+  return herm;
 }
 
 // the Hermitian symmetry runs in every sweep kind: grid, one CTA per state
@@ -1358,8 +1357,7 @@ int lb_states_set(lb_system* s, int32_t M, const double* rho0, const double* wei
   if (s->Mu != M && s->target_mode == 1) s->target_mode = 0;  // explicit targets no longer match
   s->Mu = M;
   s->wgt_u = w;
-  s->rho_herm = hermitian_matrices(rho0, M, s->N);
-  s->rho_spread = any_crest(s) || spread_matrices(rho0, M, s->N);
+  s->rho_herm = hermitian_matrices(rho0, M, s->N, &s->rho_spread);
   s->rho_finite = true;
   for (size_t t = 0; t < (size_t)2 * M * s->N * s->N; ++t)
     if (!std::isfinite(rho0[t])) {
@@ -1399,8 +1397,7 @@ int lb_objective_set(lb_system* s, int32_t kind, const double* targets, double g
   s->gamma2 = gamma2;
   s->target_mode = 1;
   s->targets.assign(targets, targets + (size_t)2 * s->Mu * s->V);
-  s->tar_herm = hermitian_matrices(targets, s->Mu, s->N);
-  s->tar_spread = any_crest(s) || spread_matrices(targets, s->Mu, s->N);
+  s->tar_herm = hermitian_matrices(targets, s->Mu, s->N, &s->tar_spread);
   if (!s->ws) update_pairs(s);
   if (s->ws) {
     s->hp.kind = kind;
@@ -1427,7 +1424,7 @@ int lb_objective_set_measure(lb_system* s, int32_t m, double gamma2) {
   s->target_mode = 1;
   s->targets.swap(t);
   s->tar_herm = true;
-  s->tar_spread = any_crest(s) || spread_matrices(s->targets.data(), 1, s->N);
+  hermitian_matrices(s->targets.data(), 1, s->N, &s->tar_spread);
   if (!s->ws) update_pairs(s);
   if (s->ws) {
     s->hp.kind = LB_J_NM;
