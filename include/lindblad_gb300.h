@@ -127,10 +127,14 @@ typedef struct lb_system_desc {
  * one power of two per state, on the integer pipe; for the Jacobi iteration
  * while every step's iteration matrix is bounded by 0.24 (the grid sweep: 1/16,
  * no coupling, no running penalty) and the step's diagonal phases are small.
- * Closer to the exact solution of the step than FP64.  The predictor's order
- * counts up to 8 for the states it keeps in registers.  A call recorded into
- * a CUDA graph, and a workspace without these sweeps' tables (smaller than
- * lb_workspace_bytes says), run LB_ARITH_F64. */
+ * An entry is rounded to 2^-60 of its state's largest one (FP64: to 2^-53 of
+ * itself).  Initial states or targets of N^2 > 16384 whose crest factor
+ * sqrt(N^2) max|x| / ||x||_2 is above 128 (a basis state) therefore run
+ * LB_ARITH_F64; for lb_propagate the given vectors decide, for lb_apply each
+ * vector.  The predictor's order counts up to 8 for the states it keeps in
+ * registers.  A call recorded into a CUDA graph, and a workspace without these
+ * sweeps' tables (smaller than lb_workspace_bytes says), run LB_ARITH_F64: a
+ * replay can differ from the same call made directly in the last digits. */
 #define LB_ARITH_F64 0
 #define LB_ARITH_FIXED 1
 

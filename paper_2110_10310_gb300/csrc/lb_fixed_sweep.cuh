@@ -50,19 +50,6 @@ constexpr int fx_max_threads() {
   return QT > 0 ? kFxPlanThreads : kFxTabThreads;
 }
 
-__constant__ int kExtrapI[kRingOrder + 1][kRingOrder] = {
-    {0, 0, 0, 0, 0, 0, 0, 0, 0, 0},
-    {1, 0, 0, 0, 0, 0, 0, 0, 0, 0},
-    {2, -1, 0, 0, 0, 0, 0, 0, 0, 0},
-    {3, -3, 1, 0, 0, 0, 0, 0, 0, 0},
-    {4, -6, 4, -1, 0, 0, 0, 0, 0, 0},
-    {5, -10, 10, -5, 1, 0, 0, 0, 0, 0},
-    {6, -15, 20, -15, 6, -1, 0, 0, 0, 0},
-    {7, -21, 35, -35, 21, -7, 1, 0, 0, 0},
-    {8, -28, 56, -70, 56, -28, 8, -1, 0, 0},
-    {9, -36, 84, -126, 126, -84, 36, -9, 1, 0},
-    {10, -45, 120, -210, 252, -210, 120, -45, 10, -1}};
-
 // one subsystem, for the table path: levels n, index stride s, bit position of
 // its digit, whether it decays, and the offsets of its ladder and decay factors
 struct FxSub {

@@ -15,7 +15,7 @@ namespace {
 // One cooperative launch keeps every SM busy on all M states at once.  Block
 // b owns a contiguous chunk of the flattened [M][V] element range; each inner
 // iteration reads the previous iterate of every element (neighbours through
-// L2, bypassing L1) and ends with a grid barrier.  Per-state maxima of
+// L1, see kNbL2) and ends with a grid barrier.  Per-state maxima of
 // |z_new - z| and |q| are combined with atomicMax on the integer bit patterns
 // (order independent), so every block takes the same stopping decision and a
 // recompute is bit-identical.

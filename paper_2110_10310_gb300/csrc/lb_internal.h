@@ -119,7 +119,7 @@ struct ProbDev {
   float2* Dinvf;             // [V] grid sweeps: (I - dt/2 D)^-1 in single precision
   int32_t ff;                // grid sweeps: FP64 iterations apply O in single-precision pairs (lb_set_precision)
   int32_t pad2;
-  // fixed-point sweeps (lb_fixed.cu; null without their workspace)
+  // fixed-point sweeps (lb_fixed_sweep.cuh, lb_gridx.cu; null without their workspace)
   int32_t kc[LB_MAXQ + LB_MAXQ * (LB_MAXQ - 1) / 2];  // 2^kc >= 4 times the largest ladder factor, per subsystem, then pair
   int32_t fxframe;           // their predictor turns its frame (the phases per step are not small)
   int32_t fxfwd;             // ... and is used in the forward solves (like the cluster sweep's: not with checkpoints)
@@ -193,7 +193,7 @@ cudaError_t launch_apply(const ProbDev* d_prob, const ProbDev& h_prob, int adjoi
 cudaError_t launch_propagate_resident(const ProbDev* d_prob, int adjoint, int64_t j0, int64_t j1, double2* x,
                                       int n_vec, const ResidentConfig& rc, cudaStream_t s);
 
-// one-CTA-per-state sweeps in fixed point (lb_fixed.cu)
+// one-CTA-per-state sweeps in fixed point (lb_fixed_sweep.cuh)
 constexpr int kFxChunkV = 128;      // largest N^2 of the chunked sweep
 constexpr size_t kFxMaxSmem = 227 * 1024;  // shared memory of one CTA
 constexpr double kFixedRho = 0.24;  // largest iteration-matrix bound rho_j they take
@@ -238,7 +238,14 @@ cudaError_t launch_sweep_grid(const ProbDev* d_prob, int mode, int init_from_q0,
                               double2* x, int nstates, int nblocks, size_t smem, int ff, cudaStream_t s);
 cudaError_t launch_backward_grid(const ProbDev* d_prob, int nblocks, size_t smem, int ff, cudaStream_t s);
 // the same sweeps in fixed point (lb_gridx.cu)
-constexpr double kGridFixedRho = 0.0625;  // largest iteration-matrix bound they take
+// Largest iteration-matrix bound they take.  One sum of gx_apply takes both
+// control factors of a subsystem, together at most 2 sqrt(2) times the bound (two
+// levels), a decay factor, and 3/8 of 64 bits for their low halves: it can pass 64
+// bits above 0.2, and stays below 0.6 of them at 1/16.  (Fixed point is the
+// faster at any bound: gradients of 4^4 levels, 200 steps, 17.6 ms against 37.6 at
+// 0.049 and 22.7 against 44.2 at 0.147; six qutrits, 30 steps, 20.2 against 55.1
+// at 0.053 and 27.3 against 68.3 at 0.14.)
+constexpr double kGridFixedRho = 0.0625;
 constexpr int kGridFixedStates = 4096;    // most states (their scales are in shared memory)
 // Largest crest factor sqrt(N^2) max|x| / ||x||_2 of a state they take: an
 // entry is rounded to its state's largest one, so over a whole state the error

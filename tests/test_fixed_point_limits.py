@@ -661,3 +661,15 @@ def test_the_shortest_horizons_in_chunks(L, levels, penalty, n_steps):
     Go, go, _ = imr.gradient(p)
     assert abs(G - Go) <= 1e-10 * abs(Go)
     assert _rel(g, go) < 1e-9
+
+
+@gpu
+@pytest.mark.parametrize("K", [0, 100])
+def test_fp64_sweeps_over_the_whole_cnot_horizon(L, K):
+    """The CNOT workload's 10000 steps in both arithmetics, to the method's targets."""
+    p = W.config2()
+    s, f = _sys(p, ckpt_every=K), _sys(p, ckpt_every=K, arithmetic=L.LB_ARITH_F64)
+    G, g = _fixed_after(s)
+    Gf, gf = f.gradient()
+    assert f.stats()["arithmetic"] == "f64"
+    assert abs(G - Gf) <= 1e-10 * abs(Gf) and _rel(g, gf) < 1e-9
