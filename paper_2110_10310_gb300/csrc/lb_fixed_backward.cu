@@ -8,9 +8,9 @@ namespace lbk {
 namespace {
 
 // sum over the warp of v without its last 16 bits, in three limbs of 27 bits (the
-// sums unsigned, unsigned and signed), to every lane.  (With all 32 bits a
-// fourth reduction per sum: the CNOT gradient 2 % slower.  2^-16 of the cut over
-// 4096 products stays 2^-6 below what one entry's rounding adds.)
+// sums unsigned, unsigned and signed), to every lane.  (All 32 bits take a
+// fourth reduction per sum: CNOT gradient, 10000 steps, 5.90 ms against 5.79.
+// 2^-16 of the cut over 4096 products stays 2^-6 below what one entry's rounding adds.)
 __device__ __forceinline__ int3 fx_warp_sum(const FxSum& v) {
   const unsigned h0 = (unsigned)v.hi;
   int3 r;

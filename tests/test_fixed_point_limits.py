@@ -195,6 +195,51 @@ def test_sums_of_products_keep_32_bits_below_the_cut(tmp_path):
         assert 0 <= a * x + b * y - ((hi << 32) + lo) * 2**32 < 2 * 2**32
 
 
+SHIFTS = r"""
+#include <cstdio>
+#include "lb_fixed.cuh"
+int main() {
+  long long x;
+  int s;
+  unsigned h;
+  while (std::scanf("%lld %d %u", &x, &s, &h) == 3)
+    std::printf("%lld %d %d %u\n", lbk::fx_shift(x, s), lbk::fx_rescale_shift(h), lbk::fx_quarter_shift(h),
+                lbk::fx_stop(1e-15f, h));
+  return 0;
+}
+"""
+
+
+def test_shifts_of_states_of_any_size(tmp_path):
+    """fx_shift rounds to nearest at every size, and the shifts that keep a
+    state's scale bring its largest high word to [2^27, 2^28) or leave it there."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    B = importlib.import_module("paper_2110_10310_gb300.build")
+    src, exe = tmp_path / "h.cu", str(tmp_path / "h")
+    src.write_text(SHIFTS)
+    r = subprocess.run([nvcc, "-std=c++17", "-O2", "-I", B.CSRC, "-o", exe, str(src)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    rng = random.Random(7)
+    cases = [(0, 0, 0), (1, 0, 1), ((1 << 61) - 1, 61, (1 << 31) - 1), (-(1 << 61), 61, 1 << 28)]
+    for _ in range(3000):
+        s = rng.randrange(-20, 62)
+        x = rng.randrange(-(1 << 61), 1 << 61) >> (max(0, -s) + rng.randrange(0, 3))
+        cases.append((x, s, rng.randrange(0, 1 << 31) >> rng.randrange(0, 31)))
+    inp = "\n".join(" ".join(str(v) for v in c) for c in cases)
+    out = subprocess.run([exe], input=inp, capture_output=True, text=True, timeout=60).stdout.split("\n")
+    for (x, s, h), line in zip(cases, out):
+        y, rs, qs, stop = (int(v) for v in line.split())
+        assert y == ((x + ((1 << s) >> 1)) >> s if s >= 0 else x << -s)
+        kept = h == 0 or 94906266 <= h < 1 << 28
+        assert rs == (0 if kept else h.bit_length() - 28)
+        quarter = h == 0 or 94906266 // 4 <= h < 1 << 26
+        assert qs == (-2 if quarter else h.bit_length() - 28)
+        want = max(1.0, 1e-15 * h * 2.0**32)
+        assert abs(stop - min(want, 0xffffff00)) <= 1.0 + 1e-6 * want
+
+
 def _long_gradient(p):
     """G's pieces and the gradient of one state in extended precision (numpy's
     longdouble): the matrix form, each stage by the Jacobi iteration."""
