@@ -542,7 +542,7 @@ def run_apply(args, rank, world, dev):
             "higher_is_better": True,
             "scaling": "weak",
             "vs_baseline": None,
-            "dtype": "f64",
+            "dtype": "f64 (int64 fixed point)" if fixed else "f64",
             "data": "synthetic",
             "config": {"workload": WORKLOADS["apply_6x3"].format(n=n),
                        "l2": "inputs ({:.0f} MB in, {:.0f} MB out) larger than L2".format(nbytes / 2e6, nbytes / 2e6),
@@ -690,7 +690,7 @@ def run_batch(args, rank, world, dev):
             "higher_is_better": True,
             "scaling": "weak",
             "vs_baseline": None,
-            "dtype": "f64",
+            "dtype": "f64 (int64 fixed point)" if st["arithmetic"] == "fixed" else "f64",
             "data": "synthetic",
             "config": {
                 "workload": WORKLOADS["batch256"],

@@ -2347,10 +2347,12 @@ static int batch_call(lb_batch* b, cudaStream_t st, int with_grad, double* G_out
   const int mode = with_grad ? 1 : 0;
   const int order = batch_order(b, st);
   if (order) return order;
-  const bool fixed = batch_fixed(b);
+  bool fixed = batch_fixed(b);
+  const bool replay = b->exec[mode] && (fixed || !b->exec_fx[mode]);
+  if (replay) fixed = b->exec_fx[mode];
   // control tables, status, objective, gather; with the gradient two sums more
   const int launches = 5 + 2 * with_grad + (fixed ? (int)b->fx.size() : 1) * (1 + with_grad);
-  if (b->exec[mode] && (fixed || !b->exec_fx[mode])) {
+  if (replay) {
     LB_CUDA(cudaGraphLaunch(b->exec[mode], st), "cudaGraphLaunch");
   } else {
     // no graph, or one of the fixed-point sweeps for controls now out of their range
@@ -2386,6 +2388,7 @@ static int batch_call(lb_batch* b, cudaStream_t st, int with_grad, double* G_out
     tot.max_iterations = std::max(tot.max_iterations, one.max_iterations);
   }
   tot.kernel_launches = launches;
+  tot.arithmetic = fixed ? LB_ARITH_FIXED : LB_ARITH_F64;
   b->last = tot;
   if (G_out) std::memcpy(G_out, G.data(), sizeof(double) * n);
   if (grad_out && with_grad) std::memcpy(grad_out, g.data(), sizeof(double) * b->n_grad);

@@ -718,3 +718,25 @@ def test_fp64_sweeps_over_the_whole_cnot_horizon(L, K):
     Gf, gf = f.gradient()
     assert f.stats()["arithmetic"] == "f64"
     assert abs(G - Gf) <= 1e-10 * abs(Gf) and _rel(g, gf) < 1e-9
+
+
+@gpu
+def test_batch_statistics_name_the_arithmetic(L):
+    """Of the sweeps that ran: the graph's, or FP64 while the controls are out of
+    the fixed-point range, or while one member asks for FP64."""
+    from paper_2110_10310_gb300.system import LindbladBatch
+
+    ps = [W.random_problem(826 + k, levels=lv, n_states=2, n_steps=12, T_ns=0.12, amp=0.02, ckpt_every=0)
+          for k, lv in enumerate([(2,), (3, 2)])]
+    ss = [_sys(p, sweep=L.LB_SWEEP_RESIDENT) for p in ps]
+    b, st = LindbladBatch(ss), torch.cuda.Stream()
+    for capture in (False, True):
+        if capture:
+            b.capture(1, stream=st)
+        for scale, want in ((1.0, "fixed"), (40.0, "f64"), (1.0, "fixed")):
+            ss[1].set_alpha(scale * ps[1].controls.alpha)
+            b.gradient(stream=st)
+            assert b.stats()["arithmetic"] == want
+    m = LindbladBatch([ss[0], _sys(ps[1], sweep=L.LB_SWEEP_RESIDENT, arithmetic=L.LB_ARITH_F64)])
+    m.gradient()
+    assert m.stats()["arithmetic"] == "f64"
