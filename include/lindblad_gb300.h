@@ -452,8 +452,8 @@ int lb_propagate(lb_system* sys, void* stream, int32_t adjoint, int64_t j0, int6
  * n_vec device vectors (Appendix A, eq. mastereq_vectorized), with
  * M^{j+1/2} = M(t_j + dt/2); x and y must not overlap.  May run beside a
  * sweep or another lb_apply of this system on another stream.  Many elements at
- * once on a grid system (3 2^17 and more, n_vec <= M, controls in the fixed-point
- * range, not recorded) take the off-diagonal part in fixed point: its error is then
+ * once on a grid system (some 10^5 and more by the number of subsystems and their
+ * levels, n_vec <= M, controls in the fixed-point range, not recorded) take the off-diagonal part in fixed point: its error is then
  * relative to the vector's largest entry (2^-60 of it times the factors), where
  * FP64's follows each entry's own terms.  LB_ARITH_F64 keeps FP64. */
 int lb_apply(lb_system* sys, void* stream, int32_t adjoint, int64_t step, const void* x_dev, void* y_dev,

@@ -381,6 +381,15 @@ bool use_fixed_on(const lb_system* s, bool herm, bool spread) {
   return fixed_cfg(s, herm).E > 0 && rho_bound(s) <= lbk::kFixedRho;
 }
 bool use_fixed(const lb_system* s, bool herm) { return use_fixed_on(s, herm, s->rho_spread && s->tar_spread); }
+// lb_apply in fixed point pays for its three launches more (21 us) and its
+// decay tables, set up in every block (9.5 ns a factor), with some 28 Q - 8 ns less
+// per 1000 elements of Q subsystems; with a tenth to spare.  Fixed point and FP64,
+// us: 3 and 4 vectors of 4^4 levels 38.9, 39.0 and 39.0, 45.1; 17 and 21 of 5^3
+// 39.3, 36.9 and 44.1, 47.1; 51 of 2 x 2 x 20 45.3, 47.2; 10 and 16 of 2 x 2 x 56
+// 81.9, 65.6 and 95.5, 102.5; 64 and 128 of 2 x 64 108.9, 96.4 and 150.9, 188.6.
+bool apply_fixed_pays(const lb_system* s, double elements) {
+  return elements * (28.0 * s->Q - 8.0) >= 23e6 + 10500.0 * n_jcoef(s);
+}
 bool is_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
@@ -2067,7 +2076,7 @@ int lb_apply(lb_system* s, void* stream, int32_t adjoint, int64_t step, const vo
   // many elements: the off-diagonal part in fixed point, the vectors split into
   // a buffer of M states (every control factor within its range); a recorded
   // call may be replayed beside another one, which would share that buffer
-  if (use_grid(s) && s->fx_ws && n_vec <= s->M && (long long)n_vec * s->V >= lbk::kApplyFixedElements &&
+  if (use_grid(s) && s->fx_ws && n_vec <= s->M && apply_fixed_pays(s, (double)n_vec * s->V) &&
       rho_bound(s) <= lbk::kFixedRho && !is_capturing(st)) {
     rc = order_after_products(s, st);
     if (rc) return rc;

@@ -100,7 +100,8 @@ __device__ GxSmem gx_setup(unsigned char* base, const ProbDev& P, int nstates, i
     const Fx d = fx_coef(__double2ll_rn(scalbn(P.cd[i], 64 - P.kc[q])));
     S.cc[i] = make_int4(u.h, u.l, d.h, d.l);
   }
-  for (int i = threadIdx.x; i < P.njcoef; i += blockDim.x) {
+  // (the product alone scales its own decay factors)
+  for (int i = threadIdx.x; M && i < P.njcoef; i += blockDim.x) {
     S.jf[i] = fx_coef(__double2ll_rn(scalbn(P.jf[i], 64)));
     S.ja[i] = fx_coef(__double2ll_rn(scalbn(P.ja[i], 64)));
   }
@@ -1139,29 +1140,30 @@ __global__ void __launch_bounds__(kGridThreads, kApplyBlocks)
                double2* __restrict__ y, int n_vec) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_ka;
+  __shared__ unsigned long long s_d[kGxWarps];
   const ProbDev& P = *pp;
   const GxSmem S = gx_setup(smem, P, n_vec, 0, 0);
   const Hdr& H = S.g->h;
   const int V = H.V, N = H.N;
   const double2* ct = P.ctab + (size_t)step * H.cq;
-  if (threadIdx.x < 32) {
-    // the largest power of two that keeps every factor below 0.45, and those
-    // that one sum of gx_apply takes (both control factors and a decay factor)
-    // below 0.75 together: its middle part adds each factor's high half times a
-    // low half of 2^31 and each one's low half times a high half of 2^28.  (A
-    // warp's maxima: one thread took 35 us over the 408 decay factors of 2 x 2 x 20 levels.)
-    double m = 0.0, c = 0.0, d = 0.0;
-    for (int q = threadIdx.x; q < gp.Q; q += 32) {
+  // the largest power of two that keeps every factor below 0.45, and those
+  // that one sum of gx_apply takes (both control factors and a decay factor)
+  // below 0.75 together: its middle part adds each factor's high half times a
+  // low half of 2^31 and each one's low half times a high half of 2^28
+  double d = 0.0;
+  for (int i = threadIdx.x; i < P.njcoef; i += blockDim.x) d = fmax(d, fmax(P.jf[i], P.ja[i]));
+  const unsigned long long dm = warp_max_u64(abs_bits(d));
+  if ((threadIdx.x & 31) == 0) s_d[threadIdx.x >> 5] = dm;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double m = 0.0, c = 0.0;
+    for (int q = 0; q < gp.Q; ++q) {
       m = fmax(m, scalbn(fmax(fabs(ct[q].x), fabs(ct[q].y)), P.kc[q]));
       c = fmax(c, scalbn(fabs(ct[q].x) + fabs(ct[q].y), P.kc[q]));
     }
-    for (int i = threadIdx.x; i < P.njcoef; i += 32) d = fmax(d, fmax(P.jf[i], P.ja[i]));
-    auto top = [](double x) { return __longlong_as_double((long long)warp_max_u64(abs_bits(x))); };
-    m = top(m);
-    c = top(c);
-    d = top(d);
+    for (int w = 0; w < kGxWarps; ++w) d = fmax(d, __longlong_as_double((long long)s_d[w]));
     m = fmax(fmax(m, d), 0.6 * (c + d));
-    if (threadIdx.x == 0) s_ka = m > 0.0 ? min(20, ilogb(0.45 / m)) : 20;
+    s_ka = m > 0.0 ? min(20, ilogb(0.45 / m)) : 20;
   }
   __syncthreads();
   const int ka = s_ka;

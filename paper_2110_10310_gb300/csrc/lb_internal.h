@@ -261,10 +261,6 @@ cudaError_t launch_backward_gx(const ProbDev* d_prob, const ProbDev& h_prob, cud
 // P.apm[i] of n_vec <= M vectors: below 0x7ff00000 when vector i is within kGridCrest
 cudaError_t launch_crest(const ProbDev& h_prob, const double2* x, int n_vec, cudaStream_t s);
 // y = M x with the off-diagonal part in fixed point (n_vec <= M)
-// Fewest elements of a call that take it: it has two launches more, k_apply half
-// the rate.  Six vectors of vec 65536 (this many) 55 us against 70 in FP64, four 47
-// against 45, two 41 against 29; 25 of vec 15625 53 against 55, 17 47 against 37.
-constexpr long long kApplyFixedElements = 3 << 17;
 cudaError_t launch_apply_gx(const ProbDev* d_prob, const ProbDev& h_prob, int adjoint, int64_t step, const double2* x,
                             double2* y, int n_vec, cudaStream_t s);
 

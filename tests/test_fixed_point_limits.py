@@ -489,13 +489,13 @@ def test_products_where_control_and_decay_factors_are_alike(L):
         assert bool(((y - ref).abs().amax(dim=(1, 2)) <= 2.0**-50 * _term_bound(p, x, 1)).all())
 
 
-# edges of the product's dispatch: 3 2^17 elements and just below, the unrolled
+# edges of the product's dispatch: the fewest vectors it takes and one less, the unrolled
 # loops (4 and 6 subsystems) and the general one, odd N, tables above 48 KB of
 # shared memory, fewer vectors than states
 @gpu
 @pytest.mark.parametrize("levels,M,n", [
-    ((4, 4, 4, 4), 6, 6), ((4, 4, 4, 4), 6, 5), ((3, 3, 3, 3, 3), 7, 7), ((3,) * 6, 1, 1), ((5, 5, 5), 26, 26),
-    ((5, 5, 5), 26, 25), ((7, 3, 7), 20, 19), ((2, 2, 56), 8, 8), ((2, 64), 24, 24)])
+    ((4, 4, 4, 4), 4, 4), ((4, 4, 4, 4), 4, 3), ((3, 3, 3, 3, 3), 4, 4), ((3,) * 6, 1, 1), ((5, 5, 5), 21, 21),
+    ((5, 5, 5), 21, 20), ((7, 3, 7), 20, 15), ((2, 2, 56), 15, 15), ((2, 64), 84, 84)])
 @pytest.mark.parametrize("decay", [True, False])
 def test_large_products_match_fp64(L, levels, M, n, decay):
     """FP64's and the integers' rounding of at most 2^-50 of the terms."""
