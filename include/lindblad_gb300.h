@@ -475,9 +475,9 @@ int lb_get_stats(lb_system* sys, lb_stats* out);
  * `stream`.  choice_out (nullable, [3]) receives the chosen LB_SWEEP_*,
  * LB_SOLVER_* and the threads per CTA (resident), CTAs per cluster (cluster)
  * or blocks (grid).  Within the fixed-point sweeps' range the Jacobi iteration
- * is one candidate, and a system of the cluster sweep then keeps that sweep
- * (its chunks) or one CTA per state, whichever runs lb_forward faster;
- * choice_out[2] is then the number of chunks or the threads per CTA.
+ * in chunks (the cluster sweep's systems) and with one CTA per state are compared
+ * with the fastest other candidate by an lb_forward each; choice_out[2] is then
+ * the number of chunks or the threads per CTA.
  * LB_ENOTCONV when no candidate converges. */
 int lb_autotune(lb_system* sys, void* stream, int32_t probe_steps, int32_t* choice_out);
 

@@ -1129,16 +1129,13 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
   const bool grid0 = use_grid(s);
   const int methods[3] = {LB_SOLVER_JACOBI, LB_SOLVER_NEUMANN, LB_SOLVER_GMRES};
   // in fixed point steps on vectors run one kernel, whatever shape the FP64
-  // sweeps would take
+  // sweeps would take, and short of the chunks' gain
   const int bound_method = s->method;
   s->method = LB_SOLVER_JACOBI;
   const bool fixed = !grid0 && use_fixed(s, false, st);
   s->method = bound_method;
   for (int m : methods) {
-    if (fixed && m == LB_SOLVER_JACOBI) {
-      cands.push_back({LB_SWEEP_RESIDENT, m, s->rc.E});
-      continue;
-    }
+    if (fixed && m == LB_SOLVER_JACOBI) continue;  // timed below
     if (grid0) {
       if (m != LB_SOLVER_GMRES) cands.push_back({LB_SWEEP_GRID, m, 0});
       continue;
@@ -1164,18 +1161,23 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
   Cand win{-1, m0, 0};
   double2* probe = at<double2>(s, s->L.qT);
   const size_t bytes = sizeof(double2) * (size_t)s->M * s->V;
-  for (const Cand& c : cands) {
-    s->method = c.method;
-    s->hp.method = c.method;
-    if (c.sweep == LB_SWEEP_CLUSTER) s->cc = cluster_cfg(s, c.E != 0);
+  // the handle as candidate c runs (the caller uploads s->hp); in fixed point in the shapes it was bound with
+  auto take = [&](const Cand& c) {
+    const bool fx = fixed && c.method == LB_SOLVER_JACOBI;
+    s->method = s->hp.method = c.method;
+    s->rc = rc0;
+    s->cc = cc0;
+    if (c.sweep == LB_SWEEP_CLUSTER && !fx) s->cc = cluster_cfg(s, c.E != 0);
     choose_cluster(s, c.sweep == LB_SWEEP_CLUSTER);
-    if (c.sweep == LB_SWEEP_RESIDENT) {
+    if (c.sweep == LB_SWEEP_RESIDENT && !fx) {
       s->rc = lbk::resident_config(s->V, s->Q, n_coef(s), n_jcoef(s), s->N, s->jp.empty(), kry_elems(s));
-      const int threads = ((s->V + c.E - 1) / c.E + 31) / 32 * 32;
       s->rc.E = c.E;
-      s->rc.threads = threads;
+      s->rc.threads = ((s->V + c.E - 1) / c.E + 31) / 32 * 32;
       s->rc.QT = (c.E == 1 && s->Q <= 4 && s->jp.empty()) ? s->Q : 0;
     }
+  };
+  for (const Cand& c : cands) {
+    take(c);
     LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
     LB_CUDA(cudaMemcpyAsync(probe, at<double2>(s, s->L.q0), bytes, cudaMemcpyDeviceToDevice, st), "probe states");
     // one untimed run (module loading, first-launch costs), one timed
@@ -1200,27 +1202,30 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
       win = c;
     }
   }
-  const bool fixed_won = fixed && win.method == LB_SOLVER_JACOBI;
-  if (fixed_won) {
-    // the sweeps of the whole horizon: in chunks (the cluster sweep's systems)
-    // against one CTA per state, by a forward call each; a tie, or neither: as bound
-    s->rc = rc0;
-    s->cc = cc0;
-    s->method = s->hp.method = win.method;
-    win.sweep = cl0 ? LB_SWEEP_CLUSTER : LB_SWEEP_RESIDENT;
-    float ms[2] = {-1.0f, -1.0f};
-    for (int cl = 0; cl < 2 && cc0.C > 0; ++cl) {
-      choose_cluster(s, cl != 0);
+  if (fixed) {
+    // the Jacobi iteration in chunks (the cluster sweep's systems) and with one CTA
+    // per state against the fastest other candidate, by a forward call each
+    std::vector<Cand> last;
+    if (cc0.C > 0) last.push_back({LB_SWEEP_CLUSTER, LB_SOLVER_JACOBI, 0});
+    last.push_back({LB_SWEEP_RESIDENT, LB_SOLVER_JACOBI, 0});
+    if (win.sweep >= 0) last.push_back(win);
+    best = -1.0f;
+    win.sweep = -1;
+    for (const Cand& c : last) {
+      take(c);
       LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
-      rc = time_forward(s, st, e0, e1, &ms[cl]);
+      float ms = -1.0f;
+      rc = time_forward(s, st, e0, e1, &ms);
       if (rc) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         return rc;
       }
+      if (ms >= 0.0f && (best < 0.0f || ms < best)) {
+        best = ms;
+        win = c;
+      }
     }
-    if (ms[1] >= 0.0f && (ms[0] < 0.0f || ms[1] < ms[0])) win.sweep = LB_SWEEP_CLUSTER;
-    else if (ms[0] >= 0.0f && (ms[1] < 0.0f || ms[0] < ms[1])) win.sweep = LB_SWEEP_RESIDENT;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1232,15 +1237,7 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
     LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
     return fail(LB_ENOTCONV, "no candidate's inner solve converged on the probe steps");
   }
-  s->method = s->hp.method = win.method;
-  s->cc = win.sweep == LB_SWEEP_CLUSTER && !fixed_won ? cluster_cfg(s, win.E != 0) : cc0;
-  choose_cluster(s, win.sweep == LB_SWEEP_CLUSTER);
-  if (win.sweep == LB_SWEEP_RESIDENT && !fixed_won) {
-    s->rc = lbk::resident_config(s->V, s->Q, n_coef(s), n_jcoef(s), s->N, s->jp.empty(), kry_elems(s));
-    s->rc.E = win.E;
-    s->rc.threads = ((s->V + win.E - 1) / win.E + 31) / 32 * 32;
-    s->rc.QT = (win.E == 1 && s->Q <= 4 && s->jp.empty()) ? s->Q : 0;
-  }
+  take(win);
   LB_CUDA(cudaMemcpyAsync(s->dp, &s->hp, sizeof(ProbDev), cudaMemcpyHostToDevice, st), "upload problem");
   LB_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
   if (use_grid(s) && s->hp.pred_restart >= 0) {
@@ -1290,7 +1287,7 @@ int lb_autotune(lb_system* s, void* stream, int32_t probe_steps, int32_t* choice
     choice_out[0] = win.sweep;
     choice_out[1] = win.method;
     choice_out[2] = win.sweep == LB_SWEEP_RESIDENT ? s->rc.threads : (s->cluster ? s->cc.C : s->gblocks);
-    if (fixed_won)
+    if (fixed && win.method == LB_SOLVER_JACOBI)
       choice_out[2] = use_chunks(s) ? s->hp.chunkC : fixed_cfg(s, s->hp.herm != 0).threads;
   }
   return LB_OK;
